@@ -57,7 +57,7 @@ struct InstDev {
   unsigned long long *topk;  // [2][NP * 3] partial leader keys (by generation parity)
   unsigned *ctr;         // [4] CTA-completion counters
   int32_t *gen;          // [1] completed generations
-  int32_t *best;         // [1] best index (get_best)
+  double2 *rpart;        // [3 ceil(N / 128)] FP64 partials of the best design (get_best)
   float *trace;          // optional fitness trace
   float *Fsched;         // [G + 1] F of every generation, or NULL for constant F; the
                          // adaptive F (f_schedule 2) writes entry g + 1 during generation g
@@ -335,9 +335,10 @@ __device__ __forceinline__ float4 ld_cur(const InstDev &I, int i, int slot, uint
 }
 
 // ---------------------------------------------------- Step 1: initialisation
-template <bool COMP, int MK = 0>
+// WT: the team is one warp (t = lane, warp reduction) instead of the whole CTA
+template <bool COMP, int MK = 0, bool WT = false>
 __device__ void init_individual(const InstDev &I, int i, Mono *sh) {
-  const int t = threadIdx.x;
+  const int t = WT ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
   const PhiloxKey K = philox_schedule(I.key);
   float *row = row_ptr(I, i, 0);
   Acc<COMP> acc;
@@ -363,9 +364,9 @@ __device__ void init_individual(const InstDev &I, int i, Mono *sh) {
   float2 D = make_float2(0.f, 0.f);
   float f = 0.f;
   if constexpr (MK != 0) {
-    multi_finish<MK, false>(I, macc, sh, f, D);
+    multi_finish<MK, WT>(I, macc, sh, f, D);
   } else {
-    const Mono m = block_reduce(acc.get(), sh);
+    const Mono m = WT ? warp_reduce(acc.get()) : block_reduce(acc.get(), sh);
     if (t == 0) {
       D = field_of(I, m);
       f = fit_of(D);
@@ -390,6 +391,26 @@ static __global__ void k_init(InstDev I) {
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *I.gen = 0;
     for (int k = 0; k < 4; ++k) I.ctr[k] = 0u;
+  }
+}
+
+// All instances of a state in one launch (blockIdx.y the instance, largest first; one-warp
+// teams, 8 per CTA).  One launch per instance kept 64 to 512 one-warp CTAs on the GPU, each
+// bound by the latency of its own chain: 27-52 us an instance, 26 ms for 512 of them.
+constexpr int INIT_WARPS = 8;
+static __global__ void __launch_bounds__(INIT_WARPS * 32)
+    k_init_many(const InstDev *__restrict__ insts, const int32_t *__restrict__ order, int n) {
+  const int w0 = blockIdx.x * INIT_WARPS + (threadIdx.x >> 5), stride = gridDim.x * INIT_WARPS;
+  for (int k = blockIdx.y; k < n; k += gridDim.y) {
+    const InstDev I = insts[order[k]];
+    for (int i = w0; i < I.NP; i += stride) {
+      if (I.compensated) init_individual<true, 0, true>(I, i, nullptr);
+      else init_individual<false, 0, true>(I, i, nullptr);
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      *I.gen = 0;
+      for (int c = 0; c < 4; ++c) I.ctr[c] = 0u;
+    }
   }
 }
 
@@ -1581,36 +1602,9 @@ static __global__ void __launch_bounds__(BATCH_WARPS * 32, 1)
 }
 
 // ------------------------------------------------ outputs: best, FP64, layout
-static __global__ void k_best(InstDev I, int32_t *index_out) {
-  __shared__ unsigned long long shk[3 * 32];
-  unsigned long long k0 = 0, k1 = 0, k2 = 0;
-  for (int i = threadIdx.x; i < I.NP; i += blockDim.x)
-    top3_insert(k0, k1, k2, sel_key(I.minimize != 0, I.fit[i], i));
-  block_top3(k0, k1, k2, shk);
-  if (threadIdx.x == 0) {
-    *I.best = key_index(k0);
-    if (index_out) *index_out = key_index(k0);
-  }
-}
-
 __device__ __forceinline__ size_t perm_pos(const InstDev &I, int j) {
   const int t = j / I.c, e = j - t * I.c;
   return ((size_t)(e >> 2) * I.T + t) * 4 + (e & 3);
-}
-
-static __global__ void k_unpermute(InstDev I, int i_fixed, float *out, int64_t ld) {
-  const int i = i_fixed >= 0 ? i_fixed : (i_fixed == -2 ? *I.best : (int)blockIdx.x);
-  const int32_t *sel = (*I.gen & 1) ? I.sel1 : I.sel0;
-  const float *row = row_ptr(I, i, sel[i]);
-  float *o = out + (i_fixed == -1 ? (int64_t)i * ld : 0);
-  for (int j = threadIdx.x; j < I.N; j += blockDim.x) o[j] = row[perm_pos(I, j)];
-}
-
-static __global__ void k_copy_fit(InstDev I, float *fit_out, float2 *d_out) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= I.NP) return;
-  if (fit_out) fit_out[i] = I.fit[i];
-  if (d_out) d_out[i] = I.dval[i];
 }
 
 struct Mono64 {
@@ -1624,51 +1618,198 @@ __device__ __forceinline__ Mono64 m64_combine(const Mono64 &L, const Mono64 &R) 
                      L.C.y + R.C.y + (R.A.x * L.B.y + R.A.y * L.B.x));
   return o;
 }
+__device__ __forceinline__ double2 shfl_down2(double2 v, int s) {
+  return make_double2(__shfl_down_sync(0xffffffffu, v.x, s), __shfl_down_sync(0xffffffffu, v.y, s));
+}
+// ordered reduction over the 32 lanes of a warp, valid in lane 0
+__device__ __forceinline__ Mono64 m64_warp_reduce(Mono64 m) {
+#pragma unroll
+  for (int s = 1; s < 32; s <<= 1) {
+    Mono64 r;
+    r.A = shfl_down2(m.A, s);
+    r.B = shfl_down2(m.B, s);
+    r.C = shfl_down2(m.C, s);
+    m = m64_combine(m, r);  // lanes that are no multiple of 2s hold values nobody reads
+  }
+  return m;
+}
+__device__ __forceinline__ double2 cmul64(const double2 &a, const double2 &b) {
+  return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+}
 
-// A11: FP64 re-evaluation of the best individual's d_eff (closed form, FP64 phasors)
-static __global__ void k_recheck64(InstDev I, double *d64_out, float *fit_out) {
-  __shared__ Mono64 sh[256];
-  const int i = *I.best;
+// e^{-i kappa q}, q = 1, 2, 3, of both mismatches (host)
+struct BestRot {
+  double2 r1[3], r2[3];
+};
+
+// The best individual (A11): its index, fitness and genes, and the partial sums of its FP64
+// re-evaluation (closed form, FP64 phasors).  Bound by the FP64 unit, which retires about two
+// lanes a cycle and SM on this GPU: one CTA doing all of it with two sincos a domain took
+// 109 us at N = 1000 and 2.08 ms at N = 1e5.  So the domains are spread over the whole GPU, a
+// warp per 128 domains in a CTA of its own, every CTA finding the best individual itself (a
+// few KB of fitness from L2, no grid-wide wait), and a lane takes 4 neighbouring domains with
+// one sincos per mismatch, the other three phasors by rotation.
+constexpr int BEST_THREADS = 128, BEST_DOMAINS = 128;
+static __global__ void __launch_bounds__(BEST_THREADS)
+    k_best(InstDev I, BestRot rot, float *genes_out, float *fit_out, int32_t *index_out, int scan) {
+  __shared__ unsigned long long shk[BEST_THREADS / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  unsigned long long key = 0;
+#pragma unroll 8
+  for (int i = threadIdx.x; i < I.NP; i += BEST_THREADS) {
+    const unsigned long long k = sel_key(I.minimize != 0, I.fit[i], i);
+    key = k > key ? k : key;
+  }
+  const uint32_t hi = (uint32_t)(key >> 32), mhi = __reduce_max_sync(0xffffffffu, hi);
+  const uint32_t mlo = __reduce_max_sync(0xffffffffu, hi == mhi ? (uint32_t)key : 0u);
+  if (lane == 0) shk[warp] = ((unsigned long long)mhi << 32) | mlo;
+  __syncthreads();
+  key = shk[0];
+#pragma unroll
+  for (int w = 1; w < BEST_THREADS / 32; ++w) key = shk[w] > key ? shk[w] : key;
+  const int i = key_index(key);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    if (index_out) *index_out = i;
+    if (fit_out) *fit_out = I.fit[i];
+  }
   const int32_t *sel = (*I.gen & 1) ? I.sel1 : I.sel0;
   const float *row = row_ptr(I, i, sel[i]);
-  const int nt = blockDim.x, t = threadIdx.x;
-  const int per = (I.N + nt - 1) / nt;
-  const int j0 = min(I.N, t * per), j1 = min(I.N, j0 + per);
+  const int b0 = blockIdx.x * BEST_DOMAINS;
+  if (genes_out && b0 + (int)threadIdx.x < I.N)
+    genes_out[b0 + threadIdx.x] = row[perm_pos(I, b0 + threadIdx.x)];
+  if (!scan || warp != 0) return;
   Mono64 m;
   m.A = m.B = m.C = make_double2(0.0, 0.0);
-  for (int j = j0; j < j1; ++j) {
-    const double d = row[perm_pos(I, j)] < 0.f ? -1.0 : 1.0;
-    double s1, c1, s2, c2;
-    sincos(reduce_2pi((double)j * I.kappa1), &s1, &c1);
-    sincos(reduce_2pi((double)j * I.kappa2), &s2, &c2);
-    const double ar = d * c2, ai = -d * s2;  // a = d p2
-    m.C.x += ar * m.B.x - ai * m.B.y;
-    m.C.y += ar * m.B.y + ai * m.B.x;
-    m.A.x += ar;
-    m.A.y += ai;
-    m.B.x += d * c1;  // b = d p1
-    m.B.y -= d * s1;
+  const int m0 = b0 + 4 * lane;
+  if (m0 < I.N) {
+    const float4 x = *(const float4 *)(row + perm_pos(I, m0));  // a group of 4 is contiguous
+    const float xs[4] = {x.x, x.y, x.z, x.w};
+    double sn, cs;
+    sincos(reduce_2pi((double)m0 * I.kappa1), &sn, &cs);
+    const double2 p1 = make_double2(cs, -sn);
+    sincos(reduce_2pi((double)m0 * I.kappa2), &sn, &cs);
+    const double2 p2 = make_double2(cs, -sn);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (m0 + q < I.N) {
+        const double d = xs[q] < 0.f ? -1.0 : 1.0;
+        const double2 c1 = q ? cmul64(p1, rot.r1[q ? q - 1 : 0]) : p1;
+        const double2 c2 = q ? cmul64(p2, rot.r2[q ? q - 1 : 0]) : p2;
+        const double2 a = make_double2(d * c2.x, d * c2.y);
+        m.C.x += a.x * m.B.x - a.y * m.B.y;
+        m.C.y += a.x * m.B.y + a.y * m.B.x;
+        m.A.x += a.x;
+        m.A.y += a.y;
+        m.B.x += d * c1.x;
+        m.B.y += d * c1.y;
+      }
+    }
   }
-  sh[t] = m;
+  m = m64_warp_reduce(m);
+  if (lane == 0) {
+    I.rpart[3 * blockIdx.x] = m.A;
+    I.rpart[3 * blockIdx.x + 1] = m.B;
+    I.rpart[3 * blockIdx.x + 2] = m.C;
+  }
+}
+
+// the partials in index order, and the field: one CTA, a programmatic dependent of k_best
+static __global__ void __launch_bounds__(BEST_THREADS)
+    k_best_close(InstDev I, int nparts, double *d64_out) {
+  __shared__ Mono64 sh[BEST_THREADS / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int per = (nparts + BEST_THREADS - 1) / BEST_THREADS;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  Mono64 m;
+  m.A = m.B = m.C = make_double2(0.0, 0.0);
+  if (warp * 32 * per < nparts) {  // the warp has partials
+    const int s0 = min(nparts, (int)threadIdx.x * per), s1 = min(nparts, s0 + per);
+    for (int s = s0; s < s1; ++s) {
+      Mono64 r;
+      r.A = I.rpart[3 * s];
+      r.B = I.rpart[3 * s + 1];
+      r.C = I.rpart[3 * s + 2];
+      m = m64_combine(m, r);
+    }
+    m = m64_warp_reduce(m);
+  }
+  if (lane == 0) sh[warp] = m;
   __syncthreads();
-  if (t == 0) {
-    Mono64 acc = sh[0];
-    for (int k = 1; k < nt; ++k) acc = m64_combine(acc, sh[k]);
-    double re, im;
-    if (I.obj == OBJ_SHG || I.obj == OBJ_MULTI_SHG) {  // SHG field: phi(kappa1) sum d p1
-      const double2 ph = I.konst64[3];
-      re = ph.x * acc.B.x - ph.y * acc.B.y;
-      im = ph.x * acc.B.y + ph.y * acc.B.x;
-    } else {  // cascaded d_eff
-      const double2 p12 = I.konst64[0], cd = I.konst64[1];
-      re = p12.x * acc.C.x - p12.y * acc.C.y + cd.x;
-      im = p12.x * acc.C.y + p12.y * acc.C.x + cd.y;
+  if (threadIdx.x != 0) return;
+  for (int w = 1; w < BEST_THREADS / 32 && w * 32 * per < nparts; ++w) m = m64_combine(m, sh[w]);
+  double re, im;
+  if (I.obj == OBJ_SHG || I.obj == OBJ_MULTI_SHG) {  // SHG field: phi(kappa1) sum d p1
+    const double2 ph = I.konst64[3];
+    re = ph.x * m.B.x - ph.y * m.B.y;
+    im = ph.x * m.B.y + ph.y * m.B.x;
+  } else {  // cascaded d_eff
+    const double2 p12 = I.konst64[0], cd = I.konst64[1];
+    re = p12.x * m.C.x - p12.y * m.C.y + cd.x;
+    im = p12.x * m.C.y + p12.y * m.C.x + cd.y;
+  }
+  d64_out[0] = re;
+  d64_out[1] = im;
+}
+
+// Rows back to natural order.  A row is a [c / 4][T] matrix of float4 groups and its natural
+// order the transposed one, so a warp takes a tile of 32 threads' groups x 8, reads it by 512 B
+// along T, and writes runs of up to 128 B along c / 4 through shared memory (16 bytes a lane
+// where the output rows allow it).  A gene at a time, with a division and reads 16 bytes apart,
+// ran at 2.7-4.3 TB/s of read + write (66 MB of N = 3300 rows in 50 us).  The fitness and
+// field outputs are copied by the same launch.
+constexpr int POP_THREADS = 256, POP_KB = 8;
+static __global__ void __launch_bounds__(POP_THREADS)
+    k_population(InstDev I, float *__restrict__ out, int64_t ld, float *__restrict__ fit_out,
+                 float2 *__restrict__ d_out) {
+  __shared__ float4 tile[POP_THREADS / 32][POP_KB * 33];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (int i = blockIdx.x * POP_THREADS + threadIdx.x; i < I.NP; i += gridDim.x * POP_THREADS) {
+    if (fit_out) fit_out[i] = I.fit[i];
+    if (d_out) d_out[i] = I.dval[i];
+  }
+  if (!out) return;
+  const int32_t *sel = (*I.gen & 1) ? I.sel1 : I.sel0;
+  const int n4 = I.c >> 2, nk = (n4 + POP_KB - 1) / POP_KB;
+  const uint32_t tiles = (uint32_t)(I.T >> 5) * nk, total = tiles * (uint32_t)I.NP;
+  const bool vec = (((uintptr_t)out & 15) == 0) && (ld & 3) == 0;
+  float4 *S = tile[warp];
+  for (uint32_t w = blockIdx.x * (POP_THREADS / 32) + warp; w < total;
+       w += gridDim.x * (POP_THREADS / 32)) {
+    const int i = (int)(w / tiles), r = (int)(w - (uint32_t)i * tiles);
+    const int t0 = r / nk * 32, k0 = r % nk * POP_KB, kb = min(POP_KB, n4 - k0);
+    const float4 *row = (const float4 *)row_ptr(I, i, sel[i]) + (size_t)k0 * I.T + t0 + lane;
+    float4 v[POP_KB];
+#pragma unroll
+    for (int k = 0; k < POP_KB; ++k)
+      if (k < kb) v[k] = row[(size_t)k * I.T];
+    __syncwarp();  // the previous tile has been read
+#pragma unroll
+    for (int k = 0; k < POP_KB; ++k)
+      if (k < kb) S[k * 33 + lane] = v[k];
+    __syncwarp();
+    float *o = out + (int64_t)i * ld;
+    const int sft = kb > 4 ? 3 : (kb > 2 ? 2 : kb - 1);  // 2^sft >= kb groups of a run
+    if (vec) {
+      for (int it = 0; it < (1 << sft); ++it) {
+        const int e = it * 32 + lane, tt = e >> sft, k = e & ((1 << sft) - 1);
+        const int j = (t0 + tt) * I.c + 4 * (k0 + k);
+        if (k >= kb || j >= I.N) continue;
+        const float4 x = S[k * 33 + tt];
+        if (j + 4 <= I.N) {
+          *(float4 *)(o + j) = x;
+        } else {
+          o[j] = x.x;
+          if (j + 1 < I.N) o[j + 1] = x.y;
+          if (j + 2 < I.N) o[j + 2] = x.z;
+        }
+      }
+    } else {
+      for (int it = 0; it < (4 << sft); ++it) {
+        const int e = it * 32 + lane, tt = e >> (sft + 2), q = e & ((4 << sft) - 1);
+        const int j = (t0 + tt) * I.c + 4 * k0 + q;
+        if (q < 4 * kb && j < I.N) o[j] = ((const float *)S)[((q >> 2) * 33 + tt) * 4 + (q & 3)];
+      }
     }
-    if (d64_out) {
-      d64_out[0] = re;
-      d64_out[1] = im;
-    }
-    if (fit_out) fit_out[0] = I.fit[i];
   }
 }
 
@@ -1691,17 +1832,12 @@ static __global__ void k_polish_pick(InstDev I, int32_t *lead_out) {
   }
 }
 
-__device__ __forceinline__ size_t perm_pos_of(const InstDev &I, int j) {
-  const int t = j / I.c, e = j - t * I.c;
-  return ((size_t)(e >> 2) * I.T + t) * 4 + (e & 3);
-}
-
 static __global__ void k_polish_theta(InstDev I, const int32_t *lead, float tau, float *theta) {
   const int k = blockIdx.x, i = lead[k];
   const int32_t *sel = (*I.gen & 1) ? I.sel1 : I.sel0;
   const float *row = row_ptr(I, i, sel[i]);
   for (int j = threadIdx.x; j < I.N; j += blockDim.x)
-    theta[(size_t)k * I.Npad + j] = __fmul_rn(tau, row[perm_pos_of(I, j)]);
+    theta[(size_t)k * I.Npad + j] = __fmul_rn(tau, row[perm_pos(I, j)]);
 }
 
 static __global__ void k_polish_step(int N, int64_t ld, float lr, float *theta, const float *grad) {
@@ -1841,6 +1977,8 @@ struct qpm_state {
   unsigned *bar = nullptr;  // [0] count, [1] unused, [2] err, [3] batch queue
   unsigned long long timeout_ns = 5000000000ull;
   InstDev *d_insts = nullptr;  // device copy of the descriptors (batched form)
+  qpm::TableJob *d_jobs = nullptr;  // the instances' tables (qpm_init of many instances)
+  int max_npad = 0, max_np = 0;
   int32_t *d_order = nullptr;  // instances by decreasing work
   size_t batch_smem = 0;       // dynamic shared memory of the batched kernel
   bool batch_ts = false;       // phasor tables in shared memory (else read from global)
@@ -2050,6 +2188,12 @@ static qpm_status enqueue_step(qpm_state *st, cudaStream_t s) {
   return QPM_OK;
 }
 
+static int best_parts(int N) { return (N + BEST_DOMAINS - 1) / BEST_DOMAINS; }
+
+static TableJob table_job(const InstDev &I) {
+  return TableJob{{I.N, I.Npad, I.T, I.c, I.kappa1, I.kappa2}, I.table, I.tpart, I.konst, I.konst64};
+}
+
 static qpm_status check_state(qpm_state *st, int gens) {
   if (!st) return fail(QPM_ERR_ARG, "NULL state");
   if (!st->inited) return fail(QPM_ERR_STATE, "qpm_init has not been called");
@@ -2169,10 +2313,13 @@ extern "C" qpm_status qpm_create(const qpm_problem *probs, const qpm_params *par
     total += align_up(NP * sizeof(unsigned long long), 256);  // DE survivor keys
     total += 2 * align_up((size_t)(q.G + 1) * sizeof(float), 256);  // F history, F base
     total += align_up((size_t)q.G * 7 * sizeof(uint32_t), 256);     // discrete GWO thresholds
-    total += 256 + 256 + 256;  // ctr, gen, best
+    total += 256 + 256;  // ctr, gen
+    total += align_up(3 * (size_t)best_parts(p.N) * sizeof(double2), 256);
   }
   const size_t desc_off = total;
   total += align_up(sizeof(InstDev) * (size_t)n_inst, 256);
+  const size_t jobs_off = total;
+  total += align_up(sizeof(TableJob) * (size_t)n_inst, 256);
   const size_t order_off = total;
   total += align_up(sizeof(int32_t) * (size_t)n_inst, 256);
   total += 256;  // barrier words
@@ -2213,11 +2360,12 @@ extern "C" qpm_status qpm_create(const qpm_problem *probs, const qpm_params *par
     }
     I.ctr = (unsigned *)take(4 * sizeof(unsigned));
     I.gen = (int32_t *)take(sizeof(int32_t));
-    I.best = (int32_t *)take(sizeof(int32_t));
+    I.rpart = (double2 *)take(3 * (size_t)best_parts(I.N) * sizeof(double2));
   }
   st->bar = (unsigned *)((char *)st->arena + total - 256);
   st->d_insts = (InstDev *)((char *)st->arena + desc_off);
   st->d_order = (int32_t *)((char *)st->arena + order_off);
+  st->d_jobs = (TableJob *)((char *)st->arena + jobs_off);
   {
     // largest instances first (longest-processing-time order for the batch queue)
     std::vector<int32_t> order(n_inst);
@@ -2272,9 +2420,17 @@ extern "C" qpm_status qpm_create(const qpm_problem *probs, const qpm_params *par
       e = cudaMemcpy(st->d_order, order.data(), sizeof(int32_t) * n_inst, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
       e = cudaMemcpy(st->d_insts, st->h.data(), sizeof(InstDev) * n_inst, cudaMemcpyHostToDevice);
+    std::vector<TableJob> jobs(n_inst);
+    for (int k = 0; k < n_inst; ++k) jobs[k] = table_job(st->h[k]);
+    if (e == cudaSuccess)
+      e = cudaMemcpy(st->d_jobs, jobs.data(), sizeof(TableJob) * n_inst, cudaMemcpyHostToDevice);
     if (e != cudaSuccess) { cudaFree(st->arena); delete st; return cuda_fail(e, "cudaMemcpy"); }
     int maxpad = 0;
-    for (int k = 0; k < n_inst; ++k) maxpad = std::max(maxpad, st->h[k].Npad);
+    for (int k = 0; k < n_inst; ++k) {
+      maxpad = std::max(maxpad, st->h[k].Npad);
+      st->max_np = std::max(st->max_np, st->h[k].NP);
+    }
+    st->max_npad = maxpad;
     st->batch_ts = (size_t)maxpad * sizeof(float4) <= BATCH_TS_MAX_BYTES;
     st->batch_smem = sizeof(float4) * stg_f4_per_thread(st->batch_ts) * BATCH_WARPS * 32 +
                      (st->batch_ts ? (size_t)maxpad * sizeof(float4) : 0);
@@ -2302,7 +2458,17 @@ extern "C" qpm_status qpm_set_trace(qpm_state *st, int32_t inst, float *trace) {
 extern "C" qpm_status qpm_init(qpm_state *st, qpm_stream_t stream) {
   if (!st) return fail(QPM_ERR_ARG, "NULL state");
   cudaStream_t s = (cudaStream_t)stream;
-  for (int k = 0; k < st->n; ++k) {
+  // many instances of one-warp teams and single kinds: three launches for all of them
+  bool many = st->n > 1;
+  for (int k = 0; many && k < st->n; ++k) many = st->h[k].T == 32 && st->h[k].obj < OBJ_MULTI_THG;
+  if (many) {
+    qpm_status r = launch_tables(st->d_jobs, st->n, st->max_npad, s);
+    if (r != QPM_OK) return r;
+    const dim3 grid(std::min(64, (st->max_np + INIT_WARPS - 1) / INIT_WARPS), std::min(st->n, 65535));
+    k_init_many<<<grid, INIT_WARPS * 32, 0, s>>>(st->d_insts, st->d_order, st->n);
+    QPM_CUDA(cudaGetLastError());
+  }
+  for (int k = 0; !many && k < st->n; ++k) {
     const InstDev &I = st->h[k];
     TableSpec ts{I.N, I.Npad, I.T, I.c, I.kappa1, I.kappa2};
     qpm_status r = launch_table(ts, I.table, I.tpart, I.konst, I.konst64, s);
@@ -2590,6 +2756,8 @@ extern "C" qpm_status qpm_set_objective(qpm_state *st, int32_t inst, const qpm_o
     st->graph_n = -1;
   }
   QPM_CUDA(cudaMemcpy(st->d_insts + inst, &I, sizeof(InstDev), cudaMemcpyHostToDevice));
+  const TableJob job = table_job(I);
+  QPM_CUDA(cudaMemcpy(st->d_jobs + inst, &job, sizeof(TableJob), cudaMemcpyHostToDevice));
   return QPM_OK;
 }
 
@@ -2669,9 +2837,13 @@ extern "C" qpm_status qpm_get_population(qpm_state *st, int32_t inst, float *gen
   const InstDev &I = st->h[inst];
   if (genes_out && ld < I.N) return fail(QPM_ERR_ARG, "ld < N");
   cudaStream_t s = (cudaStream_t)stream;
-  if (genes_out) k_unpermute<<<I.NP, 256, 0, s>>>(I, -1, genes_out, ld);
-  if (fit_out || d_eff_out)
-    k_copy_fit<<<(I.NP + 255) / 256, 256, 0, s>>>(I, fit_out, (float2 *)d_eff_out);
+  // a warp per tile of 32 x 8 groups, at most 8 CTAs per SM; no genes: a thread per individual
+  const int64_t warps = (int64_t)I.NP * (I.T / 32) * ((I.c / 4 + POP_KB - 1) / POP_KB);
+  const int64_t ctas = genes_out ? (warps * 32 + POP_THREADS - 1) / POP_THREADS
+                                 : (I.NP + POP_THREADS - 1) / POP_THREADS;
+  if (genes_out || fit_out || d_eff_out)
+    k_population<<<(int)std::min<int64_t>(ctas, 8 * sm_count()), POP_THREADS, 0, s>>>(
+        I, genes_out, ld, fit_out, (float2 *)d_eff_out);
   QPM_CUDA(cudaGetLastError());
   return QPM_OK;
 }
@@ -2683,10 +2855,26 @@ extern "C" qpm_status qpm_get_best(qpm_state *st, int32_t inst, float *genes_out
   if (!st->inited) return fail(QPM_ERR_STATE, "qpm_init has not been called");
   const InstDev &I = st->h[inst];
   cudaStream_t s = (cudaStream_t)stream;
-  k_best<<<1, 256, 0, s>>>(I, index_out);
-  if (d_eff64_out || fit_out) k_recheck64<<<1, 256, 0, s>>>(I, d_eff64_out, fit_out);
-  if (genes_out) k_unpermute<<<1, 256, 0, s>>>(I, -2, genes_out, 0);
+  BestRot rot;
+  for (int q = 1; q <= 3; ++q) {
+    rot.r1[q - 1] = make_double2(std::cos(q * I.kappa1), -std::sin(q * I.kappa1));
+    rot.r2[q - 1] = make_double2(std::cos(q * I.kappa2), -std::sin(q * I.kappa2));
+  }
+  const int parts = best_parts(I.N);
+  k_best<<<genes_out || d_eff64_out ? parts : 1, BEST_THREADS, 0, s>>>(I, rot, genes_out, fit_out,
+                                                                       index_out, d_eff64_out != nullptr);
   QPM_CUDA(cudaGetLastError());
+  if (!d_eff64_out) return QPM_OK;
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3(1);
+  cfg.blockDim = dim3(BEST_THREADS);
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  QPM_CUDA(cudaLaunchKernelEx(&cfg, k_best_close, I, parts, d_eff64_out));
   return QPM_OK;
 }
 

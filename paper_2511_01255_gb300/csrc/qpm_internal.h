@@ -33,6 +33,16 @@ int table_part_count(int32_t Npad);
 qpm_status launch_table(const TableSpec &s, float4 *table, double2 *part, float2 *konst,
                         double2 *konst64, cudaStream_t stream);
 
+// the tables and constants of n problems in two launches (d_jobs: device array)
+struct TableJob {
+  TableSpec s;
+  float4 *table;
+  double2 *part;
+  float2 *konst;
+  double2 *konst64;
+};
+qpm_status launch_tables(const TableJob *d_jobs, int n, int32_t max_npad, cudaStream_t stream);
+
 // sign-block table of the row sweeps: 8 patterns x (A, B, C) as float2 for every
 // block of 4 domains, float2 blk[(8 b + e) * 3 + k], ceil(N / 4) blocks (24 float2
 // = 192 bytes each); built in FP64, rounded to FP32

@@ -19,13 +19,21 @@ namespace qpm {
 
 static constexpr int TBL_THREADS = 256;
 
-static __global__ void __launch_bounds__(TBL_THREADS)
-    k_table(TableSpec s, float4 *__restrict__ table, double2 *__restrict__ part) {
+// CTAs of one problem's table, each with one partial diagonal sum
+__host__ __device__ static inline int table_parts(int32_t Npad) {
+  const int n = (Npad + TBL_THREADS - 1) / TBL_THREADS;
+  return n < 1024 ? (n < 1 ? 1 : n) : 1024;
+}
+
+// One problem's table and diagonal sum by `nparts` CTAs of which this is CTA `blk`: the
+// partial sums depend on nparts and blk only, so a launch for one problem and a launch for
+// many give the same bits.
+static __device__ void table_body(const TableSpec &s, int blk, int nparts,
+                                  float4 *__restrict__ table, double2 *__restrict__ part) {
   __shared__ double2 red[TBL_THREADS];
   double2 acc = make_double2(0.0, 0.0);
   const double ks = s.kappa1 + s.kappa2;
-  for (int m = blockIdx.x * TBL_THREADS + threadIdx.x; m < s.Npad;
-       m += gridDim.x * TBL_THREADS) {
+  for (int m = blk * TBL_THREADS + threadIdx.x; m < s.Npad; m += nparts * TBL_THREADS) {
     float4 e = make_float4(0.f, 0.f, 0.f, 0.f);
     if (m < s.N) {
       const double dm = (double)m;
@@ -55,7 +63,12 @@ static __global__ void __launch_bounds__(TBL_THREADS)
     }
     __syncthreads();
   }
-  if (threadIdx.x == 0) part[blockIdx.x] = red[0];
+  if (threadIdx.x == 0) part[blk] = red[0];
+}
+
+static __global__ void __launch_bounds__(TBL_THREADS)
+    k_table(TableSpec s, float4 *__restrict__ table, double2 *__restrict__ part) {
+  table_body(s, blockIdx.x, gridDim.x, table, part);
 }
 
 // phi(k) = int_0^1 e^{-iks} ds = e^{-ik/2} sin(k/2)/(k/2)
@@ -66,10 +79,10 @@ static __device__ double2 phi64(double k) {
   return make_double2(cos(h) * sc, -sin(h) * sc);
 }
 
-static __device__ double2 psi64(double k1, double k2) {
+// a = phi(k2), b = phi(k1 + k2)
+static __device__ double2 psi64(double k1, double k2, const double2 &a, const double2 &b) {
   if (fabs(k1) > 1e-7) {
     // (phi(k2) - phi(k1 + k2)) / (i k1)
-    const double2 a = phi64(k2), b = phi64(k1 + k2);
     const double xr = a.x - b.x, xi = a.y - b.y;
     return make_double2(xi / k1, -xr / k1);
   }
@@ -83,15 +96,30 @@ static __device__ double2 psi64(double k1, double k2) {
   return make_double2(0.5 - k2 * k2 / 8.0, -k2 / 3.0);
 }
 
-static __global__ void k_table_finalize(int nparts, const double2 *__restrict__ part,
-                                        double k1, double k2, float2 *konst, double2 *konst64) {
-  if (threadIdx.x != 0) return;
+// The constants of one problem by one warp, bound by the latency of its FP64 chains: the
+// three phi and psi come from different lanes at once, and the diagonal sum's parts are
+// fetched by all lanes and then added by every lane in part order (the sum's bits depend on
+// that order).  One thread doing all of it, a load per addition, took 10 us at N = 1000 and
+// 48 us at N = 1e5.
+static __device__ void finalize_body(int nparts, const double2 *__restrict__ part, double k1,
+                                     double k2, float2 *konst, double2 *konst64) {
+  const int lane = threadIdx.x & 31;
+  // lane 0 phi(k1), lane 1 phi(k2), lane 2 phi(k1 + k2); psi's small-k1 forms need none
+  const double2 ph = phi64(lane == 0 ? k1 : (lane == 1 ? k2 : k1 + k2));
+  const double2 p1 = make_double2(__shfl_sync(0xffffffffu, ph.x, 0), __shfl_sync(0xffffffffu, ph.y, 0));
+  const double2 p2 = make_double2(__shfl_sync(0xffffffffu, ph.x, 1), __shfl_sync(0xffffffffu, ph.y, 1));
+  const double2 p12 = make_double2(__shfl_sync(0xffffffffu, ph.x, 2), __shfl_sync(0xffffffffu, ph.y, 2));
   double sr = 0.0, si = 0.0;
-  for (int b = 0; b < nparts; ++b) {
-    sr += part[b].x;
-    si += part[b].y;
+  for (int b0 = 0; b0 < nparts; b0 += 32) {
+    const double2 v = b0 + lane < nparts ? part[b0 + lane] : make_double2(0.0, 0.0);
+    const int n = min(32, nparts - b0);
+    for (int b = 0; b < n; ++b) {
+      sr += __shfl_sync(0xffffffffu, v.x, b);
+      si += __shfl_sync(0xffffffffu, v.y, b);
+    }
   }
-  const double2 p1 = phi64(k1), p2 = phi64(k2), ps = psi64(k1, k2);
+  if (lane != 0) return;
+  const double2 ps = psi64(k1, k2, p2, p12);
   const double2 phi12 = make_double2(p1.x * p2.x - p1.y * p2.y, p1.x * p2.y + p1.y * p2.x);
   const double2 cdiag = make_double2(ps.x * sr - ps.y * si, ps.x * si + ps.y * sr);
   konst[0] = make_float2((float)phi12.x, (float)phi12.y);
@@ -103,6 +131,29 @@ static __global__ void k_table_finalize(int nparts, const double2 *__restrict__ 
     konst64[1] = cdiag;
     konst64[2] = ps;
     konst64[3] = p1;
+  }
+}
+
+static __global__ void k_table_finalize(int nparts, const double2 *__restrict__ part,
+                                        double k1, double k2, float2 *konst, double2 *konst64) {
+  finalize_body(nparts, part, k1, k2, konst, konst64);
+}
+
+// The same for n problems in two launches (blockIdx.y the problem): the tables of a state
+// of many instances, whose launches one after the other (7 + 10 us each) were 9 ms of a
+// 512-instance initialisation.
+static __global__ void __launch_bounds__(TBL_THREADS) k_tables(const TableJob *__restrict__ jobs, int n) {
+  for (int k = blockIdx.y; k < n; k += gridDim.y) {
+    const TableJob j = jobs[k];
+    const int nparts = table_parts(j.s.Npad);
+    if ((int)blockIdx.x < nparts) table_body(j.s, blockIdx.x, nparts, j.table, j.part);
+    __syncthreads();  // the reduction scratch is reused
+  }
+}
+static __global__ void k_tables_finalize(const TableJob *__restrict__ jobs, int n) {
+  for (int k = blockIdx.x; k < n; k += gridDim.x) {
+    const TableJob j = jobs[k];
+    finalize_body(table_parts(j.s.Npad), j.part, j.s.kappa1, j.s.kappa2, j.konst, j.konst64);
   }
 }
 
@@ -164,9 +215,15 @@ qpm_status launch_block_table(int32_t N, double kappa1, double kappa2, float2 *b
   return QPM_OK;
 }
 
-int table_part_count(int32_t Npad) {
-  const int n = (Npad + TBL_THREADS - 1) / TBL_THREADS;
-  return n < 1024 ? (n < 1 ? 1 : n) : 1024;
+int table_part_count(int32_t Npad) { return table_parts(Npad); }
+
+qpm_status launch_tables(const TableJob *d_jobs, int n, int32_t max_npad, cudaStream_t stream) {
+  const dim3 grid(table_parts(max_npad), std::min(n, 65535));
+  k_tables<<<grid, TBL_THREADS, 0, stream>>>(d_jobs, n);
+  QPM_CUDA(cudaGetLastError());
+  k_tables_finalize<<<std::min(n, 65535), 32, 0, stream>>>(d_jobs, n);
+  QPM_CUDA(cudaGetLastError());
+  return QPM_OK;
 }
 
 qpm_status launch_table(const TableSpec &s, float4 *table, double2 *part, float2 *konst,
