@@ -3,8 +3,7 @@
 // SHG field (Sec. 2.1, the single integral before the cascade):
 //   E2 prop. to int_0^L d(z) e^{-i dk z} dz = phi(kappa) sum_j d_j e^{-i kappa j},
 // used by the multi-wavelength SHG designs of Sec. 5.  A plain complex sum per
-// row: each CTA takes 8 rows, each thread 4-domain groups spaced by the CTA width
-// (coalesced float4 loads), so one phasor read serves the 8 rows.
+// row: one CTA per SM takes an equal run of rows, its warps segments of domains.
 //
 // Multi-wavelength objective (Sec. 5): f = sum_k |G0 - G_k| + beta (G_max - G_min)
 // with G_k = |d_eff(kappa1_k, kappa2_k)|, to be minimised.  The K cascaded scans
@@ -23,68 +22,156 @@
 namespace qpm {
 
 // ------------------------------------------------------------------ SHG field
-static constexpr int SHG_ROWS = 8;
-static constexpr int SHG_THREADS = 256;
+// Bound by HBM (4 bytes a domain, 2 FMA), so all that counts is bytes in flight and an even
+// share per SM.  One CTA per SM takes an equal run of rows.  Its work items are (segment of
+// 384 domains, block of 4 rows), dealt to the 16 warps as equal runs in segment-major order,
+// so a warp holds the segment's phasors in registers from item to item, issues the 12 16-byte
+// loads of an item at once (6 KB a warp, 96 KB an SM) and reduces the item's 4 row sums by
+// halving exchanges (9 shuffles for the 8 components).  Each warp adds its items into its own
+// row sums in shared memory; the CTA adds the warps' in warp order at the end.
+// 5000 rows of N = 3000 (60 MB): the form before it, a CTA per 8 rows that read the phasors
+// from L2 once per CTA, took 29.9 us: 625 CTAs on 608 slots, i.e. a second wave for 17 CTAs.
+static constexpr int SHG_WARPS = 16;
+static constexpr int SHG_Q = 2;                 // 128-domain pieces per segment
+static constexpr int SHG_SEG = 128 * SHG_Q;
+static constexpr int SHG_RB = 4;                // rows per item
+static constexpr int SHG_RMAX = 64;             // rows whose sums are kept at a time
 
+// VEC: rows of 16-byte aligned groups, lane l takes domains 4 l .. 4 l + 3 of a piece with one
+// load; else lane l takes domains l, l + 32, l + 64, l + 96, so that every load of a warp is 128
+// contiguous bytes whatever the rows' alignment.
 template <bool VEC>
-static __global__ void __launch_bounds__(SHG_THREADS)
-    k_shg(const float *__restrict__ genes, int64_t ld, int NP, int N,
+static __global__ void __launch_bounds__(SHG_WARPS * 32, 1)
+    k_shg(const float *__restrict__ genes, int64_t ld, int NP, int N, int rows_per_cta,
           const float4 *__restrict__ table, const float2 *__restrict__ konst,
           float2 *__restrict__ eout, float *__restrict__ fout) {
-  __shared__ float2 red[SHG_THREADS / 32][SHG_ROWS];
-  const int r0 = blockIdx.x * SHG_ROWS;
-  float2 S[SHG_ROWS];
-#pragma unroll
-  for (int r = 0; r < SHG_ROWS; ++r) S[r] = make_float2(0.f, 0.f);
-  for (int m = 4 * threadIdx.x; m < N; m += 4 * SHG_THREADS) {
-    float2 p[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const float4 t = m + q < N ? __ldg(table + m + q) : make_float4(0.f, 0.f, 0.f, 0.f);
-      p[q] = make_float2(t.x, t.y);  // e^{-i kappa m}
-    }
-#pragma unroll
-    for (int r = 0; r < SHG_ROWS; ++r) {
-      if (r0 + r >= NP) break;
-      const float *row = genes + (int64_t)(r0 + r) * ld;
-      float x[4];
-      if (VEC && m + 4 <= N) {
-        const float4 v = __ldg((const float4 *)(row + m));
-        x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
-      } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) x[q] = m + q < N ? __ldg(row + m + q) : 0.f;
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const float d = x[q] < 0.f ? -1.f : 1.f;
-        S[r].x = fmaf(d, p[q].x, S[r].x);
-        S[r].y = fmaf(d, p[q].y, S[r].y);
-      }
-    }
-  }
+  __shared__ float sums[SHG_WARPS][2 * SHG_RMAX];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rend = (int)min((int64_t)NP, (int64_t)(blockIdx.x + 1) * rows_per_cta);
+  const int nseg = (N + SHG_SEG - 1) / SHG_SEG;
+  const int glast = 4 * (N >> 2) - 4;  // the row's last whole group (VEC: N >= 4)
+  for (int64_t rs = (int64_t)blockIdx.x * rows_per_cta; rs < rend; rs += SHG_RMAX) {
+    const int r0 = (int)rs, rn = min(SHG_RMAX, rend - r0), nrb = (rn + SHG_RB - 1) / SHG_RB;
+    for (int e = threadIdx.x; e < SHG_WARPS * 2 * SHG_RMAX; e += SHG_WARPS * 32)
+      (&sums[0][0])[e] = 0.f;
+    __syncthreads();
+    const int64_t items = (int64_t)nseg * nrb;
+    const int64_t i0 = items * warp / SHG_WARPS, i1 = items * (warp + 1) / SHG_WARPS;
+    int seg = (int)(i0 / nrb), rb = (int)(i0 - (int64_t)seg * nrb);
+    int nseg_x = seg, nrb_x = rb;  // the item whose loads are issued next
+    // the lane's domain q of piece k of segment sg
+    auto dom = [&](int sg, int k, int q) {
+      return sg * SHG_SEG + 128 * k + (VEC ? 4 * lane + q : lane + 32 * q);
+    };
+    float4 x[SHG_RB][SHG_Q], y[SHG_RB][SHG_Q];  // this item's genes, the next one's in flight
+    auto fetch = [&]() {
 #pragma unroll
-  for (int r = 0; r < SHG_ROWS; ++r) {
+      for (int r = 0; r < SHG_RB; ++r) {
+        const int row = min(r0 + nrb_x * SHG_RB + r, rend - 1);  // a repeated row's sums are dropped
+        const float *g = genes + (int64_t)row * ld;
 #pragma unroll
-    for (int s = 16; s > 0; s >>= 1) {
-      S[r].x += __shfl_xor_sync(0xffffffffu, S[r].x, s);
-      S[r].y += __shfl_xor_sync(0xffffffffu, S[r].y, s);
+        for (int k = 0; k < SHG_Q; ++k) {
+          // no load under a condition, so that all of an item's are in flight together: past
+          // the row they repeat its last domains, whose phasors below are zero
+          if (VEC) {
+            y[r][k] = __ldg((const float4 *)(g + min(dom(nseg_x, k, 0), glast)));
+          } else {
+            y[r][k] = make_float4(
+                __ldg(g + min(dom(nseg_x, k, 0), N - 1)), __ldg(g + min(dom(nseg_x, k, 1), N - 1)),
+                __ldg(g + min(dom(nseg_x, k, 2), N - 1)), __ldg(g + min(dom(nseg_x, k, 3), N - 1)));
+          }
+        }
+      }
+      if (++nrb_x == nrb) {
+        nrb_x = 0;
+        ++nseg_x;
+      }
+    };
+    if (i0 < i1) fetch();
+    float2 p[SHG_Q * 4];  // e^{-i kappa m} of the lane's domains of the segment
+    bool fresh = true;
+    for (int64_t it = i0; it < i1; ++it) {
+#pragma unroll
+      for (int r = 0; r < SHG_RB; ++r)
+#pragma unroll
+        for (int k = 0; k < SHG_Q; ++k) x[r][k] = y[r][k];
+      if (it + 1 < i1) fetch();
+      if (VEC && (N & 3) != 0 && (seg + 1) * SHG_SEG > N) {  // the row's last, partial group
+#pragma unroll
+        for (int k = 0; k < SHG_Q; ++k) {
+          if (dom(seg, k, 0) == glast + 4) {
+#pragma unroll
+            for (int r = 0; r < SHG_RB; ++r) {
+              const float *g = genes + (int64_t)min(r0 + rb * SHG_RB + r, rend - 1) * ld;
+              x[r][k] = make_float4(__ldg(g + dom(seg, k, 0)), __ldg(g + min(dom(seg, k, 1), N - 1)),
+                                    __ldg(g + min(dom(seg, k, 2), N - 1)), 0.f);
+            }
+          }
+        }
+      }
+      if (fresh) {
+#pragma unroll
+        for (int k = 0; k < SHG_Q; ++k)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const float4 e = __ldg(table + min(dom(seg, k, q), N - 1));
+            p[4 * k + q] = dom(seg, k, q) < N ? make_float2(e.x, e.y) : make_float2(0.f, 0.f);
+          }
+        fresh = false;
+      }
+      float v[2 * SHG_RB];  // (re, im) of the 4 rows' partial sums
+#pragma unroll
+      for (int r = 0; r < SHG_RB; ++r) {
+        float sx = 0.f, sy = 0.f;
+#pragma unroll
+        for (int k = 0; k < SHG_Q; ++k) {
+          const float g4[4] = {x[r][k].x, x[r][k].y, x[r][k].z, x[r][k].w};
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const float d = g4[q] < 0.f ? -1.f : 1.f;
+            sx = fmaf(d, p[4 * k + q].x, sx);
+            sy = fmaf(d, p[4 * k + q].y, sy);
+          }
+        }
+        v[2 * r] = sx;
+        v[2 * r + 1] = sy;
+      }
+      // 8 values over 32 lanes: three halving exchanges leave lane l the value l / 4 summed
+      // over 8 lanes, two more steps sum the rest
+#pragma unroll
+      for (int w = SHG_RB, o = 16; w >= 1; w >>= 1, o >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int e = 0; e < w; ++e) {
+          const float keep = up ? v[w + e] : v[e], give = up ? v[e] : v[w + e];
+          v[e] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+      }
+      float t = v[0];
+      t += __shfl_xor_sync(0xffffffffu, t, 2);
+      t += __shfl_xor_sync(0xffffffffu, t, 1);
+      if ((lane & 3) == 0 && rb * SHG_RB + (lane >> 3) < rn) sums[warp][2 * SHG_RB * rb + (lane >> 2)] += t;
+      if (++rb == nrb) {
+        rb = 0;
+        ++seg;
+        fresh = true;
+      }
     }
-    if (lane == 0) red[warp][r] = S[r];
-  }
-  __syncthreads();
-  if (threadIdx.x < SHG_ROWS && r0 + (int)threadIdx.x < NP) {
+    __syncthreads();
     const int r = threadIdx.x;
-    float2 t = red[0][r];
-    for (int w = 1; w < SHG_THREADS / 32; ++w) {
-      t.x += red[w][r].x;
-      t.y += red[w][r].y;
+    if (r < rn) {
+      float2 t = make_float2(sums[0][2 * r], sums[0][2 * r + 1]);
+#pragma unroll
+      for (int w = 1; w < SHG_WARPS; ++w) {
+        t.x += sums[w][2 * r];
+        t.y += sums[w][2 * r + 1];
+      }
+      const float2 ph = konst[3];  // phi(kappa)
+      const float2 E = make_float2(ph.x * t.x - ph.y * t.y, ph.x * t.y + ph.y * t.x);
+      eout[r0 + r] = E;
+      if (fout) fout[r0 + r] = fit_of(E);
     }
-    const float2 ph = konst[3];  // phi(kappa)
-    const float2 E = make_float2(ph.x * t.x - ph.y * t.y, ph.x * t.y + ph.y * t.x);
-    eout[r0 + r] = E;
-    if (fout) fout[r0 + r] = fit_of(E);
+    __syncthreads();  // the sums are zeroed again
   }
 }
 
@@ -236,12 +323,14 @@ extern "C" qpm_status qpm_eval_shg(const qpm_problem *prob, const float *genes, 
   const float2 *konst;
   qpm_status st = lease.table(prob, s, &table, &konst);
   if (st != QPM_OK) return st;
-  const bool vec = (ld % 4 == 0) && (((uintptr_t)genes & 15) == 0);
-  const int grid = (NP + SHG_ROWS - 1) / SHG_ROWS;
+  const bool vec = (ld % 4 == 0) && (((uintptr_t)genes & 15) == 0) && prob->N >= 4;
+  const int rpc = (NP + sm_count() - 1) / sm_count(), grid = (NP + rpc - 1) / rpc;
   if (vec)
-    k_shg<true><<<grid, SHG_THREADS, 0, s>>>(genes, ld, NP, prob->N, table, konst, (float2 *)e_shg, fit);
+    k_shg<true><<<grid, SHG_WARPS * 32, 0, s>>>(genes, ld, NP, prob->N, rpc, table, konst,
+                                                (float2 *)e_shg, fit);
   else
-    k_shg<false><<<grid, SHG_THREADS, 0, s>>>(genes, ld, NP, prob->N, table, konst, (float2 *)e_shg, fit);
+    k_shg<false><<<grid, SHG_WARPS * 32, 0, s>>>(genes, ld, NP, prob->N, rpc, table, konst,
+                                                 (float2 *)e_shg, fit);
   QPM_CUDA(cudaGetLastError());
   return QPM_OK;
 }
