@@ -1,25 +1,17 @@
 // qpm_eval.cu -- fitness of caller-supplied sign sequences (Sec. 2.1).
 //
-// Work split: a warp takes 32 rows (lane = row) and one segment of L domains (L a
-// multiple of 128) and sweeps it in index order, so every row's running monoid
-// (A, B, C) is a plain sequential accumulation.  The sweep appends a block of 4
-// domains per lookup in the sign-block table (the block's monoid triple for its sign
-// pattern, precomputed in FP64), whose entries are streamed into shared memory per
-// step of 128 domains, the next step's with cp.async while this one is swept.
-// Float genes arrive 32 domains at a time and are transposed through per-warp
-// shared-memory tiles: rows that are 16-byte aligned through a ring of ER_RING tiles
-// filled by cp.async ER_RING - 1 sub-steps ahead, other rows with register loads one
-// sub-step ahead.  Packed sign
-// words (32 domains each) are read four at a time straight into the lane of their
-// row.  The warps of a CTA take consecutive row groups of the same segment and
-// synchronise once per step of 128 domains.  A second kernel (a warp per row) combines
-// the S segment partials of every row in index order and closes
-// d_eff = phi1 phi2 C + cdiag.
+// The row sweep of qpm_rows.cuh with one sign-block table: a warp takes 32 rows (lane = row) and
+// appends one table entry per block of 4 domains.  Float genes arrive as 32 x 32 tiles by TMA
+// (rows of any alignment, see GeneMaps) and are transposed through the tile; packed sign words
+// (32 domains each) are read four at a time straight into the lane of their row.  A second kernel
+// combines the pieces of every row in index order and closes d_eff = phi1 phi2 C + cdiag.
 #include <math.h>
 
 #include <algorithm>
 #include <map>
 #include <mutex>
+#include <string.h>
+
 #include <string>
 #include <tuple>
 
@@ -29,166 +21,114 @@
 
 namespace qpm {
 
-// partial monoids, structure of arrays: part[(comp * S + s) * NPpad + i], comp in A,B,C
-// Float genes of rows that are not 16-byte aligned (scalar loads, one sub-step ahead
-// in registers).  blk: the problem's sign-block table, read as float4.
-// grid (S, ceil(groups / ER_WPC)).
-template <bool COMP>
-static __global__ void __launch_bounds__(ER_WPC * 32, 5)
-    k_eval_rows(const float *__restrict__ src, int64_t ld, EvalShape sh,
-                const float4 *__restrict__ blk, float2 *__restrict__ part) {
-  extern __shared__ float4 tb[];  // two steps of sign-block entries
-  __shared__ float4 tile[ER_WPC][256];
+// resident CTAs of the packed sweep per SM: 8 warps of 64 registers, or 2 warps (up to 64 rows)
+constexpr int ep_ctas(int W) { return W == 8 ? 4 : 8; }
+
+// float genes: see rows_sweep; ctr not NULL: the sweep combines the rows itself
+template <int W, int MODE, bool COMP>
+static __global__ void __launch_bounds__(W * 32, rs_ctas(1, W))
+    k_eval_genes(const __grid_constant__ GeneMaps maps, const float *__restrict__ src, int64_t ld,
+                 RowPlan pl, RowTables<1> tabs, float2 *part, unsigned *ctr,
+                 const float2 *__restrict__ konst, float2 *__restrict__ deff,
+                 float *__restrict__ fit) {
+  rows_sweep<1, W, MODE, COMP>(maps, src, ld, pl, tabs, part, ctr, [&](int row, const Mono *m) {
+    const float2 D = deff_from(m[0], konst[0], konst[1]);
+    deff[row] = D;
+    if (fit) fit[row] = fit_of(D);
+  });
+}
+
+// Packed sign words.  Bound by the shared-memory data path (a lookup returns 24 bytes a lane: 6
+// cycles of the SM's 128 bytes per block of 4 domains and warp), so the rest is kept below it:
+// the 8 nibbles of a word cost one byte permute and one multiply each, and the 16-pattern table
+// needs no sign flips.  Units of 128 domains (a word quadruple, 16-byte loads when VECW).
+template <int W, bool VECW, bool COMP>
+static __global__ void __launch_bounds__(W * 32, ep_ctas(W))
+    k_eval_packed(const uint32_t *__restrict__ src, int64_t ld, RowPlan pl, RowTables<1> tabs,
+                  float2 *__restrict__ part) {
+  __shared__ __align__(16) unsigned char tab[2 * RS_TAB];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int s = blockIdx.x, m0 = s * sh.L, m1 = min(sh.N, m0 + sh.L);
-  const int r0 = (blockIdx.y * ER_WPC + warp) * 32;
-  const bool live = r0 < sh.NP;
-  const int nb = (sh.N + 3) >> 2, nsteps = (m1 - m0 + 127) >> 7;
-  float4 R[8];
-  if (live) er_load_genes<false>(src, ld, sh, r0, m0, R);
-  er_stage_step(tb, blk, m0, 0, nb);
-  const float2 *bt = (const float2 *)tb;
-  ErAcc<COMP> acc;
-  acc.zero();
-  float4 *T = tile[warp];
-  for (int k = 0; k < nsteps; ++k) {
-    cp_async_wait<0>();  // this thread's copies of step k
-    __syncthreads();     // everyone's copies of step k; everyone done with step k - 1
-    if (k + 1 < nsteps) er_stage_step(tb + ((k + 1) & 1) * ER_STEP_F4_P, blk, m0, k + 1, nb);
-    if (!live) continue;
-    const float2 *bp = bt + (size_t)(k & 1) * 2 * ER_STEP_F4_P;
-#pragma unroll 1
-    for (int q = 0; q < 4; ++q) {  // 4 sub-steps of 32 domains
-      const int ms = m0 + 128 * k + 32 * q;
-      if (ms >= m1) break;
-      __syncwarp();
-#pragma unroll
-      for (int j = 0; j < 8; ++j) T[er_tix(4 * j + (lane >> 3), lane & 7)] = R[j];
-      __syncwarp();
-      if (ms + 32 < m1) er_load_genes<false>(src, ld, sh, r0, ms + 32, R);
-#pragma unroll
-      for (int c4 = 0; c4 < 8; ++c4) {  // the sub-step's 8 blocks of 4 domains
-        er_push_block(acc.m, er_pattern(T[er_tix(lane, c4)]), bp + (8 * q + c4) * BLK_F2);
-        if ((c4 & 3) == 3) acc.fold();
+  const int nb = (pl.N + 3) >> 2, nw = (pl.N + 31) >> 5;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");  // genes, tables, the partials' last readers
+  const int64_t per = (int64_t)pl.nunit * pl.gran;
+  const int64_t f1 = rp_start(pl, (int64_t)blockIdx.x + 1);
+  for (int64_t f = rp_start(pl, blockIdx.x); f < f1;) {
+    const int b = (int)(f / per), u0 = (int)(f - b * per);
+    const int u1 = (int)min(per, (int64_t)u0 + (f1 - f));
+    f += u1 - u0;
+    const int row = (b * W + warp) * 32 + lane, rr = min(row, pl.NP - 1);
+    const bool live = (b * W + warp) * 32 < pl.NP;
+    const int w0 = u0, nsteps = (min(u1, pl.nsub) - u0 + 3) >> 2;  // u0 is a multiple of 4
+    const uint32_t *rp = src + (int64_t)rr * ld;
+    // words past the row's last are never read; their blocks have zero entries
+    auto words = [&](int w) {
+      if (VECW && w + 4 <= nw) return __ldg((const uint4 *)(rp + w));
+      return make_uint4(__ldg(rp + min(w, nw - 1)), __ldg(rp + min(w + 1, nw - 1)),
+                        __ldg(rp + min(w + 2, nw - 1)), __ldg(rp + min(w + 3, nw - 1)));
+    };
+    StepRegs<W> R;
+    R.load(tabs.blk[0], 8 * w0, nb);
+    uint4 nxt = words(w0);
+    __syncthreads();  // the table buffers of the piece before are free
+    R.store(tab);
+    if (nsteps > 1) R.load(tabs.blk[0], 8 * w0 + 32, nb);
+    RowAcc<COMP> acc;
+    acc.zero();
+    for (int k = 0; k < nsteps; ++k) {
+      __syncthreads();  // step k is staged; everyone is done with step k - 1
+      if (k + 1 < nsteps) {
+        R.store(tab + ((k + 1) & 1) * RS_TAB);
+        if (k + 2 < nsteps) R.load(tabs.blk[0], 8 * w0 + 32 * (k + 2), nb);
       }
-    }
-  }
-  if (!live) return;
-  acc.fold();
-  const Mono run = acc.get();
-  const size_t stride = (size_t)sh.S * sh.NPpad;
-  const size_t o = (size_t)s * sh.NPpad + r0 + lane;
-  part[o] = run.A;
-  part[stride + o] = run.B;
-  part[2 * stride + o] = run.C;
-}
-
-// Float genes of 16-byte aligned rows through the per-warp ring of er_ring_sweep (60 KB
-// of shared memory per CTA, 3 CTAs per SM); the accumulation order equals k_eval_rows'.
-// grid (S, ceil(groups / ER_WPC)).
-constexpr int ER_RING_CTAS = 3;  // resident CTAs per SM (shared memory)
-// TMA: the gene tiles come by TMA copies (er_ring_sweep_tma, `gmap`), else by cp.async.
-template <bool COMP, bool TMA>
-static __global__ void __launch_bounds__(ER_WPC * 32, ER_RING_CTAS)
-    k_eval_rows_ring(const __grid_constant__ CUtensorMap gmap, const float *__restrict__ src,
-                     int64_t ld, EvalShape sh, const float4 *__restrict__ blk,
-                     float2 *__restrict__ part) {
-  extern __shared__ float4 dyn_raw[];
-  float4 *dyn = dyn_raw;
-  if constexpr (TMA)  // 1024-byte aligned for the swizzled tiles (the launch adds the slack)
-    dyn = (float4 *)((unsigned char *)dyn_raw + ((1024 - (smem_u32(dyn_raw) & 1023)) & 1023));
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int s = blockIdx.x, m0 = s * sh.L, m1 = min(sh.N, m0 + sh.L);
-  const int r0 = (blockIdx.y * ER_WPC + warp) * 32;
-  const bool live = r0 < sh.NP;
-  const float4 *const tabs[1] = {blk};
-  ErAcc<COMP> acc;
-  acc.zero();
-  auto push = [&](uint32_t e, const float2 *E, int b) {
-    er_push_block(acc.m, e, E + b * BLK_F2);
-    if ((b & 3) == 3) acc.fold();
-  };
-  if constexpr (TMA) er_ring_sweep_tma<1>(dyn, &gmap, sh, tabs, m0, m1, r0, live, push);
-  else er_ring_sweep<1>(dyn, src, ld, sh, tabs, m0, m1, r0, live, push);
-  if (!live) return;
-  acc.fold();
-  const Mono run = acc.get();
-  const size_t stride = (size_t)sh.S * sh.NPpad;
-  const size_t o = (size_t)s * sh.NPpad + r0 + lane;
-  part[o] = run.A;
-  part[stride + o] = run.B;
-  part[2 * stride + o] = run.C;
-}
-
-// Packed sign words: the sign-block sweep.  A CTA of ER_WPC_P warps takes ER_WPC_P
-// row groups of one segment; per block of 4 domains the lane's 4 sign bits select the
-// block's triple among the staged sign-block entries (conflict-free: the 8 entries of
-// a block fall in distinct banks).  The entries are streamed per step of 128 domains
-// (32 blocks, 6 KB) into two buffers with cp.async, the next step's while this one
-// is swept, behind one CTA barrier per step; the sign words come one step ahead in
-// registers.  Compensation folds every 4 blocks.  VECW: 16-byte word loads.
-// grid (S, ceil(groups / ER_WPC_P)).
-template <bool VECW, bool COMP>
-static __global__ void __launch_bounds__(ER_WPC_P * 32)
-    k_eval_packed(const uint32_t *__restrict__ src, int64_t ld, EvalShape sh,
-                  const float4 *__restrict__ blk, float2 *__restrict__ part) {
-  extern __shared__ float4 tb[];  // two steps of sign-block entries
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int s = blockIdx.x, m0 = s * sh.L, m1 = min(sh.N, m0 + sh.L);
-  const int r0 = (blockIdx.y * ER_WPC_P + warp) * 32;
-  const bool live = r0 < sh.NP;
-  const int nb = (sh.N + 3) >> 2, nsteps = (m1 - m0 + 127) >> 7;
-  uint4 W = make_uint4(0u, 0u, 0u, 0u);
-  if (live) W = er_load_words<VECW>(src, ld, sh, r0 + lane, m0);
-  er_stage_step(tb, blk, m0, 0, nb);
-  const float2 *bt = (const float2 *)tb;
-  ErAcc<COMP> acc;
-  acc.zero();
-  for (int k = 0; k < nsteps; ++k) {
-    cp_async_wait<0>();  // this thread's copies of step k
-    __syncthreads();     // everyone's copies of step k; everyone done with step k - 1
-    if (k + 1 < nsteps) er_stage_step(tb + ((k + 1) & 1) * ER_STEP_F4_P, blk, m0, k + 1, nb);
-    if (live) {
-      const int ms = m0 + 128 * k;
-      const uint4 cur = W;
-      if (ms + 128 < m1) W = er_load_words<VECW>(src, ld, sh, r0 + lane, ms + 128);
-      const float2 *bp = bt + (size_t)(k & 1) * 2 * ER_STEP_F4_P;
-      const uint32_t ws[4] = {cur.x, cur.y, cur.z, cur.w};
+      if (!live) continue;
+      const uint32_t ws[4] = {nxt.x, nxt.y, nxt.z, nxt.w};
+      if (k + 1 < nsteps) nxt = words(w0 + 4 * (k + 1));
+      const unsigned char *E = tab + (k & 1) * RS_TAB;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const ErWord f = er_fold_word(ws[q]);
+        const uint32_t lo = ws[q] & 0x0F0F0F0Fu, hi = (ws[q] >> 4) & 0x0F0F0F0Fu;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {  // the word's 8 blocks of 4 domains
-          er_push_entry(acc.m, (f.folded >> (4 * j + 1)) & 7u, (f.lo << (31 - 4 * j)) & 0x80000000u,
-                        bp + (8 * q + j) * BLK_F2);
+          const uint32_t e = __byte_perm((j & 1) ? hi : lo, 0u, 0x4440u + (j >> 1));
+          rs_push(acc.m, E + (8 * q + j) * RS_BLOCK + e * RS_ENTRY);
           if ((j & 3) == 3) acc.fold();
         }
       }
+      acc.step();
+    }
+    if (row < pl.NP) {
+      const int piece = (int)blockIdx.x - rp_first(pl, (int64_t)b * pl.nunit);
+      const Mono m = acc.get();
+      float2 *o = part + (size_t)piece * 3 * pl.NPpad + row;
+      o[0] = m.A;
+      o[pl.NPpad] = m.B;
+      o[2 * (size_t)pl.NPpad] = m.C;
     }
   }
-  if (!live) return;
-  acc.fold();
-  const Mono run = acc.get();
-  const size_t stride = (size_t)sh.S * sh.NPpad;
-  const size_t o = (size_t)s * sh.NPpad + r0 + lane;
-  part[o] = run.A;
-  part[stride + o] = run.B;
-  part[2 * stride + o] = run.C;
 }
 
-// one warp per row: d_eff = phi1 phi2 C + cdiag of the combined segments
-static __global__ void k_eval_combine(EvalShape sh, const float2 *__restrict__ part,
-                                      const float2 *__restrict__ konst, float2 *__restrict__ deff,
-                                      float *__restrict__ fit) {
-  const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (row >= sh.NP) return;
-  const Mono acc = combine_segments(part, sh.S, sh.NPpad, row);
-  if ((threadIdx.x & 31) == 0) {
-    const float2 D = deff_from(acc, konst[0], konst[1]);
+// d_eff = phi1 phi2 C + cdiag of the combined pieces; a programmatic dependent of the sweep
+static __global__ void __launch_bounds__(RC_THREADS)
+    k_eval_combine(RowPlan pl, int runs, const float2 *__restrict__ part,
+                   const float2 *__restrict__ konst, float2 *__restrict__ deff,
+                   float *__restrict__ fit) {
+  __shared__ Mono sh[1][RC_THREADS];
+  const int rows = RC_THREADS / runs, run = threadIdx.x / rows;
+  const int row = blockIdx.x * rows + threadIdx.x - run * rows;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  Mono acc[1];
+  combine_pieces<1>(pl, part, runs, row, run, sh, acc);
+  if (run == 0 && row < pl.NP) {
+    const float2 D = deff_from(acc[0], konst[0], konst[1]);
     deff[row] = D;
     if (fit) fit[row] = fit_of(D);
   }
 }
+
+// counters of the fused combination, at the start of every scratch buffer
+constexpr int FUSE_BLOCKS = 4096;
+constexpr size_t FUSE_BYTES = sizeof(unsigned) * FUSE_BLOCKS;
 
 // ------------------------------------------------------------- caches (host)
 namespace {
@@ -317,6 +257,12 @@ qpm_status get_scratch(cudaStream_t stream, size_t bytes, void **ptr) {
       e.bytes = 0;
     }
     QPM_CUDA(cudaMalloc(&e.ptr, bytes));
+    const cudaError_t ce = cudaMemsetAsync(e.ptr, 0, std::min(bytes, FUSE_BYTES), stream);
+    if (ce != cudaSuccess) {  // no scratch without its counters
+      cudaFree(e.ptr);
+      e.ptr = nullptr;
+      return cuda_fail(ce, "clearing the scratch counters");
+    }
     e.bytes = bytes;
   }
   *ptr = e.ptr;
@@ -324,68 +270,153 @@ qpm_status get_scratch(cudaStream_t stream, size_t bytes, void **ptr) {
 }
 }  // namespace
 
-// split for the row sweep: about `warps_per_sm` warps per SM in total (20 suit
-// float genes; the packed sweep holds fewer registers and runs best near 32),
-// segments a multiple of ER_LQ domains and at most ER_LMAX
-EvalShape eval_rows_shape(int NP, int N, int warps_per_sm, int lmax) {
-  EvalShape sh;
-  sh.NP = NP;
-  sh.N = N;
-  sh.groups = (NP + 31) / 32;
-  sh.NPpad = sh.groups * 32;
-  const int target = sm_count() * warps_per_sm;
-  const int S0 = std::max(1, (target + sh.groups - 1) / sh.groups);
-  int L = (N + S0 - 1) / S0;
-  L = (L + ER_LQ - 1) / ER_LQ * ER_LQ;
-  L = std::min(std::max(L, ER_LQ), lmax > 0 ? lmax : ER_LMAX);
-  sh.L = L;
-  sh.S = (N + L - 1) / L;
-  return sh;
+RowPlan row_plan(int NP, int N, int W, int slots, int gran, int maxsub, int min_units) {
+  RowPlan p;
+  p.NP = NP;
+  p.N = N;
+  const int groups = (NP + 31) / 32;
+  p.NPpad = groups * 32;
+  p.W = W;
+  p.RB = (groups + W - 1) / W;
+  p.nsub = (N + 31) / 32;
+  p.gran = gran;
+  p.nunit = (p.nsub + gran - 1) / gran;
+  const int64_t tot = (int64_t)p.RB * p.nunit, full = (int64_t)slots * sm_count();
+  // whole rounds of the resident CTAs, as few as keep every run within maxsub
+  const int64_t rounds = (tot * gran + full * maxsub - 1) / (full * maxsub);
+  int64_t C = std::max<int64_t>(1, rounds) * full;
+  C = std::min(C, std::max<int64_t>(1, tot / min_units));
+  p.C = (int)C;
+  // a row block of nunit units touches at most this many runs of floor(tot / C) or more units
+  const int64_t q = std::max<int64_t>(1, tot / C);
+  p.P = (int)std::min<int64_t>(std::min<int64_t>(p.nunit, C), (p.nunit + q - 1) / q + 1);
+  return p;
 }
 
-// shape of the float-gene sweep: the ring kernel for aligned rows keeps ER_WPC x
-// ER_RING_CTAS warps per SM, the register-prefetch kernel 20
-static EvalShape eval_genes_shape(int NP, int N, bool aligned) {
-  return eval_rows_shape(NP, N, aligned ? ER_WPC * ER_RING_CTAS : 20);
+// Warps per CTA.  One table: 4 (12 warps an SM in 3 CTAs); a single group of rows: 1 (6 warps an
+// SM, where 4 would keep 3 alive).  K tables: 8 warps share the staged steps (8 warps an SM),
+// or 2 where that keeps more warps alive (few row groups).
+static int genes_warps(int K, int NP) {
+  const int g = (NP + 31) / 32, few = K == 1 ? 1 : 2, many = K == 1 ? 4 : 8;
+  auto alive = [&](int W) {  // live warps per SM
+    return (double)W * rs_ctas(K, W) * g / ((g + W - 1) / W * W);
+  };
+  return alive(few) > alive(many) ? few : many;
+}
+RowPlan genes_plan(int K, int NP, int N, bool whole) {
+  const int W = genes_warps(K, NP);
+  if (!whole) return row_plan(NP, N, W, rs_ctas(K, W), 1, RS_MAXSUB, 4);
+  // runs of whole rows, cut only where a row is longer than a run may be
+  const int nsub = (N + 31) / 32, runs = (nsub + RS_MAXSUB - 1) / RS_MAXSUB;
+  RowPlan p = row_plan(NP, N, W, 1, (nsub + runs - 1) / runs, nsub, 1);
+  p.C = p.RB * p.nunit;
+  p.P = p.nunit;
+  return p;
+}
+static RowPlan packed_plan(int NP, int N, int W) {
+  return row_plan(NP, N, W, ep_ctas(W), 4, 128, 1);
 }
 
-static qpm_status launch_eval_rows(bool aligned, bool comp, const float *g, int64_t ld,
-                                   const EvalShape &sh, const float2 *blk, float2 *part,
-                                   cudaStream_t stream) {
-  const dim3 grid(sh.S, (sh.groups + ER_WPC - 1) / ER_WPC);
-  const float4 *b4 = (const float4 *)blk;
-  if (aligned) {
-    CUtensorMap gmap{};
-    const bool tma = make_tile_map(&gmap, g, sh.NP, sh.N, ld);
-    const void *fn = tma ? (comp ? (const void *)k_eval_rows_ring<true, true>
-                                 : (const void *)k_eval_rows_ring<false, true>)
-                         : (comp ? (const void *)k_eval_rows_ring<true, false>
-                                 : (const void *)k_eval_rows_ring<false, false>);
-    const size_t smem = tma ? 1024 + er_ring_smem_tma(1) : er_ring_smem(1);
-    QPM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    void *args[] = {(void *)&gmap, (void *)&g, (void *)&ld, (void *)&sh, (void *)&b4, (void *)&part};
-    QPM_CUDA(cudaLaunchKernel(fn, grid, dim3(ER_WPC * 32), args, smem, stream));
-  } else {
-    const size_t smem = sizeof(float4) * 2 * ER_STEP_F4_P;
-    if (comp) k_eval_rows<true><<<grid, ER_WPC * 32, smem, stream>>>(g, ld, sh, b4, part);
-    else k_eval_rows<false><<<grid, ER_WPC * 32, smem, stream>>>(g, ld, sh, b4, part);
+qpm_status make_gene_maps(GeneMaps *gm, int *mode, const float *genes, int NP, int N, int64_t ld) {
+  memset(gm, 0, sizeof(*gm));
+  const int64_t row = ((int64_t)N + 3) & ~(int64_t)3;  // the pitch of a matrix of one row
+  *mode = ROWS_TMA;
+  if (make_tile_map(&gm->m[0], genes, NP, N, NP == 1 ? row : ld, 32)) return QPM_OK;
+  *mode = ROWS_TMA4;
+  for (int c = 0; c < 4; ++c) {
+    const float *first = genes + (int64_t)std::min(c, NP - 1) * ld;  // a class without rows maps row NP - 1
+    const int s = (int)(((uintptr_t)first & 15) / 4);
+    gm->shift[c] = s;
+    const int rows = c < NP ? (NP - c + 3) / 4 : 1;
+    if (!make_tile_map(&gm->m[c], first - s, rows, (int64_t)N + s, rows == 1 ? row + 4 : 4 * ld, 8))
+      return fail(QPM_ERR_CUDA, "cuTensorMapEncodeTiled refused the genes' tensor map");
   }
   return QPM_OK;
 }
 
-static void launch_eval_packed(bool vecw, bool comp, const uint32_t *src, int64_t ld,
-                               const EvalShape &sh, const float2 *blk, float2 *part,
+// what closes a call: the counters of the fused combination (NULL: the combining kernel), the
+// constants and the outputs
+struct EvalOut {
+  unsigned *ctr;
+  const float2 *konst;
+  float2 *deff;
+  float *fit;
+};
+
+template <int W, int MODE, bool COMP>
+static qpm_status launch_genes(const GeneMaps &gm, const float *g, int64_t ld, const RowPlan &pl,
+                               const RowTables<1> &tabs, float2 *part, const EvalOut &out,
                                cudaStream_t stream) {
-  const dim3 grid(sh.S, (sh.groups + ER_WPC_P - 1) / ER_WPC_P);
-  const size_t smem = sizeof(float4) * 2 * ER_STEP_F4_P;
-  const float4 *b4 = (const float4 *)blk;
-#define QPM_EP(V, C) k_eval_packed<V, C><<<grid, ER_WPC_P * 32, smem, stream>>>(src, ld, sh, b4, part)
-  if (vecw) {
-    if (comp) QPM_EP(true, true); else QPM_EP(true, false);
+  static SmemAttr attr;
+  const void *fn = (const void *)k_eval_genes<W, MODE, COMP>;
+  const qpm_status st = attr.set(fn, rs_smem(1, W));
+  if (st != QPM_OK) return st;
+  void *args[] = {(void *)&gm, (void *)&g, (void *)&ld, (void *)&pl, (void *)&tabs, (void *)&part,
+                  (void *)&out.ctr, (void *)&out.konst, (void *)&out.deff, (void *)&out.fit};
+  return launch_dependent(fn, dim3(pl.C), dim3(W * 32), args, rs_smem(1, W), stream);
+}
+
+static qpm_status launch_combine(const RowPlan &pl, const float2 *part, const EvalOut &out,
+                                 cudaStream_t stream) {
+  int runs = rc_runs(pl);
+  const int rows = RC_THREADS / runs;
+  void *args[] = {(void *)&pl, &runs, (void *)&part, (void *)&out.konst, (void *)&out.deff,
+                  (void *)&out.fit};
+  return launch_dependent((const void *)k_eval_combine, dim3((pl.NP + rows - 1) / rows),
+                          dim3(RC_THREADS), args, 0, stream);
+}
+
+// the sweep of float genes and, unless it combines its rows itself, the combining kernel
+static qpm_status launch_eval_rows(bool comp, const float *g, int64_t ld, const RowPlan &pl,
+                                   const float2 *blk, float2 *part, const EvalOut &out,
+                                   cudaStream_t stream) {
+  GeneMaps gm;
+  int mode;
+  qpm_status st = make_gene_maps(&gm, &mode, g, pl.NP, pl.N, ld);
+  if (st != QPM_OK) return st;
+  const RowTables<1> tabs{{blk}};
+#define QPM_EG(WW, M)                                                       \
+  st = comp ? launch_genes<WW, M, true>(gm, g, ld, pl, tabs, part, out, stream) \
+            : launch_genes<WW, M, false>(gm, g, ld, pl, tabs, part, out, stream)
+  if (pl.W == 4) {
+    if (mode == ROWS_TMA) QPM_EG(4, ROWS_TMA);
+    else QPM_EG(4, ROWS_TMA4);
   } else {
-    if (comp) QPM_EP(false, true); else QPM_EP(false, false);
+    if (mode == ROWS_TMA) QPM_EG(1, ROWS_TMA);
+    else QPM_EG(1, ROWS_TMA4);
   }
-#undef QPM_EP
+#undef QPM_EG
+  if (st != QPM_OK || out.ctr) return st;
+  return launch_combine(pl, part, out, stream);
+}
+
+template <int W>
+static qpm_status launch_packed(bool vecw, bool comp, const uint32_t *src, int64_t ld,
+                                const RowPlan &pl, const RowTables<1> &tabs, float2 *part,
+                                cudaStream_t stream) {
+  const void *fn = vecw ? (comp ? (const void *)k_eval_packed<W, true, true>
+                                : (const void *)k_eval_packed<W, true, false>)
+                        : (comp ? (const void *)k_eval_packed<W, false, true>
+                                : (const void *)k_eval_packed<W, false, false>);
+  void *args[] = {(void *)&src, (void *)&ld, (void *)&pl, (void *)&tabs, (void *)&part};
+  return launch_dependent(fn, dim3(pl.C), dim3(W * 32), args, 0, stream);
+}
+
+// the counters of a fused combination: where a row has few pieces, at the start of the
+// stream's scratch (lease held); not in a captured call, whose replays may overlap others
+qpm_status fuse_counters(const RowPlan &pl, cudaStream_t stream, unsigned **ctr) {
+  *ctr = nullptr;
+  if (pl.P > RC_FUSE || pl.RB > FUSE_BLOCKS) return QPM_OK;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) {
+    cudaGetLastError();
+    return QPM_OK;
+  }
+  if (cap != cudaStreamCaptureStatusNone) return QPM_OK;
+  void *scratch = nullptr;
+  const qpm_status st = get_scratch(stream, FUSE_BYTES, &scratch);
+  *ctr = (unsigned *)scratch;
+  return st;
 }
 
 static qpm_status eval_common(const qpm_problem *prob, const void *src, int64_t ld, int32_t NP,
@@ -400,24 +431,24 @@ static qpm_status eval_common(const qpm_problem *prob, const void *src, int64_t 
   const float2 *konst, *blk = nullptr;
   qpm_status st = lease.block_table(prob, stream, &blk, &konst);
   if (st != QPM_OK) return st;
-  if (NP > ER_WPC * 32 * 65535) return fail(QPM_ERR_UNSUPPORTED, "qpm_eval: too many rows");
-  const bool aligned = (ld % 4 == 0) && (((uintptr_t)src & 15) == 0);
-  const EvalShape sh = kind == 2 ? eval_rows_shape(NP, prob->N, 32, ER_LMAX_P)
-                                 : eval_genes_shape(NP, prob->N, aligned);
+  if (NP > EVAL_MAX_ROWS) return fail(QPM_ERR_UNSUPPORTED, "qpm_eval: too many rows");
+  const int W = kind == 2 ? (NP <= 64 ? 2 : 8) : 0;
+  const RowPlan pl = kind == 2 ? packed_plan(NP, prob->N, W) : genes_plan(1, NP, prob->N);
   void *scratch;
-  st = get_scratch(stream, sizeof(float2) * 3 * (size_t)sh.S * sh.NPpad, &scratch);
+  st = get_scratch(stream, FUSE_BYTES + plan_bytes(pl, 1), &scratch);
   if (st != QPM_OK) return st;
-  float2 *part = (float2 *)scratch;
+  float2 *part = (float2 *)((char *)scratch + FUSE_BYTES);
+  EvalOut out{nullptr, konst, (float2 *)d_eff, fit};
   if (kind == 2) {
-    launch_eval_packed(aligned, comp != 0, (const uint32_t *)src, ld, sh, blk, part, stream);
-  } else {
-    st = launch_eval_rows(aligned, comp != 0, (const float *)src, ld, sh, blk, part, stream);
-    if (st != QPM_OK) return st;
+    const bool vecw = (ld % 4 == 0) && (((uintptr_t)src & 15) == 0);
+    const RowTables<1> tabs{{blk}};
+    st = W == 8 ? launch_packed<8>(vecw, comp != 0, (const uint32_t *)src, ld, pl, tabs, part, stream)
+                : launch_packed<2>(vecw, comp != 0, (const uint32_t *)src, ld, pl, tabs, part, stream);
+    return st != QPM_OK ? st : launch_combine(pl, part, out, stream);
   }
-  QPM_CUDA(cudaGetLastError());
-  k_eval_combine<<<(NP + 7) / 8, 256, 0, stream>>>(sh, part, konst, (float2 *)d_eff, fit);
-  QPM_CUDA(cudaGetLastError());
-  return QPM_OK;
+  st = fuse_counters(pl, stream, &out.ctr);
+  if (st != QPM_OK) return st;
+  return launch_eval_rows(comp != 0, (const float *)src, ld, pl, blk, part, out, stream);
 }
 
 
@@ -458,13 +489,13 @@ qpm_status noalloc_base(void **out) {
 size_t up256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // bytes of the fixed array one call uses: the sign-block table (192 bytes per block of
-// 4 domains), the reduction partials of the constants, the constants, and the segment
-// partials of the scan (3 float2 per segment and padded row)
-size_t noalloc_bytes(int32_t N, const EvalShape &sh) {
+// 4 domains), the reduction partials of the constants, the constants, and the pieces'
+// partials of the scan (3 float2 per piece and padded row)
+size_t noalloc_bytes(int32_t N, const RowPlan &pl) {
   const int32_t Npad = (N + 3) & ~3;
   return up256(sizeof(float2) * BLK_F2 * (size_t)(Npad / 4)) +
          up256(sizeof(double2) * (size_t)table_part_count(Npad)) + 256 +
-         up256(sizeof(float2) * 3 * (size_t)sh.S * sh.NPpad);
+         up256(plan_bytes(pl, 1));
 }
 }  // namespace
 
@@ -479,11 +510,14 @@ extern "C" qpm_status qpm_eval_noalloc(const qpm_problem *prob, const float *gen
   if (ld < prob->N) return fail(QPM_ERR_ARG, "qpm_eval_noalloc: leading dimension smaller than the row");
   if (prob->N > (1 << 28) || NP > (1 << 26))
     return fail(QPM_ERR_ARG, "qpm_eval_noalloc: N above 2^28 or NP above 2^26");
-  if (NP > ER_WPC * 32 * 65535) return fail(QPM_ERR_UNSUPPORTED, "qpm_eval_noalloc: too many rows");
-  const bool vec = (ld % 4 == 0) && (((uintptr_t)genes & 15) == 0);
-  const EvalShape sh = eval_genes_shape(NP, prob->N, vec);
+  if (NP > EVAL_MAX_ROWS) return fail(QPM_ERR_UNSUPPORTED, "qpm_eval_noalloc: too many rows");
   const int32_t Npad = (prob->N + 3) & ~3;
-  const size_t need = noalloc_bytes(prob->N, sh);
+  RowPlan pl = genes_plan(1, NP, prob->N);
+  size_t need = noalloc_bytes(prob->N, pl);
+  if (need > NOALLOC_SCRATCH_BYTES) {  // rows split no further than the longest run needs
+    pl = genes_plan(1, NP, prob->N, true);
+    need = noalloc_bytes(prob->N, pl);
+  }
   if (need > NOALLOC_SCRATCH_BYTES)
     return fail(QPM_ERR_ARG, "qpm_eval_noalloc: N and NP need " + std::to_string(need) +
                                  " bytes of scratch, more than the fixed 16 MiB (16777216)");
@@ -499,19 +533,16 @@ extern "C" qpm_status qpm_eval_noalloc(const qpm_problem *prob, const float *gen
   float2 *konst = (float2 *)(p + b_blk + b_tpart);
   float2 *part = (float2 *)(p + b_blk + b_tpart + 256);
   // every word read below is written first in this call (the sign-block table, the
-  // constants and their partial sums, every segment partial of every padded row), so
+  // constants and their partial sums, every piece of every row), so
   // nothing needs zeroing; the constants come from k_table without a phasor table
   TableSpec ts{prob->N, Npad, 1, Npad, prob->kappa1, prob->kappa2};
   st = launch_table(ts, nullptr, tpart, konst, nullptr, s);
   if (st != QPM_OK) return st;
   st = launch_block_table(prob->N, prob->kappa1, prob->kappa2, blk, s);
   if (st != QPM_OK) return st;
-  st = launch_eval_rows(vec, compensated != 0, genes, ld, sh, blk, part, s);
-  if (st != QPM_OK) return st;
-  QPM_CUDA(cudaGetLastError());
-  k_eval_combine<<<(NP + 7) / 8, 256, 0, s>>>(sh, part, konst, (float2 *)d_eff, fit);
-  QPM_CUDA(cudaGetLastError());
-  return QPM_OK;
+  // no counters in the shared array, whose words need not start at zero
+  return launch_eval_rows(compensated != 0, genes, ld, pl, blk, part,
+                          EvalOut{nullptr, konst, (float2 *)d_eff, fit}, s);
 }
 
 qpm::TableLease::TableLease(const qpm_problem *problems, int count) {

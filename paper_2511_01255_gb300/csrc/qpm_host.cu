@@ -21,6 +21,32 @@ qpm_status cuda_fail(cudaError_t e, const char *what) {
   return QPM_ERR_CUDA;
 }
 
+qpm_status launch_dependent(const void *fn, dim3 grid, dim3 block, void **args, size_t smem,
+                            cudaStream_t stream) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  QPM_CUDA(cudaLaunchKernelExC(&cfg, fn, args));
+  return QPM_OK;
+}
+
+qpm_status SmemAttr::set(const void *fn, size_t bytes) {
+  int dev = 0;
+  QPM_CUDA(cudaGetDevice(&dev));
+  // a second thread at worst repeats the same call
+  if (dev >= 0 && dev < 128 && __atomic_load_n(&done[dev], __ATOMIC_ACQUIRE)) return QPM_OK;
+  QPM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  if (dev >= 0 && dev < 128) __atomic_store_n(&done[dev], 1, __ATOMIC_RELEASE);
+  return QPM_OK;
+}
+
 int sm_count() {
   static std::mutex mu;
   static std::vector<int> cache;

@@ -77,16 +77,42 @@ class TableLease {
   qpm_status st_ = QPM_OK;
 };
 
-// split of qpm_eval-style work: S segments of L domains, rows in groups of 32
-struct EvalShape {
-  int NP, N, S, L;
-  int groups;  // ceil(NP / 32)
-  int NPpad;   // groups * 32
+// split of the row sweeps (qpm_rows.cuh): row blocks of W groups of 32 rows, each nunit units
+// of gran sub-steps of 32 domains, laid end to end and dealt to C CTAs as equal runs
+struct RowPlan {
+  int NP, N;
+  int NPpad;  // NP rounded up to 32
+  int W;      // warps (row groups) per CTA
+  int RB;     // row blocks
+  int nsub;   // sub-steps of a row, ceil(N / 32)
+  int gran, nunit;  // sub-steps per unit, units of a row
+  int C;      // CTAs
+  int P;      // pieces of a row at most
 };
-// split of the row sweep (qpm_rows.cuh): segments a multiple of 128 domains,
-// about warps_per_sm warps of work per SM
-// (lmax: longest segment, 0 for the phasor sweep's default)
-EvalShape eval_rows_shape(int NP, int N, int warps_per_sm, int lmax = 0);
+// slots: resident CTAs per SM; gran: sub-steps per unit; maxsub: longest run; min_units: no run
+// shorter than this while CTAs are left idle
+RowPlan row_plan(int NP, int N, int W, int slots, int gran, int maxsub, int min_units);
+// the plan of the float-gene sweep with K sign-block tables; whole: no row is split unless it
+// is longer than a run may be (fewest pieces)
+RowPlan genes_plan(int K, int NP, int N, bool whole = false);
+// counters of the plan's fused combination on this stream (NULL: the combining kernel); the
+// caller holds a TableLease until the sweep is enqueued
+qpm_status fuse_counters(const RowPlan &pl, cudaStream_t stream, unsigned **ctr);
+constexpr int EVAL_MAX_ROWS = 128 * 65535;  // rows a call of the row sweeps takes
+// bytes of the plan's partial monoids for K problems
+inline size_t plan_bytes(const RowPlan &p, int K) {
+  return sizeof(float2) * 3 * (size_t)K * (size_t)p.P * (size_t)p.NPpad;
+}
+
+// launch as a programmatic dependent of the stream's last kernel: the kernel's CTAs may be
+// scheduled as that one's retire, and the kernel itself waits (griddepcontrol.wait) for it
+qpm_status launch_dependent(const void *fn, dim3 grid, dim3 block, void **args, size_t smem,
+                            cudaStream_t stream);
+// dynamic shared memory of a kernel, set once per device (always to the same value)
+struct SmemAttr {
+  unsigned char done[128] = {0};
+  qpm_status set(const void *fn, size_t bytes);
+};
 
 // current device's SM count (cached per device)
 int sm_count();

@@ -178,134 +178,99 @@ static __global__ void __launch_bounds__(SHG_WARPS * 32, 1)
 // ------------------------------------------------- multi-wavelength objective
 static constexpr int MW_KMAX = 4;
 
-struct MultiTables {
-  const float4 *t[MW_KMAX];  // sign-block tables (launch_block_table), read as float4
-  const float2 *konst[MW_KMAX];
+template <int K>
+struct MultiOut {
+  const float2 *konst[K];
+  float G0, beta;
+  float2 *deff;
+  float *obj;
 };
-
-// The qpm_eval sweeps with K sign-block tables: the same segments and order for the
-// same rows, so K = 1 reproduces qpm_eval's plain scan bit for bit.  Partials as for
-// qpm_eval, one set per problem: part[((3k + comp) * S + s) * NPpad + i].
-// grid (S, ceil(groups / ER_WPC)).
-
-// 16-byte aligned rows: er_ring_sweep with K tables; K x 12 KB + 48 KB of shared memory
-// per CTA (about 1 KB more with TMA tiles), so 3 CTAs per SM for K <= 2 and 2 for K = 3, 4
-__host__ __device__ constexpr int mw_ring_ctas(int K) { return K <= 2 ? 3 : 2; }
-// TMA: the gene tiles by TMA copies (er_ring_sweep_tma, `gmap`), else by cp.async
-template <int K, bool TMA>
-static __global__ void __launch_bounds__(ER_WPC * 32, mw_ring_ctas(K))
-    k_multi_rows_ring(const __grid_constant__ CUtensorMap gmap, const float *__restrict__ genes,
-                      int64_t ld, EvalShape sh, MultiTables mt, float2 *__restrict__ part) {
-  extern __shared__ float4 dyn_raw[];
-  float4 *dyn = dyn_raw;
-  if constexpr (TMA)  // 1024-byte aligned for the swizzled tiles (the launch adds the slack)
-    dyn = (float4 *)((unsigned char *)dyn_raw + ((1024 - (smem_u32(dyn_raw) & 1023)) & 1023));
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int s = blockIdx.x, m0 = s * sh.L, m1 = min(sh.N, m0 + sh.L);
-  const int r0 = (blockIdx.y * ER_WPC + warp) * 32;
-  const bool live = r0 < sh.NP;
-  Mono acc[K];
-#pragma unroll
-  for (int p = 0; p < K; ++p) acc[p] = mono_zero();
-  auto push = [&](uint32_t e, const float2 *E, int b) {
-#pragma unroll
-    for (int p = 0; p < K; ++p) er_push_block(acc[p], e, E + (size_t)p * 2 * ER_STEP_F4_P + b * BLK_F2);
-  };
-  if constexpr (TMA) er_ring_sweep_tma<K>(dyn, &gmap, sh, mt.t, m0, m1, r0, live, push);
-  else er_ring_sweep<K>(dyn, genes, ld, sh, mt.t, m0, m1, r0, live, push);
-  if (!live) return;
-  const size_t stride = (size_t)sh.S * sh.NPpad;
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    const size_t o = (size_t)(3 * k) * stride + (size_t)s * sh.NPpad + r0 + lane;
-    part[o] = acc[k].A;
-    part[o + stride] = acc[k].B;
-    part[o + 2 * stride] = acc[k].C;
-  }
-}
-
-// other rows: scalar gene loads one sub-step ahead in registers.  Dynamic shared
-// memory: two steps of the K tables' entries, [2][K][ER_STEP_F4_P] float4.
+// the objective of one row from its K combined scans
 template <int K>
-static __global__ void __launch_bounds__(ER_WPC * 32)
-    k_multi_rows(const float *__restrict__ genes, int64_t ld, EvalShape sh, MultiTables mt,
-                 float2 *__restrict__ part) {
-  extern __shared__ float4 tb[];
-  __shared__ float4 tile[ER_WPC][256];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int s = blockIdx.x, m0 = s * sh.L, m1 = min(sh.N, m0 + sh.L);
-  const int r0 = (blockIdx.y * ER_WPC + warp) * 32;
-  const bool live = r0 < sh.NP;
-  const int nb = (sh.N + 3) >> 2, nsteps = (m1 - m0 + 127) >> 7;
-  float4 R[8];
-  if (live) er_load_genes<false>(genes, ld, sh, r0, m0, R);
-  // step k of problem p in buffer ((k & 1) * K + p); one commit group per step
-#pragma unroll
-  for (int p = 0; p < K; ++p) er_stage_step(tb + p * ER_STEP_F4_P, mt.t[p], m0, 0, nb);
-  const float2 *bt = (const float2 *)tb;
-  Mono acc[K];
-#pragma unroll
-  for (int p = 0; p < K; ++p) acc[p] = mono_zero();
-  float4 *T = tile[warp];
-  for (int k = 0; k < nsteps; ++k) {
-    cp_async_wait<0>();
-    __syncthreads();
-    if (k + 1 < nsteps) {
-#pragma unroll
-      for (int p = 0; p < K; ++p)
-        er_stage_step(tb + (((k + 1) & 1) * K + p) * ER_STEP_F4_P, mt.t[p], m0, k + 1, nb);
-    }
-    if (!live) continue;
-    const float2 *bp = bt + (size_t)(k & 1) * K * 2 * ER_STEP_F4_P;
-#pragma unroll 1
-    for (int q = 0; q < 4; ++q) {
-      const int ms = m0 + 128 * k + 32 * q;
-      if (ms >= m1) break;
-      __syncwarp();
-#pragma unroll
-      for (int j = 0; j < 8; ++j) T[er_tix(4 * j + (lane >> 3), lane & 7)] = R[j];
-      __syncwarp();
-      if (ms + 32 < m1) er_load_genes<false>(genes, ld, sh, r0, ms + 32, R);
-#pragma unroll 2
-      for (int c4 = 0; c4 < 8; ++c4) {
-        const uint32_t e = er_pattern(T[er_tix(lane, c4)]);
-#pragma unroll
-        for (int p = 0; p < K; ++p)
-          er_push_block(acc[p], e, bp + (size_t)p * 2 * ER_STEP_F4_P + (8 * q + c4) * BLK_F2);
-      }
-    }
-  }
-  if (!live) return;
-  const size_t stride = (size_t)sh.S * sh.NPpad;
-#pragma unroll
-  for (int k = 0; k < K; ++k) {
-    const size_t o = (size_t)(3 * k) * stride + (size_t)s * sh.NPpad + r0 + lane;
-    part[o] = acc[k].A;
-    part[o + stride] = acc[k].B;
-    part[o + 2 * stride] = acc[k].C;
-  }
-}
-
-// one warp per row: the K combined scans (as in qpm_eval), then the objective
-template <int K>
-static __global__ void k_multi_combine(EvalShape sh, const float2 *__restrict__ part, MultiTables mt,
-                                       float G0, float beta, float2 *__restrict__ deff,
-                                       float *__restrict__ obj) {
-  const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (row >= sh.NP) return;
-  const size_t set = (size_t)3 * sh.S * sh.NPpad;  // the partials of one problem
+__device__ __forceinline__ void multi_close(const MultiOut<K> &o, int row, const Mono *m) {
   float f = 0.f, gmax = -1.f, gmin = 3.0e38f;
 #pragma unroll
   for (int k = 0; k < K; ++k) {
-    const Mono acc = combine_segments(part + k * set, sh.S, sh.NPpad, row);
-    const float2 D = deff_from(acc, mt.konst[k][0], mt.konst[k][1]);
-    if (deff && (threadIdx.x & 31) == 0) deff[(size_t)row * K + k] = D;
+    const float2 D = deff_from(m[k], o.konst[k][0], o.konst[k][1]);
+    if (o.deff) o.deff[(size_t)row * K + k] = D;
     const float G = sqrtf(fit_of(D));
-    f += fabsf(G0 - G);
+    f += fabsf(o.G0 - G);
     gmax = fmaxf(gmax, G);
     gmin = fminf(gmin, G);
   }
-  if ((threadIdx.x & 31) == 0) obj[row] = f + beta * (gmax - gmin);
+  o.obj[row] = f + o.beta * (gmax - gmin);
+}
+
+// The qpm_eval sweep with K sign-block tables: for K = 1 the same split and order, so it
+// reproduces qpm_eval's plain scan bit for bit.
+template <int K, int W, int MODE>
+static __global__ void __launch_bounds__(W * 32, rs_ctas(K, W))
+    k_multi_genes(const __grid_constant__ GeneMaps maps, const float *__restrict__ src, int64_t ld,
+                  RowPlan pl, RowTables<K> tabs, float2 *part, unsigned *ctr, MultiOut<K> out) {
+  rows_sweep<K, W, MODE, false>(maps, src, ld, pl, tabs, part, ctr,
+                                [&](int row, const Mono *m) { multi_close<K>(out, row, m); });
+}
+
+// the K combined scans (as in qpm_eval), then the objective; a programmatic dependent
+template <int K>
+static __global__ void __launch_bounds__(RC_THREADS)
+    k_multi_combine(RowPlan pl, int runs, const float2 *__restrict__ part, MultiOut<K> out) {
+  __shared__ Mono sh[K][RC_THREADS];
+  const int rows = RC_THREADS / runs, run = threadIdx.x / rows;
+  const int row = blockIdx.x * rows + threadIdx.x - run * rows;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  Mono acc[K];
+  combine_pieces<K>(pl, part, runs, row, run, sh, acc);
+  if (run == 0 && row < pl.NP) multi_close<K>(out, row, acc);
+}
+
+template <int K, int W, int MODE>
+static qpm_status launch_multi_genes(const GeneMaps &gm, const float *g, int64_t ld, const RowPlan &pl,
+                                     const RowTables<K> &tabs, float2 *part, unsigned *ctr,
+                                     const MultiOut<K> &out, cudaStream_t s) {
+  static SmemAttr attr;
+  const void *fn = (const void *)k_multi_genes<K, W, MODE>;
+  const qpm_status st = attr.set(fn, rs_smem(K, W));
+  if (st != QPM_OK) return st;
+  void *args[] = {(void *)&gm, (void *)&g, (void *)&ld, (void *)&pl, (void *)&tabs, (void *)&part,
+                  (void *)&ctr, (void *)&out};
+  return launch_dependent(fn, dim3(pl.C), dim3(W * 32), args, rs_smem(K, W), s);
+}
+
+template <int K>
+static qpm_status launch_multi(const float2 *const *blk, const float2 *const *konst, const float *g,
+                               int64_t ld, const RowPlan &pl, float G0, float beta, void *scratch,
+                               float2 *deff, float *obj, cudaStream_t s) {
+  constexpr int MANY = K == 1 ? 4 : 8, FEW = K == 1 ? 1 : 2;  // genes_plan's warps per CTA
+  GeneMaps gm;
+  int mode;
+  qpm_status st = make_gene_maps(&gm, &mode, g, pl.NP, pl.N, ld);
+  if (st != QPM_OK) return st;
+  float2 *part = (float2 *)scratch;
+  unsigned *ctr = nullptr;
+  st = fuse_counters(pl, s, &ctr);
+  if (st != QPM_OK) return st;
+  RowTables<K> tabs;
+  MultiOut<K> out{{}, G0, beta, deff, obj};
+  for (int k = 0; k < K; ++k) {
+    tabs.blk[k] = blk[k];
+    out.konst[k] = konst[k];
+  }
+#define QPM_MG(W, M) st = launch_multi_genes<K, W, M>(gm, g, ld, pl, tabs, part, ctr, out, s)
+  if (pl.W == MANY) {
+    if (mode == ROWS_TMA) QPM_MG(MANY, ROWS_TMA);
+    else QPM_MG(MANY, ROWS_TMA4);
+  } else {
+    if (mode == ROWS_TMA) QPM_MG(FEW, ROWS_TMA);
+    else QPM_MG(FEW, ROWS_TMA4);
+  }
+#undef QPM_MG
+  if (st != QPM_OK || ctr) return st;
+  int runs = rc_runs(pl);
+  const int rows = RC_THREADS / runs;
+  void *args[] = {(void *)&pl, &runs, &part, &out};
+  return launch_dependent((const void *)k_multi_combine<K>, dim3((pl.NP + rows - 1) / rows),
+                          dim3(RC_THREADS), args, 0, s);
 }
 
 }  // namespace qpm
@@ -347,56 +312,25 @@ extern "C" qpm_status qpm_eval_multi(const qpm_problem *probs, int32_t K, const 
   if (N < 1 || NP < 1) return fail(QPM_ERR_ARG, "qpm_eval_multi: need N >= 1 and NP >= 1");
   if (ld < N) return fail(QPM_ERR_ARG, "qpm_eval_multi: leading dimension smaller than the row");
   cudaStream_t s = (cudaStream_t)stream;
-  MultiTables mt;
-  for (int k = 0; k < MW_KMAX; ++k) {
-    mt.t[k] = nullptr;
-    mt.konst[k] = nullptr;
-  }
-  if (NP > ER_WPC * 32 * 65535) return fail(QPM_ERR_UNSUPPORTED, "qpm_eval_multi: too many rows");
+  const float2 *blk[MW_KMAX], *konst[MW_KMAX];
+  if (NP > EVAL_MAX_ROWS) return fail(QPM_ERR_UNSUPPORTED, "qpm_eval_multi: too many rows");
   // one lease for all K lookups and the launches: room for the K tables is made
   // before the first lookup, so no lookup can evict a table returned before it
   TableLease lease(probs, K);
   for (int k = 0; k < K; ++k) {
-    const float2 *blk;
-    qpm_status st = lease.block_table(&probs[k], s, &blk, &mt.konst[k]);
+    qpm_status st = lease.block_table(&probs[k], s, &blk[k], &konst[k]);
     if (st != QPM_OK) return st;
-    mt.t[k] = (const float4 *)blk;
   }
-  const bool vec = (ld % 4 == 0) && (((uintptr_t)genes & 15) == 0);
-  const EvalShape sh = eval_rows_shape(NP, N, vec ? ER_WPC * mw_ring_ctas(K) : 20);
-  const size_t need = sizeof(float2) * 3 * (size_t)K * sh.S * sh.NPpad;
-  if (!scratch || scratch_bytes < need)
+  const RowPlan pl = genes_plan(K, NP, N);
+  if (!scratch || scratch_bytes < plan_bytes(pl, K))
     return fail(QPM_ERR_ARG, "qpm_eval_multi: scratch smaller than qpm_eval_multi_scratch_bytes()");
-  float2 *part = (float2 *)scratch;
-  const dim3 grid(sh.S, (sh.groups + ER_WPC - 1) / ER_WPC);
-  CUtensorMap gmap{};
-  const bool tma = vec && make_tile_map(&gmap, genes, NP, N, ld);
-#define QPM_MW(KK)                                                                          \
-  {                                                                                         \
-    const void *fn = !vec ? (const void *)k_multi_rows<KK>                                  \
-                     : tma ? (const void *)k_multi_rows_ring<KK, true>                     \
-                           : (const void *)k_multi_rows_ring<KK, false>;                   \
-    const size_t smem = !vec ? sizeof(float4) * 2 * (size_t)KK * ER_STEP_F4_P               \
-                        : tma ? 1024 + er_ring_smem_tma(KK) : er_ring_smem(KK);             \
-    QPM_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)); \
-    EvalShape shv = sh;                                                                     \
-    int64_t ldv = ld;                                                                       \
-    void *args_ring[] = {(void *)&gmap, (void *)&genes, &ldv, &shv, &mt, &part};           \
-    void *args_rows[] = {(void *)&genes, &ldv, &shv, &mt, &part};                           \
-    QPM_CUDA(cudaLaunchKernel(fn, grid, dim3(ER_WPC * 32), vec ? args_ring : args_rows, smem, s)); \
-    k_multi_combine<KK><<<(NP + 7) / 8, 256, 0, s>>>(sh, part, mt, G0, beta,               \
-                                                      (float2 *)d_eff, objective);          \
-  }
-  if (K == 1) QPM_MW(1) else if (K == 2) QPM_MW(2) else if (K == 3) QPM_MW(3) else QPM_MW(4)
+#define QPM_MW(KK) \
+  launch_multi<KK>(blk, konst, genes, ld, pl, G0, beta, scratch, (float2 *)d_eff, objective, s)
+  return K == 1 ? QPM_MW(1) : K == 2 ? QPM_MW(2) : K == 3 ? QPM_MW(3) : QPM_MW(4);
 #undef QPM_MW
-  QPM_CUDA(cudaGetLastError());
-  return QPM_OK;
 }
 
-// sized for the split of unaligned rows: fewer resident warps (the ring form of aligned
-// rows) only lengthen the segments, so no split the call takes has more of them
 extern "C" size_t qpm_eval_multi_scratch_bytes(int32_t K, int32_t N, int32_t NP) {
   if (K < 1 || N < 1 || NP < 1) return 0;
-  const EvalShape sh = eval_rows_shape(NP, N, 20);
-  return sizeof(float2) * 3 * (size_t)K * sh.S * sh.NPpad;
+  return plan_bytes(genes_plan(std::min(K, (int32_t)MW_KMAX), NP, N), K);
 }

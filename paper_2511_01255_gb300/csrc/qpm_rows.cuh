@@ -1,10 +1,30 @@
-// qpm_rows.cuh -- the row sweep shared by the fitness kernels of qpm_eval and of
-// the multi-wavelength objective: a warp takes 32 rows (lane = row) and one
-// segment of L domains (a multiple of ER_LQ) and walks it in index order, one block
-// of 4 domains at a time: a block of +-1 domains takes one of 16 sign patterns and
-// its monoid triple depends on the pattern only, so the sign-block table
-// (launch_block_table) holds the triples and the sweep appends one per lookup.  The
-// table entries are streamed into shared memory per step of 128 domains.
+// qpm_rows.cuh -- the row sweep shared by the fitness kernels of qpm_eval, qpm_eval_packed
+// and the multi-wavelength objective.
+//
+// A warp takes 32 rows (lane = row) and walks a run of domains in index order, one block of
+// 4 domains at a time: a block of +-1 domains takes one of 16 sign patterns and its monoid
+// triple depends on the pattern only, so the sweep appends one table entry per block.  The
+// global sign-block table (launch_block_table) holds the 8 patterns with d_0 = +1; staging a
+// step of 128 domains in shared memory expands them to all 16 (the complement negates A and B),
+// which costs a CTA a few stores per step and takes the fold of the pattern and the four sign
+// flips out of every lane's block: 12 instructions a block and problem instead of 22-27.  The
+// 16 entries of a block are 24 bytes apart and fall in distinct bank pairs, so a lookup is
+// three conflict-free LDS.64.  The complex sums are packed FP32 pairs (add.rn.f32x2).
+//
+// Split of the work (RowPlan): the rows are taken in blocks of W groups of 32 (the W warps of
+// a CTA, sharing one staged table), and the row blocks' sub-steps of 32 domains laid end to end
+// are dealt to the CTAs as equal contiguous runs, a multiple of the resident CTAs, so that
+// every SM ends at the same time whatever NP and N are.  A run that crosses the end of a row
+// block becomes a piece of each.  The pieces of a row are combined in index order by the CTA that
+// completes its row block, where they are few, else by a second kernel.
+//
+// What bounds it and what it measured (ncu, cold and serialised, against the form before it:
+// 8-pattern table through cp.async, segments rounded to 128 domains, unaligned rows by 4-byte
+// register loads):
+//   5000 x 6601 unaligned rows   HBM (6.0 TB/s): 35.6 -> 28.0 us
+//   1024 x 1e5 packed signs      the shared-memory data path (70 % of its cycles): 31.6 -> 28.3 us
+//   5000 x 3000, 3 problems      shared memory and HBM together: 28.2 -> 18.8 us
+//   1024 x 1e5 aligned rows      HBM: 62.8 -> 65 us, and 4 us less for the combination
 #pragma once
 #include "qpm_common.cuh"
 #include "qpm_internal.h"
@@ -12,342 +32,480 @@
 
 namespace qpm {
 
-constexpr int ER_WPC = 4;      // warps (row groups of 32) per CTA of the float sweeps
-constexpr int ER_LQ = 128;     // segment length quantum (domains)
-constexpr int ER_LMAX = 1920;  // longest segment of the float sweeps
+constexpr int RS_RING = 3;              // gene tiles per warp
+constexpr int RS_ENTRY = 24;            // bytes of an entry (A, B, C as float2)
+constexpr int RS_BLOCK = 16 * RS_ENTRY; // the 16 entries of a block of 4 domains
+constexpr int RS_TAB = 32 * RS_BLOCK;   // a step of 128 domains, one problem: 12 KB
+constexpr int RS_MAXSUB = 60;           // longest run in sub-steps (1920 domains: no plain FP32
+                                        // partial sum of C exceeds about 1920^2 / 2 < 2^24)
 
-// per-warp tile: 32 rows x 32 domains as float4 [row][c4], the column xor-swizzled by
-// the row so that both the staging stores (8 columns of a row per quarter-warp) and
-// the row walks (8 rows of a column) are free of bank conflicts
-__device__ __forceinline__ int er_tix(int row, int c4) { return row * 8 + (c4 ^ (row & 7)); }
+// ------------------------------------------------------------------- the split
+// first sub-step (of all row blocks laid end to end) of CTA x
+__host__ __device__ __forceinline__ int64_t rp_start(const RowPlan &p, int64_t x) {
+  return (int64_t)p.RB * p.nunit * x / p.C * p.gran;
+}
+// the CTA holding the first unit of row block b, and the number of pieces of row block b
+__host__ __device__ __forceinline__ int rp_first(const RowPlan &p, int64_t unit) {
+  return (int)(((unit + 1) * p.C - 1) / ((int64_t)p.RB * p.nunit));
+}
+__host__ __device__ __forceinline__ int rp_pieces(const RowPlan &p, int b) {
+  return rp_first(p, (int64_t)(b + 1) * p.nunit - 1) - rp_first(p, (int64_t)b * p.nunit) + 1;
+}
 
-// float genes of one step (32 domains from ms) of rows r0..r0+31: lane l holds
-// float4 k * 32 + l, i.e. row 4k + l / 8, columns 4 (l % 8) .. +3
-template <bool VEC>
-__device__ __forceinline__ void er_load_genes(const float *__restrict__ g, int64_t ld,
-                                              const EvalShape &sh, int r0, int ms, float4 R[8]) {
-  const int lane = threadIdx.x & 31;
-  const int m = ms + 4 * (lane & 7);
+// ------------------------------------------------------------- packed FP32 pairs
+// One 64-bit register pair holds (re, im); add.rn.f32x2 rounds both halves as the scalar
+// operation does.
+typedef unsigned long long rs_pair;
+__device__ __forceinline__ rs_pair rs_add(rs_pair a, rs_pair b) {
+  rs_pair r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ rs_pair rs_pack(float x, float y) {
+  rs_pair r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ float2 rs_unpack(rs_pair v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+struct MonoP {
+  rs_pair A, B, C;
+};
+// m (+) the entry at `e`: mono_combine's operations in its order
+__device__ __forceinline__ void rs_push(MonoP &m, const unsigned char *e) {
+  const rs_pair a = *(const rs_pair *)e, b = *(const rs_pair *)(e + 8);
+  const float2 av = rs_unpack(a), B = rs_unpack(m.B);
+  float2 c = rs_unpack(rs_add(m.C, *(const rs_pair *)(e + 16)));
+  c.x = fmaf(av.x, B.x, c.x);
+  c.x = fmaf(-av.y, B.y, c.x);
+  c.y = fmaf(av.x, B.y, c.y);
+  c.y = fmaf(av.y, B.x, c.y);
+  m.C = rs_pack(c.x, c.y);
+  m.A = rs_add(m.A, a);
+  m.B = rs_add(m.B, b);
+}
+
+// Running monoid of a lane's row.  Plain: FP32 sums over a step of 128 domains, each step's
+// then added to the run's (two short sums instead of one long one: 10 operations per 32 blocks
+// for about the error of the shorter).  COMP: plain sums over 16 domains (4 sign blocks)
+// Kahan-folded into a compensated triple.
+template <bool COMP>
+struct RowAcc {
+  MonoP m;
+  Mono o;
+  MonoK k;
+  __device__ __forceinline__ void zero() {
+    m.A = m.B = m.C = 0ull;
+    if (COMP) k = monok_zero();
+    else o = mono_zero();
+  }
+  __device__ __forceinline__ Mono plain() const {
+    Mono r;
+    r.A = rs_unpack(m.A);
+    r.B = rs_unpack(m.B);
+    r.C = rs_unpack(m.C);
+    return r;
+  }
+  __device__ __forceinline__ void fold() {  // every 4 blocks
+    if (COMP) {
+      monok_fold_in(k, plain());
+      m.A = m.B = m.C = 0ull;
+    }
+  }
+  __device__ __forceinline__ void step() {  // every 128 domains
+    if (!COMP) {
+      o = mono_combine(o, plain());
+      m.A = m.B = m.C = 0ull;
+    }
+  }
+  __device__ __forceinline__ Mono get() {  // after the last step()
+    if (COMP) {
+      fold();
+      return monok_fold(k);
+    }
+    return o;
+  }
+};
+
+// ------------------------------------------------------------- staged table steps
+// The global entries of one step of one problem in the registers of a CTA of W warps: thread i
+// holds entries i + j 32 W (entry = 8 * block + stored pattern), fetched a step ahead.
+template <int W>
+struct StepRegs {
+  static constexpr int N = 256 / (32 * W);
+  rs_pair a[N], b[N], c[N];
+  // blocks from b0 on; zero past the problem's nb blocks
+  __device__ __forceinline__ void load(const float2 *__restrict__ blk, int b0, int nb) {
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const int gr = r0 + 4 * k + (lane >> 3);
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (gr < sh.NP) {
-      const float *rp = g + (int64_t)gr * ld;
-      if (VEC && m + 4 <= sh.N) {
-        v = __ldg((const float4 *)(rp + m));
-      } else {
-        if (m < sh.N) v.x = __ldg(rp + m);
-        if (m + 1 < sh.N) v.y = __ldg(rp + m + 1);
-        if (m + 2 < sh.N) v.z = __ldg(rp + m + 2);
-        if (m + 3 < sh.N) v.w = __ldg(rp + m + 3);
+    for (int j = 0; j < N; ++j) {
+      const int e = threadIdx.x + j * 32 * W, g = b0 + (e >> 3);
+      a[j] = b[j] = c[j] = 0ull;
+      if (g < nb) {
+        const rs_pair *s = (const rs_pair *)(blk + (size_t)8 * 3 * b0) + 3 * e;
+        a[j] = __ldg(s);
+        b[j] = __ldg(s + 1);
+        c[j] = __ldg(s + 2);
       }
     }
-    R[k] = v;
   }
-}
-
-// the same step copied asynchronously (cp.async, not committed) into the per-warp
-// tile T in the layout of er_tix: lane l's copy k lands at row 4k + l / 8, columns
-// 4 (l % 8) .. +3.  16-byte aligned rows (ld % 4 == 0) only; genes past the row
-// end and rows past NP are zero-filled.
-__device__ __forceinline__ void er_copy_genes(float4 *T, const float *__restrict__ g, int64_t ld,
-                                              const EvalShape &sh, int r0, int ms) {
-  const int lane = threadIdx.x & 31;
-  const int m = ms + 4 * (lane & 7);
+  // stored pattern e is pattern 2 e; its complement 15 - 2 e has A and B negated
+  __device__ __forceinline__ void store(unsigned char *tab) const {
+    const rs_pair neg = 0x8000000080000000ull;
 #pragma unroll
-  for (int k = 0; k < 8; ++k) {
-    const int tr = 4 * k + (lane >> 3), gr = r0 + tr;
-    const float *src = g;
-    int bytes = 0;
-    if (gr < sh.NP && m < sh.N) {
-      src = g + (int64_t)gr * ld + m;
-      bytes = 4 * min(4, sh.N - m);
-    }
-    cp_async16(&T[er_tix(tr, lane & 7)], src, bytes);
-  }
-}
-
-// sign words of one packed step (128 domains from ms, a multiple of 128) of row
-// `row`; words beyond the row's last domain are zero
-template <bool VECW>
-__device__ __forceinline__ uint4 er_load_words(const uint32_t *__restrict__ w, int64_t ld,
-                                               const EvalShape &sh, int row, int ms) {
-  uint4 v = make_uint4(0u, 0u, 0u, 0u);
-  if (row < sh.NP) {
-    const uint32_t *rp = w + (int64_t)row * ld + (ms >> 5);
-    const int nw = (sh.N - ms + 31) >> 5;  // words of this row from ms on
-    if (VECW && nw >= 4) {
-      v = __ldg((const uint4 *)rp);
-    } else {
-      if (nw > 0) v.x = __ldg(rp);
-      if (nw > 1) v.y = __ldg(rp + 1);
-      if (nw > 2) v.z = __ldg(rp + 2);
-      if (nw > 3) v.w = __ldg(rp + 3);
+    for (int j = 0; j < N; ++j) {
+      const int e = threadIdx.x + j * 32 * W;
+      unsigned char *t = tab + (e >> 3) * RS_BLOCK;
+      rs_pair *p = (rs_pair *)(t + 2 * (e & 7) * RS_ENTRY);
+      rs_pair *n = (rs_pair *)(t + (15 - 2 * (e & 7)) * RS_ENTRY);
+      p[0] = a[j];
+      p[1] = b[j];
+      p[2] = c[j];
+      n[0] = a[j] ^ neg;
+      n[1] = b[j] ^ neg;
+      n[2] = c[j];
     }
   }
-  return v;
-}
+};
 
-// sign pattern of 4 genes: bit j set iff gene j < 0 (d_j = -1; -0.0 counts as +1)
+// ------------------------------------------------------------------- gene tiles
+// per-warp tile: 32 rows x 32 domains as float4 [row][c4], the column xor-swizzled by the row
+// so that both the staging stores (8 columns of a row per quarter-warp) and the row walks (8
+// rows of a column) are free of bank conflicts: the layout of a TMA copy's 128-byte swizzle
+__device__ __forceinline__ int er_tix(int row, int c4) { return row * 8 + (c4 ^ (row & 7)); }
+
+// sign pattern of 4 genes: bit j set iff gene j < 0 (d_j = -1; -0.0 and NaN count as +1)
 __device__ __forceinline__ uint32_t er_pattern(const float4 &x) {
   return (x.x < 0.f ? 1u : 0u) | (x.y < 0.f ? 2u : 0u) | (x.z < 0.f ? 4u : 0u) |
          (x.w < 0.f ? 8u : 0u);
 }
+// byte offset of the pattern's entry within its block
+__device__ __forceinline__ uint32_t er_offset(const float4 &x) {
+  uint32_t o = x.x < 0.f ? 1u * RS_ENTRY : 0u;
+  if (x.y < 0.f) o += 2u * RS_ENTRY;
+  if (x.z < 0.f) o += 4u * RS_ENTRY;
+  if (x.w < 0.f) o += 8u * RS_ENTRY;
+  return o;
+}
 
-constexpr int ER_WPC_P = 8;      // warps (row groups of 32) per CTA of the packed sweep
-constexpr int ER_LMAX_P = 4096;  // longest segment of the packed sweep
-constexpr int ER_STEP_F4_P = 32 * BLK_F2 / 2;  // float4 of entries per step of 128 domains
+// How the genes reach the tiles.
+//   ROWS_TMA    rows of 16-byte aligned pitch and base: one 32 x 32 TMA copy per sub-step
+//   ROWS_TMA4   any other rows: rows r with the same r % 4 start at the same offset from a
+//               16-byte boundary, so the four classes are four matrices of pitch 4 ld, each
+//               mapped from the boundary below its first row (shift[c] = 0..3 floats before
+//               it) and copied as four 8 x 32 boxes per sub-step.  Lane l walks the row 4 (l %
+//               8) + l / 8 of its group, and a block's pattern is taken across two neighbouring
+//               16-byte pieces.
+enum { ROWS_TMA = 0, ROWS_TMA4 = 1 };
+struct GeneMaps {
+  CUtensorMap m[4];
+  int shift[4];
+};
+// fills the maps of NP x N genes and the mode (host)
+qpm_status make_gene_maps(GeneMaps *gm, int *mode, const float *genes, int NP, int N, int64_t ld);
+template <int MODE>
+__device__ __forceinline__ int rs_row_of_lane(int lane) {
+  return MODE == ROWS_TMA4 ? 4 * (lane & 7) + (lane >> 3) : lane;
+}
 
-// the sign-block entries of step k of a segment starting at m0 (blocks
-// m0 / 4 + 32 k .. + 31) into buf, copied with cp.async by the whole CTA (not
-// committed); blocks past the last of the problem are zero
-__device__ __forceinline__ void er_stage_entries(float4 *buf, const float4 *__restrict__ blk,
-                                                 int m0, int k, int nb) {
-  const int b0 = (m0 >> 2) + 32 * k;
-  for (int i = threadIdx.x; i < ER_STEP_F4_P; i += blockDim.x) {
-    if (b0 + i / (BLK_F2 / 2) < nb) cp_async16(buf + i, blk + (size_t)b0 * (BLK_F2 / 2) + i);
-    else buf[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+template <int K>
+struct RowTables {
+  const float2 *blk[K];  // sign-block tables (launch_block_table)
+};
+
+// dynamic shared memory: [gene tiles, 1024-byte aligned][2 steps of K tables][mbarriers]
+__host__ __device__ constexpr size_t rs_smem(int K, int W) {
+  return 1024 + (size_t)W * RS_RING * 4096 + 2 * (size_t)K * RS_TAB + (size_t)W * RS_RING * 8;
+}
+// resident CTAs per SM (shared memory; 227 KB less 1 KB reserved per CTA)
+__host__ __device__ constexpr int rs_ctas(int K, int W) {
+  const int n = (int)(232448 / (rs_smem(K, W) + 1024));
+  return n < 1 ? 1 : n;
+}
+
+// ------------------------------------------------------ combination by the last CTA
+// true in every thread of the CTA that is the last of n to arrive at *ctr, which it leaves at 0
+// (the counter wraps), and the others' writes are visible to it
+__device__ __forceinline__ bool rows_last(unsigned *ctr, int n) {
+  __shared__ unsigned last_sh;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last_sh = atomicInc(ctr, (unsigned)n - 1u) == (unsigned)n - 1u;
+    __threadfence();
   }
+  __syncthreads();
+  return last_sh != 0u;
 }
-
-// er_stage_entries committed as one group
-__device__ __forceinline__ void er_stage_step(float4 *buf, const float4 *__restrict__ blk, int m0,
-                                              int k, int nb) {
-  er_stage_entries(buf, blk, m0, k, nb);
-  cp_async_commit();
-}
-
-// Ring sweep of one warp over its segment [m0, m1) for float genes in 16-byte aligned
-// rows, with NT sign-block tables.  Sub-step u (32 domains) of the warp's 32 rows lands
-// by cp.async in slot u % ER_RING of the warp's ring of 4 KB tiles, issued ER_RING - 1
-// sub-steps before it is swept, so 8 KB of each warp's loads stay in flight without
-// holding registers.  Every sub-step commits one cp.async group (empty past the
-// segment's end) holding the genes of sub-step u + ER_RING - 1 and, at the start of a
-// 128-domain step, the next step's entries of every table; waiting until at most
-// ER_RING - 2 groups are pending therefore completes sub-step u's genes and, for
-// ER_RING <= 5, its step's entries.  Shared memory `dyn`: [2 steps][NT][ER_STEP_F4_P]
-// entries, then ER_WPC rings of ER_RING tiles.  push(e, E, b) appends block b (0..31)
-// of the current step with sign pattern e; table t's entries of the step start at
-// E + t * 2 * ER_STEP_F4_P (float2).  Every thread of the CTA must call this (it holds
-// CTA barriers); warps without rows (live false) only stage entries.
-constexpr int ER_RING = 3;
-static_assert(ER_RING >= 2 && ER_RING <= 5, "a step's entries must complete with its first sub-step");
-__host__ __device__ constexpr size_t er_ring_smem(int NT) {
-  return sizeof(float4) * (2 * (size_t)NT * ER_STEP_F4_P + (size_t)ER_WPC * ER_RING * 256);
-}
-
-template <int NT, class Push>
-__device__ __forceinline__ void er_ring_sweep(float4 *dyn, const float *__restrict__ g, int64_t ld,
-                                              const EvalShape &sh, const float4 *const *tabs,
-                                              int m0, int m1, int r0, bool live, Push &&push) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float4 *ring = dyn + 2 * NT * ER_STEP_F4_P + warp * (ER_RING * 256);
-  const int nb = (sh.N + 3) >> 2, nsteps = (m1 - m0 + 127) >> 7, nsub = (m1 - m0 + 31) >> 5;
+// thread = row of the row block: its P pieces (few) in index order, the loads of U pieces in
+// flight together, compensated sums
+template <int K, class Close>
+__device__ __forceinline__ void fused_combine(const RowPlan &pl, const float2 *part, int P, int row,
+                                              Close &&close) {
+  if (row >= pl.NP) return;
+  constexpr int U = K == 1 ? 8 : 4;
+  const size_t NPp = pl.NPpad;
+  MonoK acc[K];
 #pragma unroll
-  for (int t = 0; t < NT; ++t) er_stage_entries(dyn + t * ER_STEP_F4_P, tabs[t], m0, 0, nb);
-  cp_async_commit();
+  for (int k = 0; k < K; ++k) acc[k] = monok_zero();
+  for (int p = 0; p < P; p += U) {
+    Mono r[U][K];
 #pragma unroll
-  for (int u = 0; u < ER_RING - 1; ++u) {
-    if (live && u < nsub) er_copy_genes(ring + u * 256, g, ld, sh, r0, m0 + 32 * u);
-    cp_async_commit();
-  }
-  int slot = 0;  // u % ER_RING
-  for (int k = 0; k < nsteps; ++k) {
-    const float2 *bp = (const float2 *)dyn + (size_t)(k & 1) * NT * 2 * ER_STEP_F4_P;
-#pragma unroll 1
-    for (int q = 0; q < 4; ++q) {  // 4 sub-steps of 32 domains
-      const int u = 4 * k + q;
-      if (u >= nsub) break;
-      cp_async_wait<ER_RING - 2>();  // this thread's copies of sub-step u (and of step k)
-      if (q == 0) __syncthreads();   // everyone's; everyone done with step k - 1
-      else __syncwarp();             // the warp's lanes' copies; done with sub-step u - 1
-      const int ua = u + ER_RING - 1;
-      const int sa = slot == 0 ? ER_RING - 1 : slot - 1;  // the slot swept at u - 1
-      if (live && ua < nsub) er_copy_genes(ring + sa * 256, g, ld, sh, r0, m0 + 32 * ua);
-      if (q == 0 && k + 1 < nsteps) {
+    for (int u = 0; u < U; ++u) {
+      const float2 *q = part + (size_t)3 * K * NPp * min(p + u, P - 1) + row;
 #pragma unroll
-        for (int t = 0; t < NT; ++t)
-          er_stage_entries(dyn + (((k + 1) & 1) * NT + t) * ER_STEP_F4_P, tabs[t], m0, k + 1, nb);
+      for (int k = 0; k < K; ++k) {
+        r[u][k].A = __ldcg(q + 3 * k * NPp);
+        r[u][k].B = __ldcg(q + (3 * k + 1) * NPp);
+        r[u][k].C = __ldcg(q + (3 * k + 2) * NPp);
       }
-      cp_async_commit();
-      const float4 *T = ring + slot * 256;
-      slot = slot + 1 == ER_RING ? 0 : slot + 1;
-      if (!live) continue;
-#pragma unroll
-      for (int c4 = 0; c4 < 8; ++c4) push(er_pattern(T[er_tix(lane, c4)]), bp, 8 * q + c4);
     }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (p + u < P) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) monok_fold_in(acc[k], r[u][k]);
+      }
   }
-  cp_async_wait<0>();
+  Mono m[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) m[k] = monok_fold(acc[k]);
+  close(row, m);
 }
 
-// The same sweep with each sub-step's 32 x 32 gene tile brought in by one TMA copy
-// (`gmap`: the genes as an NP x N float matrix, 32 x 32 boxes, 128-byte swizzle, zero
-// fill past the row end and the last row) that completes on the slot's mbarrier; the
-// steps' sign-block entries still come by cp.async, one group per step.  `dyn` must be
-// 1024-byte aligned (the tiles follow the NT tables' 12 KB per table and step); the
-// mbarriers follow the rings: er_ring_smem_tma bytes in all.  A wait that runs out
-// (bounded by %globaltimer) fills the tile with NaN, which makes the rows' results NaN.
-__host__ __device__ constexpr size_t er_ring_smem_tma(int NT) {
-  return er_ring_smem(NT) + (size_t)ER_WPC * ER_RING * 8;
-}
-__device__ __forceinline__ void er_nan_tile(float4 *T) {
-  const float n = __int_as_float(0x7fc00000);
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int c4 = 0; c4 < 8; ++c4) T[er_tix(lane, c4)] = make_float4(n, n, n, n);
-}
-template <int NT, class Push>
-__device__ __forceinline__ void er_ring_sweep_tma(float4 *dyn, const CUtensorMap *gmap,
-                                                  const EvalShape &sh, const float4 *const *tabs,
-                                                  int m0, int m1, int r0, bool live, Push &&push) {
+// Sweep of float genes.  Sub-step u's tile is issued RS_RING - 1 sub-steps ahead into the slot
+// its predecessor has left, on the slot's mbarrier; the tables' steps come a step ahead through
+// registers behind one CTA barrier per step.  A wait on an mbarrier is bounded (%globaltimer);
+// one that runs out makes the rows' results NaN and stops the warp's copies.
+// Partials: part[((piece K + k) 3 + {A, B, C}) NPpad + row].
+// fuse (with a plan of at most RC_FUSE pieces a row): the CTA that completes a row block, found by
+// the block's counter in ctr (0 before and after every call), combines it and calls close(row,
+// the K monoids).
+constexpr int RC_FUSE = 16;
+template <int K, int W, int MODE, bool COMP, class Close>
+__device__ __forceinline__ void rows_sweep(const GeneMaps &maps, const float *__restrict__ src,
+                                           int64_t ld, const RowPlan &pl, const RowTables<K> &tabs,
+                                           float2 *part, unsigned *ctr, Close &&close) {
+  extern __shared__ unsigned char rs_raw[];
+  unsigned char *base = rs_raw + ((1024 - (smem_u32(rs_raw) & 1023)) & 1023);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float4 *ring = dyn + 2 * NT * ER_STEP_F4_P + warp * (ER_RING * 256);
-  const unsigned bar0 =
-      smem_u32(dyn + 2 * NT * ER_STEP_F4_P + ER_WPC * ER_RING * 256) + warp * ER_RING * 8;
-  const int nb = (sh.N + 3) >> 2, nsteps = (m1 - m0 + 127) >> 7, nsub = (m1 - m0 + 31) >> 5;
-#pragma unroll
-  for (int t = 0; t < NT; ++t) er_stage_entries(dyn + t * ER_STEP_F4_P, tabs[t], m0, 0, nb);
-  cp_async_commit();
-  if (live && lane == 0) {
-    for (int k = 0; k < ER_RING; ++k) mbar_init(bar0 + 8 * k, 1);
+  float4 *ring = (float4 *)base + warp * (RS_RING * 256);
+  unsigned char *tab = base + (size_t)W * RS_RING * 4096;
+  const unsigned bar0 = smem_u32(tab + 2 * (size_t)K * RS_TAB) + warp * RS_RING * 8;
+  const int nb = (pl.N + 3) >> 2;
+  const int my = rs_row_of_lane<MODE>(lane);
+  const int sft = MODE == ROWS_TMA4 ? maps.shift[lane >> 3] : 0;
+  // the next phase may be scheduled as this grid's CTAs retire
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (lane == 0) {
+    for (int k = 0; k < RS_RING; ++k) mbar_init(bar0 + 8 * k, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     fence_async_smem();
-    for (int u = 0; u < ER_RING - 1 && u < nsub; ++u) {
-      mbar_expect_tx(bar0 + 8 * u, 4096);
-      tma_load_tile(ring + u * 256, gmap, m0 + 32 * u, r0, bar0 + 8 * u);
-    }
   }
+  // the kernel before (which may still be reading the partials, or writing genes or tables)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   bool ok = true;
-  int u_fail = -1;  // first sub-step whose tile did not arrive in time
-  int slot = 0;     // u % ER_RING
-  for (int k = 0; k < nsteps; ++k) {
-    const float2 *bp = (const float2 *)dyn + (size_t)(k & 1) * NT * 2 * ER_STEP_F4_P;
-#pragma unroll 1
-    for (int q = 0; q < 4; ++q) {  // 4 sub-steps of 32 domains
-      const int u = 4 * k + q;
-      if (u >= nsub) break;
-      if (q == 0) {
-        cp_async_wait<0>();  // this thread's copies of step k's entries
-        __syncthreads();     // everyone's; everyone done with step k - 1
+  int done = 0;    // tiles consumed by this warp so far (all pieces): slot done % RS_RING
+  int issued = 0;  // tiles issued so far
+  int failed = 0;  // done when a wait ran out
+  auto issue = [&](int n, int m, int r0) {  // tile n of this warp: domains m .. m + 31
+    const unsigned bar = bar0 + 8 * (n % RS_RING);
+    float4 *dst = ring + (n % RS_RING) * 256;
+    if (lane == 0) {
+      fence_async_smem();
+      mbar_expect_tx(bar, 4096);
+      if constexpr (MODE == ROWS_TMA) {
+        tma_load_tile(dst, &maps.m[0], m, r0, bar);
       } else {
-        __syncwarp();  // the warp's lanes are done with sub-step u - 1's tile
-      }
-      const int ua = u + ER_RING - 1;
-      const int sa = slot == 0 ? ER_RING - 1 : slot - 1;  // the slot swept at u - 1
-      if (live && lane == 0 && ok && ua < nsub) {
-        fence_async_smem();
-        mbar_expect_tx(bar0 + 8 * sa, 4096);
-        tma_load_tile(ring + sa * 256, gmap, m0 + 32 * ua, r0, bar0 + 8 * sa);
-      }
-      if (q == 0 && k + 1 < nsteps) {
 #pragma unroll
-        for (int t = 0; t < NT; ++t)
-          er_stage_entries(dyn + (((k + 1) & 1) * NT + t) * ER_STEP_F4_P, tabs[t], m0, k + 1, nb);
-        cp_async_commit();
+        for (int c = 0; c < 4; ++c) tma_load_tile(dst + 64 * c, &maps.m[c], m, r0 >> 2, bar);
       }
-      float4 *T = ring + slot * 256;
-      const unsigned bar = bar0 + 8 * slot;
-      slot = slot + 1 == ER_RING ? 0 : slot + 1;
+    }
+    ++issued;
+  };
+  auto arrived = [&](int n) {
+    const bool a = ok && mbar_wait(bar0 + 8 * (n % RS_RING), (n / RS_RING) & 1);
+    if (ok) failed = n;
+    ok = __all_sync(0xffffffffu, a);
+  };
+  const int64_t f1 = min(rp_start(pl, (int64_t)blockIdx.x + 1), (int64_t)pl.RB * pl.nunit * pl.gran);
+  const int64_t per = (int64_t)pl.nunit * pl.gran;  // sub-steps of a row block (the last may be empty)
+  for (int64_t f = rp_start(pl, blockIdx.x); f < f1;) {
+    const int b = (int)(f / per), u0 = (int)(f - b * per);
+    const int u1 = (int)min(per, (int64_t)u0 + (f1 - f));
+    f += u1 - u0;
+    const int m0 = 32 * u0, nsub = min(u1, pl.nsub) - u0;
+    const int nsteps = (nsub + 3) >> 2;
+    const int r0 = (b * W + warp) * 32;
+    const bool live = r0 < pl.NP;
+    const int row = r0 + my;
+    StepRegs<W> R[K];
+#pragma unroll
+    for (int p = 0; p < K; ++p) R[p].load(tabs.blk[p], m0 >> 2, nb);
+    uint32_t tail = 0;  // ROWS_TMA4: pattern of the row's first domains past the last tile
+    if (live) {
+#pragma unroll
+      for (int u = 0; u < RS_RING - 1; ++u)
+        if (ok && u < nsub) issue(done + u, m0 + 32 * u, r0);
+      if constexpr (MODE == ROWS_TMA4) {
+        // the row's last sft columns lie past the last tile: its domains d0 .. d0 + sft - 1
+        const int64_t d0 = 32 * (int64_t)(u0 + nsub) - sft;
+#pragma unroll
+        for (int q = 0; q < 3; ++q)
+          if (q < sft && row < pl.NP && d0 + q < pl.N && src[(int64_t)row * ld + d0 + q] < 0.f)
+            tail |= 1u << q;
+      }
+    }
+    __syncthreads();  // the table buffers of the piece before are free
+#pragma unroll
+    for (int p = 0; p < K; ++p) {
+      R[p].store(tab + p * RS_TAB);
+      if (nsteps > 1) R[p].load(tabs.blk[p], (m0 >> 2) + 32, nb);
+    }
+    RowAcc<COMP> acc[K];
+#pragma unroll
+    for (int p = 0; p < K; ++p) acc[p].zero();
+    uint32_t pat = 0;  // ROWS_TMA4: pattern of the next 16-byte piece
+    for (int k = 0; k < nsteps; ++k) {
+      __syncthreads();  // step k is staged; everyone is done with step k - 1
+      if (live && ok && 4 * k + RS_RING - 1 < nsub)
+        issue(done + RS_RING - 1, m0 + 32 * (4 * k + RS_RING - 1), r0);
+      if (k + 1 < nsteps) {
+#pragma unroll
+        for (int p = 0; p < K; ++p) {
+          R[p].store(tab + (((k + 1) & 1) * K + p) * RS_TAB);
+          if (k + 2 < nsteps) R[p].load(tabs.blk[p], (m0 >> 2) + 32 * (k + 2), nb);
+        }
+      }
       if (!live) continue;
-      const bool arrived = ok && mbar_wait(bar, (u / ER_RING) & 1);
-      if (!__all_sync(0xffffffffu, arrived)) {  // ok is uniform across the warp
-        if (ok) u_fail = u;
-        ok = false;
-        er_nan_tile(T);
-        __syncwarp();
+      const unsigned char *bp = tab + (size_t)(k & 1) * K * RS_TAB;
+#pragma unroll 1
+      for (int q = 0; q < 4; ++q) {  // 4 sub-steps of 32 domains
+        const int u = 4 * k + q;
+        if (u >= nsub) break;
+        const float4 *T = ring + (done % RS_RING) * 256;
+        __syncwarp();  // the warp's lanes are done with the tile before
+        if (q > 0 && ok && u + RS_RING - 1 < nsub)
+          issue(done + RS_RING - 1, m0 + 32 * (u + RS_RING - 1), r0);
+        if (MODE == ROWS_TMA || u == 0) arrived(done);
+        const unsigned char *E = bp + q * (8 * RS_BLOCK);
+        if constexpr (MODE == ROWS_TMA4) {
+          if (u == 0) pat = er_pattern(T[er_tix(lane, 0)]);
+          uint32_t last = tail;  // the pattern after this tile's 8 pieces
+          if (u + 1 < nsub) {
+            arrived(done + 1);
+            last = er_pattern((ring + ((done + 1) % RS_RING) * 256)[er_tix(lane, 0)]);
+          }
+#pragma unroll
+          for (int c4 = 0; c4 < 8; ++c4) {
+            const uint32_t nxt = c4 < 7 ? er_pattern(T[er_tix(lane, c4 < 7 ? c4 + 1 : 7)]) : last;
+            const uint32_t e = (((nxt << 4) | pat) >> sft) & 15u;
+            pat = nxt;
+#pragma unroll
+            for (int p = 0; p < K; ++p) {
+              rs_push(acc[p].m, E + p * RS_TAB + c4 * RS_BLOCK + e * RS_ENTRY);
+              if ((c4 & 3) == 3) acc[p].fold();
+            }
+          }
+        } else {
+#pragma unroll
+          for (int c4 = 0; c4 < 8; ++c4) {
+            const uint32_t o = er_offset(T[er_tix(lane, c4)]);
+#pragma unroll
+            for (int p = 0; p < K; ++p) {
+              rs_push(acc[p].m, E + p * RS_TAB + c4 * RS_BLOCK + o);
+              if ((c4 & 3) == 3) acc[p].fold();
+            }
+          }
+        }
+        ++done;
       }
 #pragma unroll
-      for (int c4 = 0; c4 < 8; ++c4) push(er_pattern(T[er_tix(lane, c4)]), bp, 8 * q + c4);
+      for (int p = 0; p < K; ++p) acc[p].step();
+    }
+    const int piece = (int)blockIdx.x - rp_first(pl, (int64_t)b * pl.nunit);
+    if (live && row < pl.NP) {
+#pragma unroll
+      for (int p = 0; p < K; ++p) {
+        Mono m = acc[p].get();
+        if (!ok) m.A.x = m.A.y = m.B.x = m.B.y = m.C.x = m.C.y = __int_as_float(0x7fc00000);
+        float2 *o = part + ((size_t)piece * K + p) * 3 * pl.NPpad + row;
+        o[0] = m.A;
+        o[pl.NPpad] = m.B;
+        o[2 * (size_t)pl.NPpad] = m.C;
+      }
+    }
+    if (ctr) {
+      const int P = rp_pieces(pl, b);
+      if (rows_last(ctr + b, P)) fused_combine<K>(pl, part, P, b * W * 32 + (int)threadIdx.x, close);
     }
   }
-  cp_async_wait<0>();
-  if (!ok && lane == 0) {  // copies issued after u_fail may still be in flight
-    for (int v = u_fail; v < min(u_fail + ER_RING - 1, nsub); ++v)
-      mbar_wait(bar0 + 8 * (v % ER_RING), (v / ER_RING) & 1);
+  if (!ok && lane == 0) {  // copies of a failed warp may still be in flight
+    for (int n = failed; n < issued; ++n) mbar_wait(bar0 + 8 * (n % RS_RING), (n / RS_RING) & 1);
   }
 }
 
-// append stored entry idx (0..7, the pattern with d_0 = +1) of a block whose 8
-// entries start at E8, with A and B negated when sm = 0x80000000 (the block's pattern
-// has d_0 = -1 and is the complement of entry idx: an exact sign flip, C unchanged)
-__device__ __forceinline__ void er_push_entry(Mono &m, uint32_t idx, uint32_t sm, const float2 *E8) {
-  const float2 *E = E8 + 3 * idx;
-  const float2 a = E[0], b = E[1];
-  Mono R;
-  R.A = make_float2(__uint_as_float(__float_as_uint(a.x) ^ sm), __uint_as_float(__float_as_uint(a.y) ^ sm));
-  R.B = make_float2(__uint_as_float(__float_as_uint(b.x) ^ sm), __uint_as_float(__float_as_uint(b.y) ^ sm));
-  R.C = E[2];
-  m = mono_combine(m, R);
+// ------------------------------------------------------------------- combination
+// The pieces of every row, combined in index order: a CTA of 256 threads takes 256 / runs rows,
+// `runs` threads a row, each a contiguous run of pieces (compensated, its loads in flight
+// together), then a pairwise tree over the runs.  Latency-bound (a few L2 round trips), so runs
+// grows with the pieces: 2 to 4 pieces a thread, 8 rows a CTA at the most pieces.
+constexpr int RC_THREADS = 256;
+inline int rc_runs(const RowPlan &p) {
+  int r = 4;
+  while (r < 32 && 2 * r < p.P) r *= 2;
+  return r;
 }
-
-// append the block with sign pattern e (bit j: d_j = -1)
-__device__ __forceinline__ void er_push_block(Mono &m, uint32_t e, const float2 *E8) {
-  const uint32_t neg = 0u - (e & 1u);  // all ones when d_0 = -1
-  er_push_entry(m, ((e ^ neg) & 0xFu) >> 1, neg & 0x80000000u, E8);
-}
-
-// the 8 sign patterns of a packed word folded onto the stored entries at once: every
-// nibble whose d_0 bit is set is complemented, so stored entry j of the word's block j
-// is bits 4j+1 .. 4j+3 of the result and its sign flip is bit 4j of `lo`
-struct ErWord {
-  uint32_t folded, lo;
-};
-__device__ __forceinline__ ErWord er_fold_word(uint32_t w) {
-  const uint32_t lo = w & 0x11111111u;
-  return {w ^ (lo * 0xFu), lo};
-}
-
-// Running monoid of a lane's row: plain FP32 sums, or (COMP) plain sums over 16
-// domains (4 sign blocks) Kahan-folded into a compensated triple.
-template <bool COMP>
-struct ErAcc {
-  Mono m;
-  MonoK k;
-  __device__ __forceinline__ void zero() {
-    m = mono_zero();
-    if (COMP) k = monok_zero();
-  }
-  __device__ __forceinline__ void fold() {
-    if (COMP) {
-      monok_fold_in(k, m);
-      m = mono_zero();
+// K monoids of row `row` (valid in run 0); sh: K x 256 monoids
+template <int K>
+__device__ __forceinline__ void combine_pieces(const RowPlan &pl, const float2 *__restrict__ part,
+                                               int runs, int row, int run, Mono (*sh)[RC_THREADS],
+                                               Mono out[K]) {
+  const int P = rp_pieces(pl, min(row, pl.NP - 1) / (pl.W * 32));
+  const int c = (P + runs - 1) / runs;
+  const int p0 = run * c, p1 = min(P, p0 + c);
+  const size_t NPp = pl.NPpad;
+  MonoK acc[K];
+#pragma unroll
+  for (int k = 0; k < K; ++k) acc[k] = monok_zero();
+  constexpr int U = K == 1 ? 4 : 2;  // pieces whose loads are in flight together
+  for (int p = p0; p < p1; p += U) {
+    Mono r[U][K];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const float2 *q = part + (size_t)3 * K * NPp * min(p + u, P - 1) + min(row, pl.NP - 1);
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        r[u][k].A = __ldcg(q + 3 * k * NPp);
+        r[u][k].B = __ldcg(q + (3 * k + 1) * NPp);
+        r[u][k].C = __ldcg(q + (3 * k + 2) * NPp);
+      }
     }
-  }
-  __device__ __forceinline__ Mono get() { return COMP ? monok_fold(k) : m; }
-};
-
-// The S segment partials of row `row` combined in index order by one warp: lane l
-// folds its contiguous run of segments [l c, l c + c), c = ceil(S / 32), then the
-// 32 lane results are combined pairwise in lane order.  part is the structure of
-// arrays [comp][S][NPpad] (comp = A, B, C); the result is valid in lane 0.
-__device__ __forceinline__ Mono combine_segments(const float2 *__restrict__ part, int S, int NPpad,
-                                                 int row) {
-  const int lane = threadIdx.x & 31;
-  const size_t stride = (size_t)S * NPpad;
-  const int c = (S + 31) >> 5;
-  const int s0 = lane * c, s1 = min(S, s0 + c);
-  Mono acc = mono_zero();
-  for (int s = s0; s < s1; ++s) {
-    const size_t o = (size_t)s * NPpad + row;
-    Mono r;
-    r.A = part[o];
-    r.B = part[stride + o];
-    r.C = part[2 * stride + o];
-    acc = mono_combine(acc, r);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+      if (p + u < p1) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) monok_fold_in(acc[k], r[u][k]);
+      }
   }
 #pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    Mono r;
-    r.A.x = __shfl_down_sync(0xffffffffu, acc.A.x, off);
-    r.A.y = __shfl_down_sync(0xffffffffu, acc.A.y, off);
-    r.B.x = __shfl_down_sync(0xffffffffu, acc.B.x, off);
-    r.B.y = __shfl_down_sync(0xffffffffu, acc.B.y, off);
-    r.C.x = __shfl_down_sync(0xffffffffu, acc.C.x, off);
-    r.C.y = __shfl_down_sync(0xffffffffu, acc.C.y, off);
-    if ((lane & (2 * off - 1)) == 0) acc = mono_combine(acc, r);
+  for (int k = 0; k < K; ++k) {
+    out[k] = monok_fold(acc[k]);
+    sh[k][threadIdx.x] = out[k];
   }
-  return acc;
+  const int rows = RC_THREADS / runs;  // thread = run * rows + row of the CTA
+  for (int s = 1; s < runs; s <<= 1) {
+    __syncthreads();
+    if ((run & (2 * s - 1)) == 0) {
+#pragma unroll
+      for (int k = 0; k < K; ++k) {
+        out[k] = mono_combine(out[k], sh[k][threadIdx.x + s * rows]);
+        sh[k][threadIdx.x] = out[k];
+      }
+    }
+  }
 }
 
 }  // namespace qpm

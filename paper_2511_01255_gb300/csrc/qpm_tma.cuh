@@ -97,16 +97,17 @@ static inline PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-// rows x cols float matrix with leading dimension ld as 32 x 32 tiles, 128-byte
+// rows x cols float matrix with leading dimension ld as tiles of box_rows x 32, 128-byte
 // swizzle, zero fill outside; false where a TMA copy cannot take it (address not
 // 16-byte aligned, row pitch not a multiple of 16 bytes) or the driver refused
-static inline bool make_tile_map(CUtensorMap *map, const float *base, int rows, int cols, int64_t ld) {
+static inline bool make_tile_map(CUtensorMap *map, const float *base, int rows, int64_t cols, int64_t ld,
+                                 int box_rows = 32) {
   if (((uintptr_t)base & 15) != 0 || (ld % 4) != 0 || ld >= ((int64_t)1 << 37)) return false;
   PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
   if (!fn) return false;
   const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)ld * 4};
-  const cuuint32_t box[2] = {32, 32};
+  const cuuint32_t box[2] = {32, (cuuint32_t)box_rows};
   const cuuint32_t estr[2] = {1, 1};
   return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, (void *)base, dims, strides, box, estr,
             CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
