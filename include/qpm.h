@@ -244,9 +244,9 @@ qpm_status qpm_measure_latency(int32_t kind, int32_t ctas, double *ns_out, qpm_s
  * 32-bit patterns x:
  *   kind 0: the GWO mean's division by 3 (Markstein's residual correction of
  *           x * RN(1/3)) against the IEEE division x / 3 (two NaNs agree);
- *   kind 1: the GWO's r1 and 2 r2 built in the significand of a float in [1, 2)
- *           or [2, 4) against the same values through int-to-float conversions,
- *           r1 = (x >> 16) 2^-16, r2 = (x & 0xFFFF) 2^-16;
+ *   kind 1: the GWO's r1 and 2 r2 built in the significand of a float above 2^23 and
+ *           brought down by one exact multiply-add, against the same values through
+ *           int-to-float conversions, r1 = (x >> 16) 2^-16, r2 = (x & 0xFFFF) 2^-16;
  *   kind 2: the crossover test as one integer compare (x <= 256 floor(2^24 CR)
  *           + 255) against U <= CR in FP32, U = (x >> 8) 2^-24, for CR = 0,
  *           2^-24, 1.5 2^-24, 0.5, 0.9f and its two neighbours, 1.

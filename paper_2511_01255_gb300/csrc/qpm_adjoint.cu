@@ -66,21 +66,8 @@ static int rx_nseg(int N) { return (N + rx_seg_len(N) - 1) / rx_seg_len(N); }
 // saved block of a row: [A (2 floats), 2 unused, then per segment 8 floats]
 static int64_t rx_saved_floats(int N) { return 4 + 8 * (int64_t)rx_nseg(N); }
 
-// Packed FP32 pairs (sm_100+): one 64-bit register pair holds (re, im) of a complex
-// sum, and add/mul/fma.rn.f32x2 apply the IEEE-rounded single operation to both
-// halves in one instruction.  The forward keeps its a-, b- and d^2 q-sums this way
-// (operands straight from the phasor loads); its a P product stays scalar.
-typedef unsigned long long f2x;
-__device__ __forceinline__ f2x f2_pack(float lo, float hi) {
-  f2x r; asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi)); return r; }
-__device__ __forceinline__ float2 f2_unpack(f2x v) {
-  float2 r; asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v)); return r; }
-__device__ __forceinline__ f2x f2_fma(f2x a, f2x b, f2x c) {
-  f2x r; asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c)); return r; }
-__device__ __forceinline__ f2x f2_mul(f2x a, f2x b) {
-  f2x r; asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
-__device__ __forceinline__ f2x f2_add(f2x a, f2x b) {
-  f2x r; asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b)); return r; }
+// The forward keeps its a-, b- and d^2 q-sums as packed pairs (operands straight from the phasor
+// loads); its a P product stays scalar.
 // ------------------------------------------------------------- tanh and tiles
 __device__ __forceinline__ float ex2_approx(float y) {
   float r;

@@ -24,7 +24,7 @@ namespace qpm {
 struct PhiloxKey {
   uint32_t k0[10], k1[10];
 };
-__device__ __forceinline__ PhiloxKey philox_schedule(uint2 key) {
+__host__ __device__ __forceinline__ PhiloxKey philox_schedule(uint2 key) {
   PhiloxKey K;
 #pragma unroll
   for (int r = 0; r < 10; ++r) {
@@ -59,15 +59,56 @@ __device__ __forceinline__ uint4 rng4(const PhiloxKey &K, uint32_t inst, uint32_
 __device__ __forceinline__ float u24(uint32_t w) {
   return __fmul_rn(__uint2float_rn(w >> 8), 0x1p-24f);
 }
-// The GWO pair of one leader and gene: r1 = (w >> 16) 2^-16 and r2 = (w & 0xFFFF) 2^-16.
-// The update needs r1 and C = 2 r2, built without a conversion: the 16 bits go to the
-// top of the significand of a float in [1, 2) (for r1) or [2, 4) (for 2 r2), which is
-// then 1 + r1 or 2 + 2 r2, and one exact subtraction leaves the value.
-__device__ __forceinline__ float u16hi(uint32_t w) {  // r1
-  return __fsub_rn(__uint_as_float(0x3F800000u | ((w >> 9) & 0x007FFF80u)), 1.0f);
+// ------------------------------------------------------------- packed FP32 pairs
+// One 64-bit register pair holds two floats; the .f32x2 operations (sm_100+) round both halves
+// as the scalar operation does, in one instruction.  Used where issue slots bound a loop.
+typedef unsigned long long f2x;
+__device__ __forceinline__ f2x f2_pack(float lo, float hi) {
+  f2x r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
 }
-__device__ __forceinline__ float twice_u16lo(uint32_t w) {  // 2 r2
-  return __fsub_rn(__uint_as_float(0x40000000u | ((w << 7) & 0x007FFF80u)), 2.0f);
+__device__ __forceinline__ float2 f2_unpack(f2x v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ f2x f2_fma(f2x a, f2x b, f2x c) {
+  f2x r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f2x f2_mul(f2x a, f2x b) {
+  f2x r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f2x f2_add(f2x a, f2x b) {
+  f2x r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+// Note: a packed add of a packed product was measured coming out fused (one rounding, .rn or
+// not, also when written as a multiply-add by +1).  Where the product has to round by itself it
+// is taken with the opposite sign and subtracted: f2_sub is not fused with it.
+// a - b: b (-1) is exact, so the sum is the one rounding of the subtraction
+__device__ __forceinline__ f2x f2_sub(f2x a, f2x b) {
+  return f2_fma(b, f2_pack(-1.f, -1.f), a);
+}
+
+// The GWO pair of one leader and gene: r1 = (w >> 16) 2^-16 and r2 = (w & 0xFFFF) 2^-16.
+// The update needs r1 and C = 2 r2, built without a conversion: one byte permute puts the 16
+// bits at the bottom of the significand of 2^23 + n, and one fused multiply-add, exact here,
+// scales and takes the offset off (two genes' at once).
+__device__ __forceinline__ f2x u16hi2(uint32_t w0, uint32_t w1) {  // r1 of two words
+  const f2x f = f2_pack(__uint_as_float(__byte_perm(w0, 0x4B000000u, 0x7632u)),
+                        __uint_as_float(__byte_perm(w1, 0x4B000000u, 0x7632u)));
+  return f2_fma(f, f2_pack(0x1p-16f, 0x1p-16f), f2_pack(-128.f, -128.f));
+}
+__device__ __forceinline__ f2x twice_u16lo2(uint32_t w0, uint32_t w1) {  // 2 r2 of two words
+  const f2x f = f2_pack(__uint_as_float(__byte_perm(w0, 0x4B000000u, 0x7610u)),
+                        __uint_as_float(__byte_perm(w1, 0x4B000000u, 0x7610u)));
+  return f2_fma(f, f2_pack(0x1p-15f, 0x1p-15f), f2_pack(-256.f, -256.f));
 }
 // crossover test U <= CR for U = (w >> 8) 2^-24 and CR in [0, 1], as one integer
 // compare: (w >> 8) <= floor(2^24 CR)  <=>  w <= 256 floor(2^24 CR) + 255
@@ -114,6 +155,14 @@ __device__ __forceinline__ float div3_rn(float x) {
   const float rem = __fmaf_rn(-q, 3.0f, x);
   return fabsf(rem) > 0.0f ? __fmaf_rn(rem, r, q) : q;
 }
+// the same for two values at once
+__device__ __forceinline__ float2 div3_rn2(f2x x) {
+  const f2x r = f2_pack(0x1.555556p-2f, 0x1.555556p-2f);
+  const f2x q = f2_mul(x, r);
+  const f2x rem = f2_fma(q, f2_pack(-3.0f, -3.0f), x);
+  const float2 t = f2_unpack(f2_fma(rem, r, q)), qv = f2_unpack(q), rv = f2_unpack(rem);
+  return make_float2(fabsf(rv.x) > 0.0f ? t.x : qv.x, fabsf(rv.y) > 0.0f ? t.y : qv.y);
+}
 
 // ------------------------------------------------------- asynchronous copies
 // 16 bytes global -> shared through L2 (cp.async.cg), no registers held while in
@@ -154,17 +203,47 @@ __device__ __forceinline__ Mono mono_combine(const Mono &L, const Mono &R) {
   return o;
 }
 
-// append one domain with sign d (+-1.0f) and phasors p = (p1.re, p1.im, p2.re, p2.im)
-__device__ __forceinline__ void mono_push(Mono &m, float d, const float4 &p) {
-  const float ar = d * p.z, ai = d * p.w;  // a = d p2
-  m.C.x = fmaf(ar, m.B.x, m.C.x);
-  m.C.x = fmaf(-ai, m.B.y, m.C.x);
-  m.C.y = fmaf(ar, m.B.y, m.C.y);
-  m.C.y = fmaf(ai, m.B.x, m.C.y);
-  m.A.x += ar;
-  m.A.y += ai;
-  m.B.x = fmaf(d, p.x, m.B.x);  // b = d p1, added after its use: strict prefix
-  m.B.y = fmaf(d, p.y, m.B.y);
+// A running monoid in registers: A and B as pairs (their sums are packed operations), C as two
+// scalars (its products cross the halves).
+struct MonoQ {
+  f2x A, B;
+  float cx, cy;
+  __device__ __forceinline__ void zero() {
+    A = B = 0ull;
+    cx = cy = 0.f;
+  }
+  __device__ __forceinline__ Mono mono() const {
+    Mono o;
+    o.A = f2_unpack(A);
+    o.B = f2_unpack(B);
+    o.C = make_float2(cx, cy);
+    return o;
+  }
+};
+// append one domain with sign d (dd = (d, d), +-1.0f) and phasors p = (p1.re, p1.im, p2.re, p2.im)
+__device__ __forceinline__ void mono_push(MonoQ &m, f2x dd, const float4 &p) {
+  const f2x a = f2_mul(dd, f2_pack(p.z, p.w));  // a = d p2
+  const float2 av = f2_unpack(a), bv = f2_unpack(m.B);
+  m.cx = fmaf(av.x, bv.x, m.cx);
+  m.cx = fmaf(-av.y, bv.y, m.cx);
+  m.cy = fmaf(av.x, bv.y, m.cy);
+  m.cy = fmaf(av.y, bv.x, m.cy);
+  m.A = f2_add(m.A, a);
+  m.B = f2_fma(dd, f2_pack(p.x, p.y), m.B);  // b = d p1, added after its use: strict prefix
+}
+// (d, d) of four genes, d = (x < 0) ? -1 : +1
+struct Signs4 {
+  f2x d[4];
+};
+__device__ __forceinline__ Signs4 signs4(const float4 &u) {
+  const float v[4] = {u.x, u.y, u.z, u.w};
+  Signs4 r;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const float d = v[q] < 0.f ? -1.f : 1.f;
+    r.d[q] = f2_pack(d, d);
+  }
+  return r;
 }
 
 // compensated running triple: every running sum carries its Kahan compensation term

@@ -105,7 +105,7 @@ static __global__ void k_check_div3(unsigned long long *bad, uint32_t *first) {
   uint32_t f = 0xFFFFFFFFu;
   for (uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; b < (1ull << 32); b += stride) {
     const float x = __uint_as_float((uint32_t)b);
-    const float q = div3_rn(x), ref = __fdiv_rn(x, 3.0f);
+    const float q = div3_rn2(f2_pack(1.0f, x)).y, ref = __fdiv_rn(x, 3.0f);
     const bool same = __float_as_uint(q) == __float_as_uint(ref) || (q != q && ref != ref);
     if (!same) {
       ++n;
@@ -128,8 +128,8 @@ static __global__ void k_check_gwo_uniforms(unsigned long long *bad, uint32_t *f
     const uint32_t w = (uint32_t)b;
     const float r1 = __fmul_rn(__uint2float_rn(w >> 16), 0x1p-16f);
     const float r2 = __fmul_rn(__uint2float_rn(w & 0xFFFFu), 0x1p-16f);
-    const bool same = __float_as_uint(u16hi(w)) == __float_as_uint(r1) &&
-                      __float_as_uint(twice_u16lo(w)) == __float_as_uint(__fmul_rn(2.0f, r2));
+    const bool same = __float_as_uint(f2_unpack(u16hi2(w, ~w)).x) == __float_as_uint(r1) &&
+                      __float_as_uint(f2_unpack(twice_u16lo2(~w, w)).y) == __float_as_uint(__fmul_rn(2.0f, r2));
     if (!same) {
       ++n;
       f = min(f, w);

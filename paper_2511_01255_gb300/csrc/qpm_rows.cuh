@@ -52,40 +52,21 @@ __host__ __device__ __forceinline__ int rp_pieces(const RowPlan &p, int b) {
   return rp_first(p, (int64_t)(b + 1) * p.nunit - 1) - rp_first(p, (int64_t)b * p.nunit) + 1;
 }
 
-// ------------------------------------------------------------- packed FP32 pairs
-// One 64-bit register pair holds (re, im); add.rn.f32x2 rounds both halves as the scalar
-// operation does.
-typedef unsigned long long rs_pair;
-__device__ __forceinline__ rs_pair rs_add(rs_pair a, rs_pair b) {
-  rs_pair r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ rs_pair rs_pack(float x, float y) {
-  rs_pair r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
-  return r;
-}
-__device__ __forceinline__ float2 rs_unpack(rs_pair v) {
-  float2 r;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
 struct MonoP {
-  rs_pair A, B, C;
+  f2x A, B, C;
 };
 // m (+) the entry at `e`: mono_combine's operations in its order
 __device__ __forceinline__ void rs_push(MonoP &m, const unsigned char *e) {
-  const rs_pair a = *(const rs_pair *)e, b = *(const rs_pair *)(e + 8);
-  const float2 av = rs_unpack(a), B = rs_unpack(m.B);
-  float2 c = rs_unpack(rs_add(m.C, *(const rs_pair *)(e + 16)));
+  const f2x a = *(const f2x *)e, b = *(const f2x *)(e + 8);
+  const float2 av = f2_unpack(a), B = f2_unpack(m.B);
+  float2 c = f2_unpack(f2_add(m.C, *(const f2x *)(e + 16)));
   c.x = fmaf(av.x, B.x, c.x);
   c.x = fmaf(-av.y, B.y, c.x);
   c.y = fmaf(av.x, B.y, c.y);
   c.y = fmaf(av.y, B.x, c.y);
-  m.C = rs_pack(c.x, c.y);
-  m.A = rs_add(m.A, a);
-  m.B = rs_add(m.B, b);
+  m.C = f2_pack(c.x, c.y);
+  m.A = f2_add(m.A, a);
+  m.B = f2_add(m.B, b);
 }
 
 // Running monoid of a lane's row.  Plain: FP32 sums over a step of 128 domains, each step's
@@ -104,9 +85,9 @@ struct RowAcc {
   }
   __device__ __forceinline__ Mono plain() const {
     Mono r;
-    r.A = rs_unpack(m.A);
-    r.B = rs_unpack(m.B);
-    r.C = rs_unpack(m.C);
+    r.A = f2_unpack(m.A);
+    r.B = f2_unpack(m.B);
+    r.C = f2_unpack(m.C);
     return r;
   }
   __device__ __forceinline__ void fold() {  // every 4 blocks
@@ -136,7 +117,7 @@ struct RowAcc {
 template <int W>
 struct StepRegs {
   static constexpr int N = 256 / (32 * W);
-  rs_pair a[N], b[N], c[N];
+  f2x a[N], b[N], c[N];
   // blocks from b0 on; zero past the problem's nb blocks
   __device__ __forceinline__ void load(const float2 *__restrict__ blk, int b0, int nb) {
 #pragma unroll
@@ -144,7 +125,7 @@ struct StepRegs {
       const int e = threadIdx.x + j * 32 * W, g = b0 + (e >> 3);
       a[j] = b[j] = c[j] = 0ull;
       if (g < nb) {
-        const rs_pair *s = (const rs_pair *)(blk + (size_t)8 * 3 * b0) + 3 * e;
+        const f2x *s = (const f2x *)(blk + (size_t)8 * 3 * b0) + 3 * e;
         a[j] = __ldg(s);
         b[j] = __ldg(s + 1);
         c[j] = __ldg(s + 2);
@@ -153,13 +134,13 @@ struct StepRegs {
   }
   // stored pattern e is pattern 2 e; its complement 15 - 2 e has A and B negated
   __device__ __forceinline__ void store(unsigned char *tab) const {
-    const rs_pair neg = 0x8000000080000000ull;
+    const f2x neg = 0x8000000080000000ull;
 #pragma unroll
     for (int j = 0; j < N; ++j) {
       const int e = threadIdx.x + j * 32 * W;
       unsigned char *t = tab + (e >> 3) * RS_BLOCK;
-      rs_pair *p = (rs_pair *)(t + 2 * (e & 7) * RS_ENTRY);
-      rs_pair *n = (rs_pair *)(t + (15 - 2 * (e & 7)) * RS_ENTRY);
+      f2x *p = (f2x *)(t + 2 * (e & 7) * RS_ENTRY);
+      f2x *n = (f2x *)(t + (15 - 2 * (e & 7)) * RS_ENTRY);
       p[0] = a[j];
       p[1] = b[j];
       p[2] = c[j];
