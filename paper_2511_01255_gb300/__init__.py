@@ -54,6 +54,18 @@ class Objective(ctypes.Structure):
                 ("G0", ctypes.c_float), ("beta", ctypes.c_float)]
 
 
+class _Torch:
+    """torch, imported by the first use of an attribute (the library itself loads without it)."""
+
+    def __getattr__(self, name):
+        global torch, _raw_stream
+        import torch
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        return getattr(torch, name)
+
+
+torch = _Torch()
+_raw_stream = None
 _lib = None
 _P = ctypes.c_void_p
 
@@ -116,36 +128,39 @@ def lib(build=True):
 
 def _check(status):
     if status != 0:
-        raise QpmError(status, lib().qpm_last_error().decode(errors="replace"))
+        raise QpmError(status, _lib.qpm_last_error().decode(errors="replace"))
 
 
+# The marshalling of a call is what its small sizes cost on the host (14 us of a 256 x 1000
+# qpm_eval before the checks below were written out, 3.6 us of them in the library), so the
+# checks go straight to the tensor's own attributes and the stream comes as a raw handle.
 def _ptr(t):
     """Device (or host) address of a tensor, None for None."""
-    if t is None:
-        return None
-    return ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream=None):
-    import torch
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    """cudaStream_t of a torch stream, or of the current one of the current device."""
+    if stream is not None:
+        return stream.cuda_stream
+    dev = torch.cuda.current_device()  # also initialises CUDA
+    return _raw_stream(dev) if _raw_stream is not None else torch.cuda.current_stream().cuda_stream
 
 
 def _cuda(t, what, dtypes, min_numel=0, contiguous=True):
-    """Check that t is a CUDA tensor on the current device with one of `dtypes`,
+    """Check that t is a CUDA tensor on the current device with one of `dtypes` (None: float32),
     at least `min_numel` elements and (if asked) contiguous, before its address
     goes to the library: a wrong pointer would otherwise become an out-of-bounds
     access on the device instead of a Python error."""
-    import torch
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{what}: need a torch tensor, got {type(t).__name__}")
     if not t.is_cuda:
         raise ValueError(f"{what}: need a CUDA tensor, got one on {t.device}")
-    if t.device.index != torch.cuda.current_device():
+    if t.get_device() != torch.cuda.current_device():
         raise ValueError(f"{what}: tensor is on {t.device}, the current device is "
                          f"cuda:{torch.cuda.current_device()}")
-    if t.dtype not in dtypes:
+    if (t.dtype is not torch.float32) if dtypes is None else (t.dtype not in dtypes):
+        dtypes = dtypes or (torch.float32,)
         raise ValueError(f"{what}: need dtype {' or '.join(str(d) for d in dtypes)}, got {t.dtype}")
     if contiguous and not t.is_contiguous():
         raise ValueError(f"{what}: need a contiguous tensor")
@@ -156,7 +171,6 @@ def _cuda(t, what, dtypes, min_numel=0, contiguous=True):
 
 def _host(t, what, dtype, min_numel):
     """Same for the host (CPU) buffers of qpm_solve."""
-    import torch
     if not isinstance(t, torch.Tensor) or t.is_cuda or t.dtype != dtype or not t.is_contiguous():
         raise ValueError(f"{what}: need a contiguous CPU tensor of dtype {dtype}")
     if t.numel() < min_numel:
@@ -164,37 +178,30 @@ def _host(t, what, dtype, min_numel):
     return t
 
 
-def _f32():
-    import torch
-    return (torch.float32,)
-
-
-def _i32():
-    import torch
-    return (torch.int32,)
-
-
 def _rows(t, what, min_cols=0, dtypes=None):
     """(rows, leading dimension) of a row-major 2-D CUDA tensor with unit column
     stride and at least min_cols columns (float32 unless `dtypes` says otherwise)."""
-    _cuda(t, what, dtypes or _f32(), contiguous=False)
-    if t.dim() != 2 or (t.shape[1] > 1 and t.stride(1) != 1):
+    _cuda(t, what, dtypes, contiguous=False)
+    if t.dim() != 2:
         raise ValueError(f"{what}: need a 2-D tensor with contiguous rows")
-    if t.shape[1] < min_cols:
-        raise ValueError(f"{what}: need at least {min_cols} columns, got {t.shape[1]}")
-    if t.shape[0] < 1:
+    rows, cols = t.shape
+    ld, sc = t.stride()
+    if cols > 1 and sc != 1:
+        raise ValueError(f"{what}: need a 2-D tensor with contiguous rows")
+    if cols < min_cols:
+        raise ValueError(f"{what}: need at least {min_cols} columns, got {cols}")
+    if rows < 1:
         raise ValueError(f"{what}: need at least one row")
-    ld = t.stride(0) if t.shape[0] > 1 else max(t.stride(0), t.shape[1])
-    return t.shape[0], ld
+    return rows, (ld if rows > 1 else max(ld, cols))
 
 
 def _out(t, what, min_numel, dtypes=None, optional=True):
-    """An output buffer: None (where allowed) or a contiguous CUDA tensor."""
+    """An output buffer: None (where allowed) or a contiguous CUDA tensor; its address."""
     if t is None:
         if not optional:
             raise ValueError(f"{what}: required")
         return None
-    return _cuda(t, what, dtypes or _f32(), min_numel)
+    return _cuda(t, what, dtypes, min_numel).data_ptr()
 
 
 def _problem(N, kappa1, kappa2):
@@ -205,21 +212,18 @@ def qpm_eval(N, kappa1, kappa2, genes, d_eff, fit=None, compensated=0, stream=No
     """d_eff (float32 [NP, 2]) and fit of the rows of genes (float32 CUDA [NP, ld])."""
     p = _problem(N, kappa1, kappa2)
     NP, ld = _rows(genes, "genes", N)
-    _out(d_eff, "d_eff", 2 * NP, optional=False)
-    _out(fit, "fit", NP)
-    _check(lib().qpm_eval(ctypes.byref(p), _ptr(genes), ld, NP, _ptr(d_eff), _ptr(fit),
+    d, f = _out(d_eff, "d_eff", 2 * NP, optional=False), _out(fit, "fit", NP)
+    _check(lib().qpm_eval(ctypes.byref(p), genes.data_ptr(), ld, NP, d, f,
                           int(compensated), _stream(stream)))
 
 
 def qpm_eval_packed(N, kappa1, kappa2, signs, d_eff, fit=None, compensated=0, stream=None):
     """Same from packed signs (int32/uint32 CUDA [NP, ld_words], bit set -> d = -1)."""
-    import torch
     p = _problem(N, kappa1, kappa2)
-    NP, ld = _rows(signs, "signs", (int(N) + 31) // 32,
-                   (torch.int32,) + ((torch.uint32,) if hasattr(torch, "uint32") else ()))
-    _out(d_eff, "d_eff", 2 * NP, optional=False)
-    _out(fit, "fit", NP)
-    _check(lib().qpm_eval_packed(ctypes.byref(p), _ptr(signs), ld, NP, _ptr(d_eff), _ptr(fit),
+    words = (torch.int32, torch.uint32) if hasattr(torch, "uint32") else (torch.int32,)
+    NP, ld = _rows(signs, "signs", (int(N) + 31) // 32, words)
+    d, f = _out(d_eff, "d_eff", 2 * NP, optional=False), _out(fit, "fit", NP)
+    _check(lib().qpm_eval_packed(ctypes.byref(p), signs.data_ptr(), ld, NP, d, f,
                                  int(compensated), _stream(stream)))
 
 
@@ -227,9 +231,8 @@ def qpm_eval_noalloc(N, kappa1, kappa2, genes, d_eff, fit=None, compensated=0, s
     """qpm_eval without any device allocation (fixed 16 MiB scratch inside the library)."""
     p = _problem(N, kappa1, kappa2)
     NP, ld = _rows(genes, "genes", N)
-    _out(d_eff, "d_eff", 2 * NP, optional=False)
-    _out(fit, "fit", NP)
-    _check(lib().qpm_eval_noalloc(ctypes.byref(p), _ptr(genes), ld, NP, _ptr(d_eff), _ptr(fit),
+    d, f = _out(d_eff, "d_eff", 2 * NP, optional=False), _out(fit, "fit", NP)
+    _check(lib().qpm_eval_noalloc(ctypes.byref(p), genes.data_ptr(), ld, NP, d, f,
                                   int(compensated), _stream(stream)))
 
 
@@ -265,24 +268,23 @@ def qpm_relaxed_saved_floats(N):
 
 def relaxed_saved(B, N, device="cuda"):
     """A saved block for B rows of N domains (float32 [B, qpm_relaxed_saved_floats(N)])."""
-    import torch
     return torch.empty((B, qpm_relaxed_saved_floats(N)), dtype=torch.float32, device=device)
 
 
-def _check_saved(saved, B, N):
-    _cuda(saved, "saved", _f32(), B * qpm_relaxed_saved_floats(N))
-    if saved.data_ptr() % 16:
+def _saved(saved, B, N):
+    """Address of a checked saved block."""
+    p = _cuda(saved, "saved", None, B * qpm_relaxed_saved_floats(N)).data_ptr()
+    if p % 16:
         raise ValueError("saved: need a 16-byte aligned block")
+    return p
 
 
 def qpm_deff_relaxed_fwd(N, kappa1, kappa2, theta, d_eff, fit, saved, stream=None):
     p = _problem(N, kappa1, kappa2)
     B, ld = _rows(theta, "theta", N)
-    _out(d_eff, "d_eff", 2 * B, optional=False)
-    _out(fit, "fit", B)
-    _check_saved(saved, B, N)
-    _check(lib().qpm_deff_relaxed_fwd(ctypes.byref(p), _ptr(theta), ld, B, _ptr(d_eff), _ptr(fit),
-                                      _ptr(saved), _stream(stream)))
+    d, f = _out(d_eff, "d_eff", 2 * B, optional=False), _out(fit, "fit", B)
+    _check(lib().qpm_deff_relaxed_fwd(ctypes.byref(p), theta.data_ptr(), ld, B, d, f,
+                                      _saved(saved, B, N), _stream(stream)))
 
 
 def qpm_deff_relaxed_bwd(N, kappa1, kappa2, theta, d_eff, saved, grad_fit, grad_theta,
@@ -292,16 +294,13 @@ def qpm_deff_relaxed_bwd(N, kappa1, kappa2, theta, d_eff, saved, grad_fit, grad_
     Bg, ldg = _rows(grad_theta, "grad_theta", N)
     if Bg < B:
         raise ValueError(f"grad_theta: need at least {B} rows, got {Bg}")
-    _out(d_eff, "d_eff", 2 * B, optional=False)
-    _out(grad_fit, "grad_fit", B)
-    _check_saved(saved, B, N)
-    _check(lib().qpm_deff_relaxed_bwd(ctypes.byref(p), _ptr(theta), ld, B, _ptr(d_eff),
-                                      _ptr(saved), _ptr(grad_fit), _ptr(grad_theta), ldg,
+    d, gf = _out(d_eff, "d_eff", 2 * B, optional=False), _out(grad_fit, "grad_fit", B)
+    _check(lib().qpm_deff_relaxed_bwd(ctypes.byref(p), theta.data_ptr(), ld, B, d,
+                                      _saved(saved, B, N), gf, grad_theta.data_ptr(), ldg,
                                       _stream(stream)))
 
 
 def _relaxed_function():
-    import torch
 
     class QpmDeff(torch.autograd.Function):
         """f = |d_eff|^2 of each row of theta (d = tanh(theta)); backward is the
@@ -311,9 +310,8 @@ def _relaxed_function():
         def forward(ctx, theta, kappa1, kappa2):
             theta = theta.contiguous()
             B, N = theta.shape
-            D = torch.empty((B, 2), dtype=torch.float32, device=theta.device)
-            f = torch.empty(B, dtype=torch.float32, device=theta.device)
             S = relaxed_saved(B, N, theta.device)
+            D, f = S.new_empty((B, 2)), S.new_empty(B)
             qpm_deff_relaxed_fwd(N, kappa1, kappa2, theta, D, f, S)
             ctx.save_for_backward(theta, D, S)
             ctx.kappa = (kappa1, kappa2)
@@ -346,25 +344,21 @@ def qpm_eval_shg(N, kappa, genes, e_shg, fit=None, stream=None):
     """SHG field integral of each gene row (dk w = kappa)."""
     p = _problem(N, kappa, 0.0)
     NP, ld = _rows(genes, "genes", N)
-    _out(e_shg, "e_shg", 2 * NP, optional=False)
-    _out(fit, "fit", NP)
-    _check(lib().qpm_eval_shg(ctypes.byref(p), _ptr(genes), ld, NP, _ptr(e_shg), _ptr(fit),
-                              _stream(stream)))
+    e, f = _out(e_shg, "e_shg", 2 * NP, optional=False), _out(fit, "fit", NP)
+    _check(lib().qpm_eval_shg(ctypes.byref(p), genes.data_ptr(), ld, NP, e, f, _stream(stream)))
 
 
 def qpm_eval_multi(N, kappas, genes, G0, beta, objective, d_eff=None, stream=None):
     """Multi-wavelength objective for the (kappa1, kappa2) pairs in `kappas`."""
-    import torch
     K = len(kappas)
-    probs = (Problem * K)(*[_problem(N, k1, k2) for k1, k2 in kappas])
+    probs = (Problem * K)(*[(int(N), float(k1), float(k2)) for k1, k2 in kappas])
     NP, ld = _rows(genes, "genes", N)
-    _out(objective, "objective", NP, optional=False)
-    _out(d_eff, "d_eff", 2 * K * NP)
-    nbytes = lib().qpm_eval_multi_scratch_bytes(K, N, NP)
+    o, d = _out(objective, "objective", NP, optional=False), _out(d_eff, "d_eff", 2 * K * NP)
+    L = lib()
+    nbytes = L.qpm_eval_multi_scratch_bytes(K, N, NP)
     scratch = torch.empty(max(1, nbytes), dtype=torch.uint8, device=genes.device)
-    _check(lib().qpm_eval_multi(probs, K, _ptr(genes), ld, NP, float(G0), float(beta),
-                                _ptr(d_eff), _ptr(objective), _ptr(scratch), nbytes,
-                                _stream(stream)))
+    _check(L.qpm_eval_multi(probs, K, genes.data_ptr(), ld, NP, float(G0), float(beta), d, o,
+                            scratch.data_ptr(), nbytes, _stream(stream)))
 
 
 def qpm_release_caches():
@@ -434,7 +428,6 @@ def qpm_set_objective(st, inst, kind, kappas=(), G0=0.0, beta=0.0):
 def qpm_get_F(st, inst=0, F_out=None, stream=None):
     """F of every generation of instance `inst` (float32 CUDA [G + 1]; allocated when
     F_out is None)."""
-    import torch
     _, _, G = qpm_instance_shape(st, inst)
     if F_out is None:
         F_out = torch.empty(G + 1, dtype=torch.float32, device="cuda")
@@ -474,18 +467,17 @@ def qpm_set_population(st, inst, genes, generation, stream=None):
 
 def qpm_get_best(st, inst, genes_out=None, d_eff64_out=None, fit_out=None, index_out=None,
                  stream=None):
-    import torch
     N, _, _ = qpm_instance_shape(st, inst)
     _out(genes_out, "genes_out", N)
     _out(d_eff64_out, "d_eff64_out", 2, (torch.float64,))
     _out(fit_out, "fit_out", 1)
-    _out(index_out, "index_out", 1, _i32())
+    _out(index_out, "index_out", 1, (torch.int32,))
     _check(lib().qpm_get_best(st, int(inst), _ptr(genes_out), _ptr(d_eff64_out), _ptr(fit_out),
                               _ptr(index_out), _stream(stream)))
 
 
 def qpm_polish_leaders(st, inst=0, steps=8, lr=0.5, tau=3.0, accepted_out=None, stream=None):
-    _out(accepted_out, "accepted_out", 3, _i32())
+    _out(accepted_out, "accepted_out", 3, (torch.int32,))
     _check(lib().qpm_polish_leaders(st, int(inst), int(steps), float(lr), float(tau),
                                     _ptr(accepted_out), _stream(stream)))
 
@@ -504,7 +496,6 @@ def qpm_set_wait_timeout_ns(st, ns):
 def qpm_solve(N, kappa1, kappa2, params, mode, best_genes_host, best_deff64_host,
               best_fit_host=None):
     """End to end with host (CPU) tensors; synchronous."""
-    import torch
     p = _problem(N, kappa1, kappa2)
     _host(best_genes_host, "best_genes_host", torch.float32, N)
     _host(best_deff64_host, "best_deff64_host", torch.float64, 2)
@@ -562,7 +553,6 @@ class State:
         return qpm_generation(self.h)
 
     def population(self, inst=0):
-        import torch
         N = self.problems[inst][0]
         NP = self.params[inst].NP
         X = torch.empty((NP, N), dtype=torch.float32, device="cuda")
@@ -572,7 +562,6 @@ class State:
         return X, f, D
 
     def best(self, inst=0):
-        import torch
         N = self.problems[inst][0]
         x = torch.empty(N, dtype=torch.float32, device="cuda")
         d64 = torch.empty(2, dtype=torch.float64, device="cuda")
