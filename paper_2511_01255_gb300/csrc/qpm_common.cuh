@@ -189,12 +189,13 @@ __device__ __forceinline__ Mono mono_zero() {
   m.A = m.B = m.C = make_float2(0.f, 0.f);
   return m;
 }
-// L (+) R, L on the lower indices
+// L (+) R, L on the lower indices (the sums as packed pairs, each rounding as the scalar one)
 __device__ __forceinline__ Mono mono_combine(const Mono &L, const Mono &R) {
   Mono o;
-  o.A = make_float2(L.A.x + R.A.x, L.A.y + R.A.y);
-  o.B = make_float2(L.B.x + R.B.x, L.B.y + R.B.y);
-  float cr = L.C.x + R.C.x, ci = L.C.y + R.C.y;
+  o.A = f2_unpack(f2_add(f2_pack(L.A.x, L.A.y), f2_pack(R.A.x, R.A.y)));
+  o.B = f2_unpack(f2_add(f2_pack(L.B.x, L.B.y), f2_pack(R.B.x, R.B.y)));
+  const float2 c = f2_unpack(f2_add(f2_pack(L.C.x, L.C.y), f2_pack(R.C.x, R.C.y)));
+  float cr = c.x, ci = c.y;
   cr = fmaf(R.A.x, L.B.x, cr);
   cr = fmaf(-R.A.y, L.B.y, cr);
   ci = fmaf(R.A.x, L.B.y, ci);
@@ -296,14 +297,11 @@ __device__ __forceinline__ Mono mono_shfl_down(const Mono &m, int s) {
   return o;
 }
 
-// ordered reduction over the 32 lanes of a warp (lane 0 gets lanes 0..31 combined)
+// ordered reduction over the 32 lanes of a warp (lane 0 gets lanes 0..31 combined): at step s the
+// lanes that are multiples of 2s are right, the others hold values nobody reads
 __device__ __forceinline__ Mono warp_reduce(Mono m) {
-  const int lane = threadIdx.x & 31;
 #pragma unroll
-  for (int s = 1; s < 32; s <<= 1) {
-    const Mono r = mono_shfl_down(m, s);
-    if ((lane & (2 * s - 1)) == 0) m = mono_combine(m, r);
-  }
+  for (int s = 1; s < 32; s <<= 1) m = mono_combine(m, mono_shfl_down(m, s));
   return m;
 }
 

@@ -208,24 +208,6 @@ struct MultiAcc {
   }
 };
 
-// ordered warp reduction of the b-sums alone (the SHG field): the same tree and the
-// same additions as warp_reduce's B
-__device__ __forceinline__ float2 warp_reduce_b(float2 b) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int s = 1; s < 32; s <<= 1) {
-    const float rx = __shfl_down_sync(0xffffffffu, b.x, s);
-    const float ry = __shfl_down_sync(0xffffffffu, b.y, s);
-    if ((lane & (2 * s - 1)) == 0) b = make_float2(b.x + rx, b.y + ry);
-  }
-  return b;
-}
-
-// reduce the K scans (WT: a warp team) and form the objective: f and the first
-// problem's field D0 are valid in the team's first thread; every thread returns.
-// The K warp reductions are independent and run together; a CTA team then passes
-// the warps' partials through shared memory once (sh holds KMAX x warps monoids)
-// and its thread 0 combines them in warp order, as block_reduce does.
 // Several teams per CTA (the multi-wavelength kinds with shared-memory tables): a team
 // is the T consecutive threads [team T, team T + T); team_sync is the team's own
 // named barrier (1 + team), a warp barrier for one-warp teams, or the CTA barrier
@@ -242,67 +224,119 @@ __device__ __forceinline__ void team_sync(const InstDev &I) {
   }
 }
 
+// One step of the K-fold ordered reduction: `n` problems a lane go to n / 2.  Of a pair of lanes
+// s apart the lower keeps the first half of the problems and the upper the second half, each
+// gets the other's partial of what it keeps, and both combine them lower lanes first.
+template <int n, bool SHG, int KM>
+__device__ __forceinline__ void multi_halve(Mono (&m)[KM], int s) {
+  const bool up = (threadIdx.x & s) != 0;
+#pragma unroll
+  for (int e = 0; e < n / 2; ++e) {
+    const Mono keep = up ? m[n / 2 + e] : m[e], give = up ? m[e] : m[n / 2 + e];
+    Mono got;
+    got.B.x = __shfl_xor_sync(0xffffffffu, give.B.x, s);
+    got.B.y = __shfl_xor_sync(0xffffffffu, give.B.y, s);
+    if (SHG) {
+      m[e].B = make_float2(keep.B.x + got.B.x, keep.B.y + got.B.y);
+    } else {
+      got.A.x = __shfl_xor_sync(0xffffffffu, give.A.x, s);
+      got.A.y = __shfl_xor_sync(0xffffffffu, give.A.y, s);
+      got.C.x = __shfl_xor_sync(0xffffffffu, give.C.x, s);
+      got.C.y = __shfl_xor_sync(0xffffffffu, give.C.y, s);
+      // mono_combine of (lower, upper): its sums commute, its product does not
+      Mono L = keep, R = got;
+      if (up) {
+        L.B = got.B;
+        R.A = keep.A;
+        L.A = got.A;
+        R.B = keep.B;
+      }
+      m[e] = mono_combine(L, R);
+    }
+  }
+}
+
+// Reduce the K scans of a team (WT: a warp team) and form the objective: f and the first
+// problem's field D0 are valid in the team's first thread; every thread returns.
+// The K ordered warp reductions run as one: the first steps halve the number of problems a
+// lane carries (multi_halve), after which each of KM lanes finishes one problem's.  The same
+// tree of the same additions per problem as K separate reductions, in about a third of the
+// shuffles (K = 3: 6 monoids exchanged instead of 15).  A CTA team then passes the warps'
+// partials through shared memory (sh holds KM x warps monoids); lane k of its first warp adds
+// problem k's in warp order and forms G_k, and the first thread sums the objective in order.
 template <int MK, bool WT>
 __device__ void multi_finish(const InstDev &I, MultiAcc<MK> &acc, Mono *sh, float &f, float2 &D0) {
-  constexpr int KM = MultiAcc<MK>::KMAX;
+  constexpr int KM = MultiAcc<MK>::KMAX;  // 4 or 8
   constexpr bool SHG = MK == OBJ_MULTI_SHG;
-  const int t = WT ? (int)(threadIdx.x & 31) : team_thread(I);
+  const int t = WT ? (int)(threadIdx.x & 31) : team_thread(I), lane = threadIdx.x & 31;
   Mono m[KM];
 #pragma unroll
-  for (int k = 0; k < KM; ++k) {
-    if (k < I.K) {
-      m[k] = acc.m[k].mono();
-      if (SHG) m[k].B = warp_reduce_b(m[k].B);
-      else m[k] = warp_reduce(m[k]);
+  for (int k = 0; k < KM; ++k) m[k] = acc.m[k].mono();  // zero past K
+  if (KM == 8) {
+    multi_halve<8, SHG>(m, 1);
+    multi_halve<4, SHG>(m, 2);
+    multi_halve<2, SHG>(m, 4);
+  } else {
+    multi_halve<4, SHG>(m, 1);
+    multi_halve<2, SHG>(m, 2);
+  }
+  // lane l < KM now carries problem k(l): the bits of l in reverse
+  const int prob = KM == 8 ? ((lane & 1) << 2) | (lane & 2) | ((lane >> 2) & 1)
+                           : ((lane & 1) << 1) | ((lane >> 1) & 1);
+  Mono r = m[0];
+#pragma unroll
+  for (int s = KM; s < 32; s <<= 1) {
+    if (SHG) {
+      r.B.x += __shfl_down_sync(0xffffffffu, r.B.x, s);
+      r.B.y += __shfl_down_sync(0xffffffffu, r.B.y, s);
+    } else {
+      r = mono_combine(r, mono_shfl_down(r, s));
     }
   }
   if (!WT) {
     // the team's warps and its share of the scratch
-    const int lane = threadIdx.x & 31, warp = t >> 5, nw = I.T >> 5;
+    const int warp = t >> 5, nw = I.T >> 5;
     sh += (size_t)((int)threadIdx.x / I.T) * KM * nw;
     if (nw > 1) {
-      if (lane == 0) {
-#pragma unroll
-        for (int k = 0; k < KM; ++k)
-          if (k < I.K) {
-            if (SHG) sh[k * nw + warp].B = m[k].B;
-            else sh[k * nw + warp] = m[k];
-          }
+      if (lane < KM) {
+        if (SHG) sh[prob * nw + warp].B = r.B;
+        else sh[prob * nw + warp] = r;
       }
       team_sync(I);
-      if (t == 0) {
-#pragma unroll
-        for (int k = 0; k < KM; ++k)
-          if (k < I.K)
-            for (int w = 1; w < nw; ++w) {
-              const Mono &r = sh[k * nw + w];
-              if (SHG) m[k].B = make_float2(m[k].B.x + r.B.x, m[k].B.y + r.B.y);
-              else m[k] = mono_combine(m[k], r);
-            }
+      if (t < KM) {
+        for (int w = 1; w < nw; ++w) {
+          const Mono &q = sh[prob * nw + w];
+          if (SHG) r.B = make_float2(r.B.x + q.B.x, r.B.y + q.B.y);
+          else r = mono_combine(r, q);
+        }
       }
     }
+  }
+  if (t >= 32) return;  // whole warps: the objective is the first warp's
+  float2 Dk = make_float2(0.f, 0.f);
+  float G = 0.f;
+  if (lane < KM && prob < I.K) {
+    if (MK == OBJ_MULTI_THG) {
+      Dk = deff_from(r, I.mkonst[prob][0], I.mkonst[prob][1]);
+    } else {
+      const float2 ph = I.mkonst[prob][3];
+      Dk = make_float2(ph.x * r.B.x - ph.y * r.B.y, ph.x * r.B.y + ph.y * r.B.x);
+    }
+    G = sqrtf(fit_of(Dk));
   }
   float obj = 0.f, gmax = -1.f, gmin = 3.0e38f;
-  if (t == 0) {
 #pragma unroll
-    for (int k = 0; k < KM; ++k) {
-      if (k < I.K) {
-        const Mono &mk = m[k];
-        float2 Dk;
-        if (MK == OBJ_MULTI_THG) {
-          Dk = deff_from(mk, I.mkonst[k][0], I.mkonst[k][1]);
-        } else {
-          const float2 ph = I.mkonst[k][3];
-          Dk = make_float2(ph.x * mk.B.x - ph.y * mk.B.y, ph.x * mk.B.y + ph.y * mk.B.x);
-        }
-        const float G = sqrtf(fit_of(Dk));
-        obj += fabsf(I.G0 - G);
-        gmax = fmaxf(gmax, G);
-        gmin = fminf(gmin, G);
-        if (k == 0) D0 = Dk;
-      }
+  for (int k = 0; k < KM; ++k) {
+    if (k < I.K) {
+      const int src = KM == 8 ? ((k & 1) << 2) | (k & 2) | ((k >> 2) & 1)
+                              : ((k & 1) << 1) | ((k >> 1) & 1);
+      const float Gk = __shfl_sync(0xffffffffu, G, src);
+      obj += fabsf(I.G0 - Gk);
+      gmax = fmaxf(gmax, Gk);
+      gmin = fminf(gmin, Gk);
     }
   }
+  D0 = Dk;  // lane 0 carries problem 0
   f = obj + I.beta * (gmax - gmin);
 }
 
@@ -1286,7 +1320,7 @@ static __global__ void __launch_bounds__(512, 1) k_gwo_mt(InstDev I) {
 
 // Steps 4-5 with the four-leader discrete GWO (launches form)
 template <bool COMP>
-static __global__ void k_gwo_disc(InstDev I) {
+static __global__ void __maxnreg__(80) k_gwo_disc(InstDev I) {
   extern __shared__ float4 dyn[];
   Mono *sh = (Mono *)dyn;
   const int g = *I.gen;
