@@ -368,6 +368,8 @@ static __global__ void __launch_bounds__(RX_WPC * 32, 5)
   rx_carve<NST>(rx_raw, sh.L, ph, tiles, bars);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int seg = blockIdx.y, m0 = seg * sh.L;
+  // a programmatic dependent of whatever ran before, which may have written theta or the tables
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int r0 = (blockIdx.x * RX_WPC + warp) * 32;
   float4 *wt = tiles + (size_t)warp * NST * (RX_TILE / 16);  // this warp's NST tiles
   const unsigned bar0 = smem_u32(bars + warp * NST);
@@ -416,6 +418,8 @@ static __global__ void __launch_bounds__(RX_WPC * 32, 5)
   rx_carve<NST>(rx_raw, sh.L, ph, tiles, bars);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int seg = blockIdx.y, m0 = seg * sh.L;
+  // a programmatic dependent of whatever ran before, which may have written theta or the tables
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int r0 = (blockIdx.x * RX_WPC + warp) * 32;
   const int nsteps = sh.L / RX_STEP;
   float4 *wt = tiles + (size_t)warp * NST * (RX_TILE / 16);
@@ -576,16 +580,6 @@ static dim3 rx_grid(const RelaxShape &sh) {
   return dim3((groups + RX_WPC - 1) / RX_WPC, sh.S);
 }
 
-// dynamic shared memory above the default 48 KB: the kernel's opt-in, set before each
-// launch (a host-side attribute write) to what the longest segment needs, so that a
-// launch with shorter segments never lowers it under one captured earlier
-template <int NST, class K>
-static qpm_status rx_launch_attr(K kernel) {
-  QPM_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)rx_smem_bytes<NST>(RX_LMAX)));
-  return QPM_OK;
-}
-
 }  // namespace qpm
 
 using namespace qpm;
@@ -609,25 +603,13 @@ extern "C" qpm_status qpm_deff_relaxed_fwd(const qpm_problem *prob, const float 
   CUtensorMap tmap{};
   const bool tma = make_tile_map(&tmap, theta, B, sh.N, ld);
   const size_t smem = rx_smem_bytes<RX_NST_F>(sh.L);
-  if (tma) {
-    if ((st = rx_launch_attr<RX_NST_F>(k_relaxed_fwd<true>)) != QPM_OK) return st;
-    k_relaxed_fwd<true><<<grid, RX_WPC * 32, smem, s>>>(tmap, theta, sh, tab, saved);
-  } else {
-    if ((st = rx_launch_attr<RX_NST_F>(k_relaxed_fwd<false>)) != QPM_OK) return st;
-    k_relaxed_fwd<false><<<grid, RX_WPC * 32, smem, s>>>(tmap, theta, sh, tab, saved);
-  }
-  QPM_CUDA(cudaGetLastError());
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((B + 7) / 8);
-  cfg.blockDim = dim3(256);
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  QPM_CUDA(cudaLaunchKernelEx(&cfg, k_relaxed_combine, sh, konst, saved, D, fit));
-  return QPM_OK;
+  static SmemAttr attr[2];
+  const void *fn = tma ? (const void *)k_relaxed_fwd<true> : (const void *)k_relaxed_fwd<false>;
+  if ((st = attr[tma].set(fn, rx_smem_bytes<RX_NST_F>(RX_LMAX))) != QPM_OK) return st;
+  void *args[] = {&tmap, (void *)&theta, &sh, (void *)&tab, &saved};
+  if ((st = launch_dependent(fn, grid, dim3(RX_WPC * 32), args, smem, s)) != QPM_OK) return st;
+  void *cargs[] = {&sh, (void *)&konst, &saved, &D, &fit};
+  return launch_dependent((const void *)k_relaxed_combine, dim3((B + 7) / 8), dim3(256), cargs, 0, s);
 }
 
 template <bool TI, bool TO, bool VG>
@@ -635,12 +617,15 @@ static qpm_status launch_bwd(dim3 grid, size_t smem, cudaStream_t s, const CUten
                              const CUtensorMap &gmap, const float *theta, const RelaxShape &sh,
                              const float4 *tab, const float2 *konst, const float2 *D,
                              const float *saved, const float *gf, float *grad, int64_t ldg) {
-  qpm_status st = rx_launch_attr<RX_NST_B>(k_relaxed_bwd<TI, TO, VG>);
+  // dynamic shared memory above the default 48 KB: set to what the longest segment needs, so
+  // that a launch with shorter segments never lowers it under one captured earlier
+  static SmemAttr attr;
+  const void *fn = (const void *)k_relaxed_bwd<TI, TO, VG>;
+  qpm_status st = attr.set(fn, rx_smem_bytes<RX_NST_B>(RX_LMAX));
   if (st != QPM_OK) return st;
-  k_relaxed_bwd<TI, TO, VG><<<grid, RX_WPC * 32, smem, s>>>(tmap, gmap, theta, sh, tab, konst, D,
-                                                            saved, gf, grad, ldg);
-  QPM_CUDA(cudaGetLastError());
-  return QPM_OK;
+  void *args[] = {(void *)&tmap, (void *)&gmap, (void *)&theta, (void *)&sh,   (void *)&tab, (void *)&konst,
+                  (void *)&D,    (void *)&saved, (void *)&gf,   (void *)&grad, (void *)&ldg};
+  return launch_dependent(fn, grid, dim3(RX_WPC * 32), args, smem, s);
 }
 
 extern "C" qpm_status qpm_deff_relaxed_bwd(const qpm_problem *prob, const float *theta, int64_t ld,

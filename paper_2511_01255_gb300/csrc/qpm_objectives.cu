@@ -47,6 +47,8 @@ static __global__ void __launch_bounds__(SHG_WARPS * 32, 1)
           float2 *__restrict__ eout, float *__restrict__ fout) {
   __shared__ float sums[SHG_WARPS][2 * SHG_RMAX];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // a programmatic dependent of whatever ran before, which may have written genes or the table
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int rend = (int)min((int64_t)NP, (int64_t)(blockIdx.x + 1) * rows_per_cta);
   const int nseg = (N + SHG_SEG - 1) / SHG_SEG;
   const int glast = 4 * (N >> 2) - 4;  // the row's last whole group (VEC: N >= 4)
@@ -290,14 +292,10 @@ extern "C" qpm_status qpm_eval_shg(const qpm_problem *prob, const float *genes, 
   if (st != QPM_OK) return st;
   const bool vec = (ld % 4 == 0) && (((uintptr_t)genes & 15) == 0) && prob->N >= 4;
   const int rpc = (NP + sm_count() - 1) / sm_count(), grid = (NP + rpc - 1) / rpc;
-  if (vec)
-    k_shg<true><<<grid, SHG_WARPS * 32, 0, s>>>(genes, ld, NP, prob->N, rpc, table, konst,
-                                                (float2 *)e_shg, fit);
-  else
-    k_shg<false><<<grid, SHG_WARPS * 32, 0, s>>>(genes, ld, NP, prob->N, rpc, table, konst,
-                                                 (float2 *)e_shg, fit);
-  QPM_CUDA(cudaGetLastError());
-  return QPM_OK;
+  float2 *e = (float2 *)e_shg;
+  void *args[] = {(void *)&genes, &ld, &NP, (void *)&prob->N, (void *)&rpc, (void *)&table, (void *)&konst, &e, &fit};
+  return launch_dependent(vec ? (const void *)k_shg<true> : (const void *)k_shg<false>, dim3(grid),
+                          dim3(SHG_WARPS * 32), args, 0, s);
 }
 
 extern "C" qpm_status qpm_eval_multi(const qpm_problem *probs, int32_t K, const float *genes,
