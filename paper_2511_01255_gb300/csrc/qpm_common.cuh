@@ -316,8 +316,16 @@ __device__ __forceinline__ Mono block_reduce(Mono m, Mono *sh) {
   if (nw == 1) return m;
   if (lane == 0) sh[warp] = m;
   __syncthreads();
-  if (threadIdx.x == 0)
-    for (int w = 1; w < nw; ++w) m = mono_combine(m, sh[w]);
+  if (threadIdx.x == 0) {
+    for (int w0 = 1; w0 < nw; w0 += 8) {  // eight totals in flight, folded in order
+      Mono r[8];
+#pragma unroll
+      for (int j = 0; j < 8; ++j) r[j] = sh[min(w0 + j, nw - 1)];
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        if (w0 + j < nw) m = mono_combine(m, r[j]);
+    }
+  }
   return m;
 }
 

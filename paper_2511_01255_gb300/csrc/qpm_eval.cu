@@ -137,8 +137,10 @@ struct TableEntry {
   double2 *part = nullptr;
   float2 *konst = nullptr;
   cudaEvent_t ready = nullptr;
+  bool built = false;     // `ready` was seen complete: no stream needs to wait for it any more
   float2 *blk = nullptr;  // sign-block table, built on the first packed call
   cudaEvent_t blk_ready = nullptr;
+  bool blk_built = false;
 };
 struct ScratchEntry {
   void *ptr = nullptr;
@@ -181,6 +183,21 @@ size_t device_table_count(int dev) {
   return n;
 }
 
+// `stream` waits for `ev`, unless it was seen complete (a wait costs every call about 0.4 us of host
+// time).  Not asked while the stream is captured, where querying an event is not allowed.
+qpm_status wait_built(cudaStream_t stream, cudaEvent_t ev, bool &built) {
+  if (built) return QPM_OK;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
+      cudaEventQuery(ev) == cudaSuccess) {
+    built = true;
+    return QPM_OK;
+  }
+  cudaGetLastError();  // not ready, or a capture elsewhere forbids the query
+  QPM_CUDA(cudaStreamWaitEvent(stream, ev, 0));
+  return QPM_OK;
+}
+
 // phasor table in natural order for (device, problem); built on `stream` on a miss.
 // blk (if non-NULL) receives the sign-block table, built on `stream` the first time
 // it is asked for.  Never evicts: TableLease makes room before its first lookup.
@@ -214,7 +231,8 @@ qpm_status get_table(const qpm_problem *p, cudaStream_t stream, const float4 **t
     }
     it = g_tables.emplace(key, e).first;
   } else {
-    QPM_CUDA(cudaStreamWaitEvent(stream, it->second.ready, 0));
+    const qpm_status st = wait_built(stream, it->second.ready, it->second.built);
+    if (st != QPM_OK) return st;
   }
   *table = it->second.table;
   *konst = it->second.konst;
@@ -238,7 +256,8 @@ qpm_status get_table(const qpm_problem *p, cudaStream_t stream, const float4 **t
       e.blk = b;
       e.blk_ready = ev;
     } else {
-      QPM_CUDA(cudaStreamWaitEvent(stream, e.blk_ready, 0));
+      const qpm_status st = wait_built(stream, e.blk_ready, e.blk_built);
+      if (st != QPM_OK) return st;
     }
     *blk = e.blk;
   }

@@ -657,7 +657,8 @@ __device__ unsigned long long de_individual(const InstDev &I, const PhiloxKey &K
       p = st[2 * nt];
       q = st[3 * nt];
     } else {
-      a = ld_cur<NC, DUAL>(I, i, si, off);
+      // a known own slot needs one row read, not both
+      a = own_slot >= 0 ? ld_cur<NC, false>(I, i, si, off) : ld_cur<NC, DUAL>(I, i, si, off);
       b = ld_cur<NC, DUAL>(I, r.x, s1, off);
       p = ld_cur<NC, DUAL>(I, r.y, s2, off);
       q = ld_cur<NC, DUAL>(I, r.z, s3, off);
