@@ -207,6 +207,7 @@ __host__ __device__ constexpr int rs_ctas(int K, int W) {
 }
 
 // ------------------------------------------------------ combination by the last CTA
+constexpr int RC_FUSE = 16;  // most pieces of a row that the sweep combines itself
 // true in every thread of the CTA that is the last of n to arrive at *ctr, which it leaves at 0
 // (the counter wraps), and the others' writes are visible to it
 __device__ __forceinline__ bool rows_last(unsigned *ctr, int n) {
@@ -220,39 +221,34 @@ __device__ __forceinline__ bool rows_last(unsigned *ctr, int n) {
   __syncthreads();
   return last_sh != 0u;
 }
-// thread = row of the row block: its P pieces (few) in index order, the loads of U pieces in
-// flight together, compensated sums
+// thread = row of the row block: its P pieces (RC_FUSE at most), all loads of a problem in flight
+// together, combined pairwise in index order (as accurate as a compensated chain at these
+// lengths, and a fifth of its latency)
 template <int K, class Close>
 __device__ __forceinline__ void fused_combine(const RowPlan &pl, const float2 *part, int P, int row,
                                               Close &&close) {
   if (row >= pl.NP) return;
-  constexpr int U = K == 1 ? 8 : 4;
   const size_t NPp = pl.NPpad;
-  MonoK acc[K];
+  Mono m[K];
 #pragma unroll
-  for (int k = 0; k < K; ++k) acc[k] = monok_zero();
-  for (int p = 0; p < P; p += U) {
-    Mono r[U][K];
+  for (int k = 0; k < K; ++k) {
+    Mono r[RC_FUSE];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const float2 *q = part + (size_t)3 * K * NPp * min(p + u, P - 1) + row;
-#pragma unroll
-      for (int k = 0; k < K; ++k) {
-        r[u][k].A = __ldcg(q + 3 * k * NPp);
-        r[u][k].B = __ldcg(q + (3 * k + 1) * NPp);
-        r[u][k].C = __ldcg(q + (3 * k + 2) * NPp);
+    for (int p = 0; p < RC_FUSE; ++p) {
+      r[p] = mono_zero();
+      if (p < P) {
+        const float2 *q = part + ((size_t)K * p + k) * 3 * NPp + row;
+        r[p].A = __ldcg(q);
+        r[p].B = __ldcg(q + NPp);
+        r[p].C = __ldcg(q + 2 * NPp);
       }
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (p + u < P) {
+    for (int s = 1; s < RC_FUSE; s <<= 1)
 #pragma unroll
-        for (int k = 0; k < K; ++k) monok_fold_in(acc[k], r[u][k]);
-      }
+      for (int p = 0; p < RC_FUSE; p += 2 * s) r[p] = mono_combine(r[p], r[p + s]);
+    m[k] = r[0];
   }
-  Mono m[K];
-#pragma unroll
-  for (int k = 0; k < K; ++k) m[k] = monok_fold(acc[k]);
   close(row, m);
 }
 
@@ -264,7 +260,6 @@ __device__ __forceinline__ void fused_combine(const RowPlan &pl, const float2 *p
 // fuse (with a plan of at most RC_FUSE pieces a row): the CTA that completes a row block, found by
 // the block's counter in ctr (0 before and after every call), combines it and calls close(row,
 // the K monoids).
-constexpr int RC_FUSE = 16;
 template <int K, int W, int MODE, bool COMP, class Close>
 __device__ __forceinline__ void rows_sweep(const GeneMaps &maps, const float *__restrict__ src,
                                            int64_t ld, const RowPlan &pl, const RowTables<K> &tabs,
