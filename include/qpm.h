@@ -149,11 +149,10 @@ int32_t qpm_abi_version(void);
  * buffer grown on demand.  The cache holds at most 64 problems per device: a call
  * that needs room for new problems first synchronises the device and frees all of
  * that device's tables and scratch (never while another host thread's call is
- * between its table lookup and its launches).  Rows that start on 16-byte boundaries (genes or
- * signs 16-byte aligned, ld or ld_words a multiple of 4) are read with 16-byte
- * accesses; other rows are read 4 bytes at a time, which is slower but gives
- * results within the same tolerance.  Errors: N < 1, NP < 1, ld < N ->
- * QPM_ERR_ARG.
+ * between its table lookup and its launches).  Gene rows of any alignment are read as
+ * TMA tiles; sign rows that start on 16-byte boundaries (signs 16-byte aligned,
+ * ld_words a multiple of 4) are read with 16-byte accesses, others 4 bytes at a time.
+ * Errors: N < 1, NP < 1, ld < N -> QPM_ERR_ARG.
  * ------------------------------------------------------------------------- */
 qpm_status qpm_eval(const qpm_problem *prob, const float *genes, int64_t ld, int32_t NP,
                     float *d_eff, float *fit, int32_t compensated, qpm_stream_t stream);
@@ -171,7 +170,7 @@ qpm_status qpm_eval_packed(const qpm_problem *prob, const uint32_t *signs, int64
  *   to be minimised, for K <= 4 problems of equal N sharing one read of the
  *   genes.  d_eff device float2 [NP][K] (may be NULL), objective device float [NP].
  *   scratch: caller-owned device memory of at least
- *   qpm_eval_multi_scratch_bytes(K, N, NP) bytes (segment partials).
+ *   qpm_eval_multi_scratch_bytes(K, N, NP) bytes (the rows' partial sums).
  * Phasor tables as for qpm_eval.  Errors: K outside [1, 4], unequal N, N < 1,
  * NP < 1, ld < N, small scratch -> QPM_ERR_ARG.
  * ------------------------------------------------------------------------- */
@@ -192,10 +191,11 @@ size_t qpm_eval_multi_scratch_bytes(int32_t K, int32_t N, int32_t NP);
  * image, which every GPU that loads the library holds until the process exits:
  *   bytes = 192 ceil(N / 4) (sign-block table, rounded up to 256)
  *         + 16 min(1024, ceil(N / 256)) + 256 (the constants and their partial sums)
- *         + 24 S NPpad (segment partials; NPpad = 32 ceil(NP / 32), S the number of
- *           segments the row sweep splits N into, which grows with the SM count)
- *   must not exceed 16777216.  On a 152-SM GB300 that admits N up to about 3.1e5
- *   domains for up to 256 rows, 2.75e5 for 1024 rows and 1.7e5 for 4096 rows.
+ *         + 24 S NPpad (partial sums; NPpad = 32 ceil(NP / 32), S the most pieces the
+ *           row sweep cuts a row into, which grows with the SM count; where that does
+ *           not fit, rows are cut only every 1920 domains, S = ceil(N / 1920))
+ *   must not exceed 16777216.  On a 152-SM GB300 that admits N up to about 3.2e5
+ *   domains for up to 256 rows, 2.75e5 for 1024 rows and 1.68e5 for 4096 rows.
  *   - The first call on each device looks up that array's device address
  *     (cudaGetSymbolAddress) with the device current; make this first call
  *     before any stream capture on that device.

@@ -24,13 +24,15 @@ namespace qpm {
 // ------------------------------------------------------------------ SHG field
 // Bound by HBM (4 bytes a domain, 2 FMA), so all that counts is bytes in flight and an even
 // share per SM.  One CTA per SM takes an equal run of rows.  Its work items are (segment of
-// 384 domains, block of 4 rows), dealt to the 16 warps as equal runs in segment-major order,
-// so a warp holds the segment's phasors in registers from item to item, issues the 12 16-byte
-// loads of an item at once (6 KB a warp, 96 KB an SM) and reduces the item's 4 row sums by
-// halving exchanges (9 shuffles for the 8 components).  Each warp adds its items into its own
-// row sums in shared memory; the CTA adds the warps' in warp order at the end.
-// 5000 rows of N = 3000 (60 MB): the form before it, a CTA per 8 rows that read the phasors
-// from L2 once per CTA, took 29.9 us: 625 CTAs on 608 slots, i.e. a second wave for 17 CTAs.
+// 256 domains, block of 4 rows), dealt to the 16 warps as equal runs in segment-major order,
+// so a warp holds the segment's phasors in registers from item to item, issues the 8 16-byte
+// loads of an item at once with the next item's already in flight (up to 8 KB a warp, 128 KB an
+// SM) and reduces the item's 4 row sums by halving exchanges (9 shuffles for the 8 components).
+// Each warp adds its items into its own row sums in shared memory, the CTA the warps' in warp
+// order at the end, both compensated.
+// 5000 rows of N = 3000 (60 MB, 8.9 us at the copy rate), per call: 30.7 us for the form before
+// it, a CTA per 8 rows (625 CTAs on 608 slots, a second wave for 17 of them, and loads under
+// conditions that were issued one at a time); 14.1 us now.
 static constexpr int SHG_WARPS = 16;
 static constexpr int SHG_Q = 2;                 // 128-domain pieces per segment
 static constexpr int SHG_SEG = 128 * SHG_Q;
@@ -45,7 +47,7 @@ static __global__ void __launch_bounds__(SHG_WARPS * 32, 1)
     k_shg(const float *__restrict__ genes, int64_t ld, int NP, int N, int rows_per_cta,
           const float4 *__restrict__ table, const float2 *__restrict__ konst,
           float2 *__restrict__ eout, float *__restrict__ fout) {
-  __shared__ float sums[SHG_WARPS][2 * SHG_RMAX];
+  __shared__ float sums[SHG_WARPS][2 * SHG_RMAX], comp[SHG_WARPS][2 * SHG_RMAX];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // a programmatic dependent of whatever ran before, which may have written genes or the table
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -55,7 +57,7 @@ static __global__ void __launch_bounds__(SHG_WARPS * 32, 1)
   for (int64_t rs = (int64_t)blockIdx.x * rows_per_cta; rs < rend; rs += SHG_RMAX) {
     const int r0 = (int)rs, rn = min(SHG_RMAX, rend - r0), nrb = (rn + SHG_RB - 1) / SHG_RB;
     for (int e = threadIdx.x; e < SHG_WARPS * 2 * SHG_RMAX; e += SHG_WARPS * 32)
-      (&sums[0][0])[e] = 0.f;
+      (&sums[0][0])[e] = (&comp[0][0])[e] = 0.f;
     __syncthreads();
     const int64_t items = (int64_t)nseg * nrb;
     const int64_t i0 = items * warp / SHG_WARPS, i1 = items * (warp + 1) / SHG_WARPS;
@@ -152,7 +154,10 @@ static __global__ void __launch_bounds__(SHG_WARPS * 32, 1)
       float t = v[0];
       t += __shfl_xor_sync(0xffffffffu, t, 2);
       t += __shfl_xor_sync(0xffffffffu, t, 1);
-      if ((lane & 3) == 0 && rb * SHG_RB + (lane >> 3) < rn) sums[warp][2 * SHG_RB * rb + (lane >> 2)] += t;
+      if ((lane & 3) == 0 && rb * SHG_RB + (lane >> 3) < rn) {
+        const int e = 2 * SHG_RB * rb + (lane >> 2);
+        kahan_add(sums[warp][e], comp[warp][e], t);
+      }
       if (++rb == nrb) {
         rb = 0;
         ++seg;
@@ -162,11 +167,11 @@ static __global__ void __launch_bounds__(SHG_WARPS * 32, 1)
     __syncthreads();
     const int r = threadIdx.x;
     if (r < rn) {
-      float2 t = make_float2(sums[0][2 * r], sums[0][2 * r + 1]);
+      float2 t = make_float2(0.f, 0.f), c = t;
 #pragma unroll
-      for (int w = 1; w < SHG_WARPS; ++w) {
-        t.x += sums[w][2 * r];
-        t.y += sums[w][2 * r + 1];
+      for (int w = 0; w < SHG_WARPS; ++w) {
+        kahan_add(t.x, c.x, __fsub_rn(sums[w][2 * r], comp[w][2 * r]));
+        kahan_add(t.y, c.y, __fsub_rn(sums[w][2 * r + 1], comp[w][2 * r + 1]));
       }
       const float2 ph = konst[3];  // phi(kappa)
       const float2 E = make_float2(ph.x * t.x - ph.y * t.y, ph.x * t.y + ph.y * t.x);
