@@ -531,6 +531,27 @@ __device__ __forceinline__ void push4_staged(Acc<COMP> &acc, const float4 *tbl, 
                          WT ? BATCH_WARPS * 32 : (int)blockDim.x, 0, 0, u);
 }
 
+// The DE donors of the individuals first, first + stride, ...: lane l of a warp draws those of the
+// l-th next one, 32 at a time, and each is handed out by shuffles.  (Every thread of the team
+// drawing the same four numbers per individual was a tenth of the DE phase at N = 3300; 5000
+// rows of it 157.2 -> 152.5 us per generation.  k_de and the batched form, where it made no
+// difference beyond 2 % either way, draw per individual.)
+struct Donors {
+  int4 mine;
+  int k;
+  __device__ __forceinline__ Donors() : k(0) {}
+  __device__ __forceinline__ int4 next(const InstDev &I, const PhiloxKey &K, int g, int i, int stride) {
+    if ((k & 31) == 0) {
+      const int64_t e = (int64_t)i + (int64_t)(threadIdx.x & 31) * stride;
+      mine = de_indices(K, I.inst, (uint32_t)g, e < I.NP ? (int)e : i, I.NP, I.N);
+    }
+    const int s = k & 31;
+    ++k;
+    return make_int4(__shfl_sync(0xffffffffu, mine.x, s), __shfl_sync(0xffffffffu, mine.y, s),
+                     __shfl_sync(0xffffffffu, mine.z, s), __shfl_sync(0xffffffffu, mine.w, s));
+  }
+};
+
 // ---------------------------------------------------- the updates of 4 genes
 // DE rand/1/bin of 4 neighbouring genes: v = fl(x_r1 + fl(F fl(x_r2 - x_r3))) (no FMA), clamped;
 // u = v if U <= CR (integer form, w) or j == jrand, else x.  jm: jrand - (the first gene's index).
@@ -710,14 +731,20 @@ __device__ unsigned long long de_individual(const InstDev &I, const PhiloxKey &K
   return key;
 }
 
+// a_g = 2 (G - g) / G
+__device__ __forceinline__ float a_of(const InstDev &I, int g) {
+  return __fdiv_rn((float)(2 * (I.G - g)), (float)I.G);
+}
+
 // ------------------------------------------------ Step 4-5: GWO + selection
+// a = a_of(I, g), computed once per phase
 // PRE: the three GWO random words of the thread's first group of 4 domains were
 // drawn earlier (while waiting at the grid barrier) and are passed in wpre.
 // One word per leader and gene gives that leader's (r1, r2) as its 16-bit halves.
 template <bool COMP, bool NC, bool TS, bool DUAL, bool WT = false, bool PRE = false,
           bool STG = false, int MK = 0>
 __device__ void gwo_individual(const InstDev &I, const PhiloxKey &K, const float4 *tbl, int g,
-                               int i, int32_t *sel, int la, int lb, int ld, Mono *sh,
+                               float a, int i, int32_t *sel, int la, int lb, int ld, Mono *sh,
                                const uint4 *wpre = nullptr,
                                float4 own0 = make_float4(0.f, 0.f, 0.f, 0.f),
                                float4 own1 = make_float4(0.f, 0.f, 0.f, 0.f),
@@ -734,7 +761,6 @@ __device__ void gwo_individual(const InstDev &I, const PhiloxKey &K, const float
   const int sa = lslot ? lslot[0] : sel[la], sb = lslot ? lslot[1] : sel[lb];
   const int sd = lslot ? lslot[2] : sel[ld];
   float4 *out = (float4 *)row_ptr(I, i, si ^ 1) + t;
-  const float a = __fdiv_rn((float)(2 * (I.G - g)), (float)I.G);
   const float two_a = __fmul_rn(2.0f, a);
   const int n4 = WT ? I.c / 4 : team_groups(I, t);
   const float *rx = row_ptr(I, i, si), *r0 = row_ptr(I, la, sa), *r1 = row_ptr(I, lb, sb);
@@ -1165,12 +1191,13 @@ static __global__ void __maxnreg__(MK ? 128 : 80) k_gwo(InstDev I) {
   const PhiloxKey K = philox_schedule(I.key);
   int32_t *sel = (g & 1) ? I.sel0 : I.sel1;
   const int la = I.lead[0], lb = I.lead[1], ld = I.lead[2];
+  const float a = a_of(I, g);
   int turn = 0;
   for (int i = blockIdx.x; i < I.NP; i += gridDim.x) {
     if (i == la || i == lb || i == ld) continue;  // the leaders do not move
     if (MK) __syncthreads();  // their one reduction scratch is reused
     gwo_individual<COMP, true, TSS, DUAL, false, false, STG, MK>(
-        I, K, I.table, g, i, sel, la, lb, ld, MK ? sh : red_next(sh, turn), nullptr, make_float4(0.f, 0.f, 0.f, 0.f),
+        I, K, I.table, g, a, i, sel, la, lb, ld, MK ? sh : red_next(sh, turn), nullptr, make_float4(0.f, 0.f, 0.f, 0.f),
         make_float4(0.f, 0.f, 0.f, 0.f), nullptr, stg);
   }
   if (I.trace && blockIdx.x == 0 && threadIdx.x < 3) {
@@ -1308,13 +1335,14 @@ static __global__ void __launch_bounds__(512, 1) k_gwo_mt(InstDev I) {
   const PhiloxKey K = philox_schedule(I.key);
   int32_t *sel = (g & 1) ? I.sel0 : I.sel1;
   const int la = I.lead[0], lb = I.lead[1], ld = I.lead[2];
+  const float a = a_of(I, g);
   int cur = team_thread(I) == 0 ? (int)atomicAdd(&I.ctr[3], 1u) : 0;
   for (;;) {
     const int i = mt_next(I, &I.ctr[3], cur);
     if (i >= I.NP) break;
     if (i == la || i == lb || i == ld) continue;  // the leaders do not move
     gwo_individual<false, true, true, false, false, false, true, MK>(
-        I, K, I.table, g, i, sel, la, lb, ld, sh, nullptr, make_float4(0.f, 0.f, 0.f, 0.f),
+        I, K, I.table, g, a, i, sel, la, lb, ld, sh, nullptr, make_float4(0.f, 0.f, 0.f, 0.f),
         make_float4(0.f, 0.f, 0.f, 0.f), nullptr, stg, -1, nullptr, smt);
   }
   if (I.trace && blockIdx.x == 0 && threadIdx.x < 3) {
@@ -1342,12 +1370,10 @@ static __global__ void __maxnreg__(80) k_gwo_disc(InstDev I) {
   const int la = I.lead[0], lb = I.lead[1], lc = I.lead[2], ld = I.lead[3];
   const float *L0 = row_ptr(I, la, sel[la]), *L1 = row_ptr(I, lb, sel[lb]);
   const float *L2 = row_ptr(I, lc, sel[lc]), *L3 = row_ptr(I, ld, sel[ld]);
+  int turn = 0;
   for (int i = blockIdx.x; i < I.NP; i += gridDim.x) {
     if (i == la || i == lb || i == lc || i == ld) continue;
-    // the reduction scratch is reused; letting the warps run ahead (red_next) measured slower
-    // here (99.6 against 92.9 us per generation at 2451 rows of N = 2331)
-    __syncthreads();
-    gwo_discrete_individual<COMP>(I, K, g, i, sel, L0, L1, L2, L3, sh);
+    gwo_discrete_individual<COMP>(I, K, g, i, sel, L0, L1, L2, L3, red_next(sh, turn));
   }
   if (I.trace && blockIdx.x == 0 && threadIdx.x < 4)
     I.trace[(size_t)I.NP * (2 + 2 * (size_t)g) + I.lead[threadIdx.x]] = __int_as_float(0x7fc00000);
@@ -1477,8 +1503,9 @@ static __global__ void __launch_bounds__(MAXT, MAXT > 256 ? 1 : 2)
   for (; g < g_end; ++g) {
     const int32_t *sel_in = (g & 1) ? I.sel1 : I.sel0;
     int32_t *sel_out = (g & 1) ? I.sel0 : I.sel1;
+    Donors donors;
     for (int i = blockIdx.x; i < I.NP; i += gridDim.x) {
-      const int4 r = pre ? r_pre : de_indices(K, I.inst, (uint32_t)g, i, I.NP, I.N);
+      const int4 r = pre ? r_pre : donors.next(I, K, g, i, gridDim.x);
       int slot = 0, impr = 0;
       const unsigned long long key =
           de_individual<COMP, false, TS, DUAL, false, STG>(I, K, tbl, g, i, r, sel_in, sel_out,
@@ -1491,6 +1518,7 @@ static __global__ void __launch_bounds__(MAXT, MAXT > 256 ? 1 : 2)
       }
     }
     grid_arrive(bar, target);
+    const float a = a_of(I, g);
     uint4 wpre[3];
     if (pre) {
       const uint32_t jg = (uint32_t)((threadIdx.x * I.c) >> 2);
@@ -1524,7 +1552,7 @@ static __global__ void __launch_bounds__(MAXT, MAXT > 256 ? 1 : 2)
       if (i == la || i == lb || i == ld) continue;
       if (pre) {
         int gslot = 0;
-        gwo_individual<COMP, false, TS, DUAL, false, true>(I, K, tbl, g, i, sel_out, la, lb, ld,
+        gwo_individual<COMP, false, TS, DUAL, false, true>(I, K, tbl, g, a, i, sel_out, la, lb, ld,
                                                            red_next(sh, turn), wpre, own0, own1, lslot_sh,
                                                            nullptr, own_slot_sh, &gslot);
         // read by every thread after the next barrier's CTA synchronisation
@@ -1532,7 +1560,7 @@ static __global__ void __launch_bounds__(MAXT, MAXT > 256 ? 1 : 2)
       }
       else
         gwo_individual<COMP, false, TS, DUAL, false, false, STG>(
-            I, K, tbl, g, i, sel_out, la, lb, ld, red_next(sh, turn), nullptr,
+            I, K, tbl, g, a, i, sel_out, la, lb, ld, red_next(sh, turn), nullptr,
             make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f), lslot_sh, stg);
     }
     if (I.trace && blockIdx.x == 0 && threadIdx.x < 3) {
@@ -1655,10 +1683,11 @@ __device__ void batch_instance(const InstDev &I, const PhiloxKey &K, int gens, f
     // cluster barrier after the GWO phase orders it before the next DE phase
     if (I.adaptive && crank == 0) adaptive_F_block(I, I.dekey, g);
     const int la = lead_sh[0], lb = lead_sh[1], ld = lead_sh[2];
+    const float a = a_of(I, g);
     for (int i = gw; i < I.NP; i += gstride) {
       if (i == la || i == lb || i == ld) continue;
       gwo_individual<COMP, false, TS, false, true, false, true>(
-          I, K, tbl, g, i, sel_out, la, lb, ld, nullptr, nullptr, make_float4(0.f, 0.f, 0.f, 0.f),
+          I, K, tbl, g, a, i, sel_out, la, lb, ld, nullptr, nullptr, make_float4(0.f, 0.f, 0.f, 0.f),
           make_float4(0.f, 0.f, 0.f, 0.f), nullptr, stg);
     }
     if (I.trace && crank == 0 && threadIdx.x < 3) {
