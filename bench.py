@@ -125,11 +125,10 @@ K_RELAXED_DRAM_BYTES = (67191040 + 679424) + (4265984 + 0) + (71792896 + 1489177
 PHILOX_CALLS_PER_GENE_GEN = 0.25 + 0.75  # crossover word + three GWO words, 4 genes per call
 
 # The packed-sign sweep appends a block of 4 domains per lookup in the sign-block
-# table: per block 2 ops to take its 4 bits from the word, 3 to fold the pattern onto
-# the 8 stored ones, 3 shared-memory loads of (A, B, C), 4 sign flips and the 10 of
-# one monoid combination -> 22 issue slots per 4 domain-evals.  This is the
-# implementation's own count.
-PACKED_OPS_PER_DOMAIN = 22 / 4
+# table: per block 2 ops to take its 4 bits from the word and form the entry's offset,
+# 3 shared-memory loads of (A, B, C) and the 7 of one monoid combination with packed
+# sums -> 12 issue slots per 4 domain-evals.  This is the implementation's own count.
+PACKED_OPS_PER_DOMAIN = 12 / 4
 # The method's count for one domain of a direct scan (no table): the complex
 # multiply-add of a B into C (4 FFMA), A += a (2), B += b (2 FFMA), a = d p2 (2) ->
 # 10 FP32 lane-ops; in FP32 flops (an FFMA counts 2) 6 FFMA + 4 others = 16 - 4 = 12.

@@ -438,7 +438,8 @@ static __global__ void k_init(InstDev I) {
 
 // All instances of a state in one launch (blockIdx.y the instance, largest first; one-warp
 // teams, 8 per CTA).  One launch per instance kept 64 to 512 one-warp CTAs on the GPU, each
-// bound by the latency of its own chain: 27-52 us an instance, 26 ms for 512 of them.
+// bound by the latency of its own chain: 27-52 us an instance.  512 instances of 64 individuals,
+// tables included: 28.9 ms -> 0.52 ms.
 constexpr int INIT_WARPS = 8;
 static __global__ void __launch_bounds__(INIT_WARPS * 32)
     k_init_many(const InstDev *__restrict__ insts, const int32_t *__restrict__ order, int n) {
@@ -624,7 +625,7 @@ __device__ __forceinline__ float4 gwo_update4(const float4 &x, const float4 &L0,
 // The CTA reductions of consecutive individuals take turns on two scratch buffers, so that the
 // other warps start on the next individual while thread 0 still folds the warps' totals and
 // selects: the barrier inside the next reduction is what frees this one's buffer.  (With one
-// buffer and a barrier per individual, 5000 rows of N = 3300 took 164 us per generation.)
+// buffer and a barrier per individual, 5000 rows of N = 3300 took 164 us per generation; 157 with two.)
 __device__ __forceinline__ Mono *red_next(Mono *sh, int &turn) {
   turn ^= 1;
   return sh + (turn ? 0 : (int)(blockDim.x >> 5));
@@ -1135,6 +1136,11 @@ __device__ bool last_cta(unsigned *ctr) {
 // dynamic shared memory of k_de and k_gwo: [row + table staging (long rows)][reduction]
 // The multi-wavelength kinds (MK) stage the rows only: their K phasor tables are read
 // through L1, which keeps them (the rows bypass it).
+//
+// Registers: 80 a thread keep three 256-thread CTAs on an SM (N = 12000, NP = 1000, graph form:
+// 134-138 us per generation; with 72 registers 139, with 64 149).  Launch bounds of 512 threads
+// let the compiler take 128 and halve the CTAs of short rows (discrete GWO 110 against 94 us at
+// N = 2331).  The K scans of MK need 128, for CTAs of up to 512 threads.
 template <bool COMP, bool DUAL, int MK = 0>
 static __global__ void __maxnreg__(MK ? 128 : 80) k_de(InstDev I) {
   constexpr bool STG = !DUAL, TSS = MK != 0;
@@ -1779,7 +1785,8 @@ struct BestRot {
 // 109 us at N = 1000 and 2.08 ms at N = 1e5.  So the domains are spread over the whole GPU, a
 // warp per 128 domains in a CTA of its own, every CTA finding the best individual itself (a
 // few KB of fitness from L2, no grid-wide wait), and a lane takes 4 neighbouring domains with
-// one sincos per mismatch, the other three phasors by rotation.
+// one sincos per mismatch, the other three phasors by rotation: 118 -> 15 us a call at N = 1000
+// and NP = 256, 171 -> 17 at 3300 and 5000, 2.16 ms -> 25 us at 1e5 and 1024.
 constexpr int BEST_THREADS = 128, BEST_DOMAINS = 128;
 static __global__ void __launch_bounds__(BEST_THREADS)
     k_best(InstDev I, BestRot rot, float *genes_out, float *fit_out, int32_t *index_out, int scan) {
@@ -1886,8 +1893,9 @@ static __global__ void __launch_bounds__(BEST_THREADS)
 // order the transposed one, so a warp takes a tile of 32 threads' groups x 8, reads it by 512 B
 // along T, and writes runs of up to 128 B along c / 4 through shared memory (16 bytes a lane
 // where the output rows allow it).  A gene at a time, with a division and reads 16 bytes apart,
-// ran at 2.7-4.3 TB/s of read + write (66 MB of N = 3300 rows in 50 us).  The fitness and
-// field outputs are copied by the same launch.
+// ran at 2.7-4.3 TB/s of read + write (66 MB of N = 3300 rows in 50 us; a call 54 -> 31
+// us, of N = 1e5 and NP = 1024 182 -> 135).  The fitness and field outputs are copied by the same
+// launch.
 constexpr int POP_THREADS = 256, POP_KB = 8;
 static __global__ void __launch_bounds__(POP_THREADS)
     k_population(InstDev I, float *__restrict__ out, int64_t ld, float *__restrict__ fit_out,

@@ -23,6 +23,7 @@
 // register loads):
 //   5000 x 6601 unaligned rows   HBM (6.0 TB/s): 35.6 -> 28.0 us
 //   1024 x 1e5 packed signs      the shared-memory data path (70 % of its cycles): 31.6 -> 28.3 us
+//                                (26.4 per call with the combining kernel, 36.9 before)
 //   5000 x 3000, 3 problems      shared memory and HBM together: 28.2 -> 18.8 us
 //   1024 x 1e5 aligned rows      HBM: 62.8 -> 65 us, and 4 us less for the combination
 #pragma once
@@ -207,7 +208,11 @@ __host__ __device__ constexpr int rs_ctas(int K, int W) {
 }
 
 // ------------------------------------------------------ combination by the last CTA
-constexpr int RC_FUSE = 16;  // most pieces of a row that the sweep combines itself
+// Most pieces of a row that the sweep combines itself: the combining kernel costs a call 4-6 us
+// after the sweep (256 x 1000: 17.9 -> 7.4 us per call without it, together with the shorter host
+// path), but one CTA's threads have the loads of about 16 pieces (6 registers each) in flight at a
+// time, and rows cut finer than that are few and long, where the kernel spreads them over the GPU.
+constexpr int RC_FUSE = 16;
 // true in every thread of the CTA that is the last of n to arrive at *ctr, which it leaves at 0
 // (the counter wraps), and the others' writes are visible to it
 __device__ __forceinline__ bool rows_last(unsigned *ctr, int n) {
