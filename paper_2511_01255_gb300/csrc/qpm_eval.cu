@@ -22,7 +22,7 @@
 namespace qpm {
 
 // Resident CTAs of the packed sweep per SM: 3 of 8 warps, whose 80 registers hold the lookups of
-// several blocks in flight (1024 x 1e5, per call: 26.4 us; 4 of them at 64 registers 30.0, 2 at
+// several blocks in flight (1024 x 1e5, per call: 26.4 us with the combination of then; 4 of them at 64 registers 30.0, 2 at
 // 115 registers 28.0; 4-warp CTAs 28.8-37.1), or 8 of 2 warps (up to 64 rows).
 constexpr int ep_ctas(int W) { return W == 8 ? 3 : 8; }
 
@@ -190,12 +190,15 @@ size_t device_table_count(int dev) {
 qpm_status wait_built(cudaStream_t stream, cudaEvent_t ev, bool &built) {
   if (built) return QPM_OK;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone &&
-      cudaEventQuery(ev) == cudaSuccess) {
-    built = true;
-    return QPM_OK;
+  if (cudaStreamIsCapturing(stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
+    // another thread's global-mode capture forbids queries here, and a forbidden one ends it
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    QPM_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+    built = cudaEventQuery(ev) == cudaSuccess;
+    QPM_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
+    if (built) return QPM_OK;
   }
-  cudaGetLastError();  // not ready, or a capture elsewhere forbids the query
+  cudaGetLastError();  // not ready
   QPM_CUDA(cudaStreamWaitEvent(stream, ev, 0));
   return QPM_OK;
 }
