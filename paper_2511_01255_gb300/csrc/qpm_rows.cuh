@@ -21,9 +21,9 @@
 // What bounds it and what it measured (ncu, cold and serialised, against the form before it:
 // 8-pattern table through cp.async, segments rounded to 128 domains, unaligned rows by 4-byte
 // register loads):
-//   5000 x 6601 unaligned rows   HBM (6.0 TB/s): 35.6 -> 28.0 us
+//   5000 x 6601 unaligned rows   HBM (5.7 TB/s while the SMs are active): 35.6 -> 28.0 us
 //   1024 x 1e5 packed signs      the shared-memory data path (70 % of its cycles): 31.6 -> 28.3 us
-//                                (26.4 per call with the combining kernel, 36.9 before)
+//                                (25.8 per call with the combining kernel, 36.9 before)
 //   5000 x 3000, 3 problems      shared memory and HBM together: 28.2 -> 18.8 us
 //   1024 x 1e5 aligned rows      HBM: 62.8 -> 65 us, and 4 us less for the combination
 #pragma once
@@ -430,8 +430,12 @@ __device__ __forceinline__ void rows_sweep(const GeneMaps &maps, const float *__
 
 // ------------------------------------------------------------------- combination
 // The pieces of every row, combined in index order: a CTA of 256 threads takes 256 / runs rows,
-// `runs` threads a row, each a contiguous run of pieces (compensated, its loads in flight
-// together), then a pairwise tree over the runs.  Latency-bound (a few L2 round trips), so runs
+// `runs` threads a row, each a contiguous run of pieces, then a pairwise tree over the runs.  A
+// run is combined pairwise in groups whose loads are in flight together; where it has several
+// groups they are summed compensated.  (Compensated from piece to piece, 1024 x 1e5 packed signs
+// took 26.4 us per call instead of 25.8, for the same error against 64 bits.)  Up to RC_FUSE pieces
+// it is fused_combine's tree, so a row has the same bits either way.
+// Latency-bound (a few L2 round trips), so runs
 // grows with the pieces: 2 to 4 pieces a thread, 8 rows a CTA at the most pieces.
 constexpr int RC_THREADS = 256;
 inline int rc_runs(const RowPlan &p) {
@@ -450,7 +454,10 @@ __device__ __forceinline__ void combine_pieces(const RowPlan &pl, const float2 *
   const size_t NPp = pl.NPpad;
   MonoK acc[K];
 #pragma unroll
-  for (int k = 0; k < K; ++k) acc[k] = monok_zero();
+  for (int k = 0; k < K; ++k) {
+    acc[k] = monok_zero();
+    out[k] = mono_zero();
+  }
   constexpr int U = K == 1 ? 4 : 2;  // pieces whose loads are in flight together
   for (int p = p0; p < p1; p += U) {
     Mono r[U][K];
@@ -465,15 +472,21 @@ __device__ __forceinline__ void combine_pieces(const RowPlan &pl, const float2 *
       }
     }
 #pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (p + u < p1) {
+    for (int k = 0; k < K; ++k) {
 #pragma unroll
-        for (int k = 0; k < K; ++k) monok_fold_in(acc[k], r[u][k]);
-      }
+      for (int u = 1; u < U; ++u)
+        if (p + u >= p1) r[u][k] = mono_zero();
+#pragma unroll
+      for (int s = 1; s < U; s <<= 1)
+#pragma unroll
+        for (int u = 0; u < U; u += 2 * s) r[u][k] = mono_combine(r[u][k], r[u + s][k]);
+      if (c <= U) out[k] = r[0][k];
+      else monok_fold_in(acc[k], r[0][k]);
+    }
   }
 #pragma unroll
   for (int k = 0; k < K; ++k) {
-    out[k] = monok_fold(acc[k]);
+    if (c > U) out[k] = monok_fold(acc[k]);
     sh[k][threadIdx.x] = out[k];
   }
   const int rows = RC_THREADS / runs;  // thread = run * rows + row of the CTA

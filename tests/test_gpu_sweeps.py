@@ -104,3 +104,39 @@ def test_shg_rows(q, orc, N, NP, pad, off):
     ref = orc.shg_genes(X, K1)
     # random rows cancel: floor at 1e-3 of the all-up magnitude scale N
     assert (np.abs(E[:, 0] + 1j * E[:, 1] - ref) / np.maximum(np.abs(ref), 1e-3 * N)).max() < TOL_D
+
+
+# A captured call leaves the rows to the combining kernel, which takes the same tree over up to 16
+# pieces: the same bits as the sweep's own combination.
+@pytest.mark.parametrize("N,NP,K", [(129, 129, 1), (1000, 256, 1), (1923, 40, 1), (5003, 2100, 1),
+                                    (1000, 256, 2), (5003, 2100, 3)])
+def test_captured_rows_same_bits(q, N, NP, K):
+    import torch
+    view, _ = rows_of(NP, N, N, 0, N + K)
+    kaps = [(K1 * (1 + 0.01 * k), K2) for k in range(K)]
+    D = torch.empty((NP, 2 * K), device="cuda")
+    f = torch.empty(NP, device="cuda")
+    s = torch.cuda.Stream()
+
+    def call():
+        if K == 1:
+            q.qpm_eval(N, K1, K2, view, D, f, 1)
+        else:
+            q.qpm_eval_multi(N, kaps, view, 1e5, 0.5, f, D)
+
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        call()  # tables and the stream's scratch
+        s.synchronize()
+        call()  # sees the tables complete
+        s.synchronize()
+        ref = D.clone()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=s):
+        call()
+    for _ in range(2):
+        D.fill_(float("nan"))
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(D, ref)
