@@ -22,8 +22,9 @@
 namespace qpm {
 
 // Resident CTAs of the packed sweep per SM: 3 of 8 warps, whose 80 registers hold the lookups of
-// several blocks in flight (1024 x 1e5, per call: 26.4 us with the combination of then; 4 of them at 64 registers 30.0, 2 at
-// 115 registers 28.0; 4-warp CTAs 28.8-37.1), or 8 of 2 warps (up to 64 rows).
+// several blocks in flight (1024 x 1e5, per call: 26.4 us with the combination of then; 4 of them
+// at 64 registers 30.0, 2 at 115 registers 28.0; 4-warp CTAs 28.8-37.1), or 8 of 2 warps (up to
+// 64 rows).
 constexpr int ep_ctas(int W) { return W == 8 ? 3 : 8; }
 
 // float genes: see rows_sweep; ctr not NULL: the sweep combines the rows itself
