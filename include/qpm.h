@@ -170,7 +170,8 @@ qpm_status qpm_eval_packed(const qpm_problem *prob, const uint32_t *signs, int64
  *   to be minimised, for K <= 4 problems of equal N sharing one read of the
  *   genes.  d_eff device float2 [NP][K] (may be NULL), objective device float [NP].
  *   scratch: caller-owned device memory of at least
- *   qpm_eval_multi_scratch_bytes(K, N, NP) bytes (the rows' partial sums).
+ *   qpm_eval_multi_scratch_bytes(K, N, NP) bytes, 8-byte aligned (the rows' partial sums
+ *   and the words that count them; it may hold anything before the call).
  * Phasor tables as for qpm_eval.  Errors: K outside [1, 4], unequal N, N < 1,
  * NP < 1, ld < N, small scratch -> QPM_ERR_ARG.
  * ------------------------------------------------------------------------- */

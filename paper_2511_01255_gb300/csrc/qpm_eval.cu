@@ -8,6 +8,8 @@
 #include <math.h>
 
 #include <algorithm>
+#include <atomic>
+#include <chrono>
 #include <map>
 #include <mutex>
 #include <string.h>
@@ -27,14 +29,14 @@ namespace qpm {
 // 64 rows).
 constexpr int ep_ctas(int W) { return W == 8 ? 3 : 8; }
 
-// float genes: see rows_sweep; ctr not NULL: the sweep combines the rows itself
+// float genes: see rows_sweep; words in `fuse`: the sweep combines the rows itself
 template <int W, int MODE, bool COMP>
 static __global__ void __launch_bounds__(W * 32, rs_ctas(1, W))
     k_eval_genes(const __grid_constant__ GeneMaps maps, const float *__restrict__ src, int64_t ld,
-                 RowPlan pl, RowTables<1> tabs, float2 *part, unsigned *ctr,
+                 RowPlan pl, RowTables<1> tabs, float2 *part, RowFuse fuse,
                  const float2 *__restrict__ konst, float2 *__restrict__ deff,
                  float *__restrict__ fit) {
-  rows_sweep<1, W, MODE, COMP>(maps, src, ld, pl, tabs, part, ctr, [&](int row, const Mono *m) {
+  rows_sweep<1, W, MODE, COMP>(maps, src, ld, pl, tabs, part, fuse, [&](int row, const Mono *m) {
     const float2 D = deff_from(m[0], konst[0], konst[1]);
     deff[row] = D;
     if (fit) fit[row] = fit_of(D);
@@ -128,10 +130,6 @@ static __global__ void __launch_bounds__(RC_THREADS)
     if (fit) fit[row] = fit_of(D);
   }
 }
-
-// counters of the fused combination, at the start of every scratch buffer
-constexpr int FUSE_BLOCKS = 4096;
-constexpr size_t FUSE_BYTES = sizeof(unsigned) * FUSE_BLOCKS;
 
 // ------------------------------------------------------------- caches (host)
 namespace {
@@ -282,12 +280,6 @@ qpm_status get_scratch(cudaStream_t stream, size_t bytes, void **ptr) {
       e.bytes = 0;
     }
     QPM_CUDA(cudaMalloc(&e.ptr, bytes));
-    const cudaError_t ce = cudaMemsetAsync(e.ptr, 0, std::min(bytes, FUSE_BYTES), stream);
-    if (ce != cudaSuccess) {  // no scratch without its counters
-      cudaFree(e.ptr);
-      e.ptr = nullptr;
-      return cuda_fail(ce, "clearing the scratch counters");
-    }
     e.bytes = bytes;
   }
   *ptr = e.ptr;
@@ -359,10 +351,10 @@ qpm_status make_gene_maps(GeneMaps *gm, int *mode, const float *genes, int NP, i
   return QPM_OK;
 }
 
-// what closes a call: the counters of the fused combination (NULL: the combining kernel), the
-// constants and the outputs
+// what closes a call: the fused combination (no words: the combining kernel), the constants and
+// the outputs
 struct EvalOut {
-  unsigned *ctr;
+  RowFuse fuse;
   const float2 *konst;
   float2 *deff;
   float *fit;
@@ -377,7 +369,7 @@ static qpm_status launch_genes(const GeneMaps &gm, const float *g, int64_t ld, c
   const qpm_status st = attr.set(fn, rs_smem(1, W));
   if (st != QPM_OK) return st;
   void *args[] = {(void *)&gm, (void *)&g, (void *)&ld, (void *)&pl, (void *)&tabs, (void *)&part,
-                  (void *)&out.ctr, (void *)&out.konst, (void *)&out.deff, (void *)&out.fit};
+                  (void *)&out.fuse, (void *)&out.konst, (void *)&out.deff, (void *)&out.fit};
   return launch_dependent(fn, dim3(pl.C), dim3(W * 32), args, rs_smem(1, W), stream);
 }
 
@@ -411,7 +403,7 @@ static qpm_status launch_eval_rows(bool comp, const float *g, int64_t ld, const 
     else QPM_EG(1, ROWS_TMA4);
   }
 #undef QPM_EG
-  if (st != QPM_OK || out.ctr) return st;
+  if (st != QPM_OK || out.fuse.words) return st;
   return launch_combine(pl, part, out, stream);
 }
 
@@ -427,21 +419,26 @@ static qpm_status launch_packed(bool vecw, bool comp, const uint32_t *src, int64
   return launch_dependent(fn, dim3(pl.C), dim3(W * 32), args, 0, stream);
 }
 
-// the counters of a fused combination: where a row has few pieces, at the start of the
-// stream's scratch (lease held); not in a captured call, whose replays may overlap others
-qpm_status fuse_counters(const RowPlan &pl, cudaStream_t stream, unsigned **ctr) {
-  *ctr = nullptr;
-  if (pl.P > RC_FUSE || pl.RB > FUSE_BLOCKS) return QPM_OK;
+size_t fuse_bytes(const RowPlan &pl) {
+  return pl.P <= RC_FUSE ? sizeof(unsigned long long) * (size_t)RF_STRIDE * (size_t)pl.RB : 0;
+}
+
+RowFuse row_fuse(const RowPlan &pl, void *words, cudaStream_t stream) {
+  // tags count up from a start that no memory holds by chance (the clock, spread over 64 bits)
+  static std::atomic<unsigned long long> tag{
+      ((unsigned long long)std::chrono::steady_clock::now().time_since_epoch().count() | 1ull) *
+      0x9E3779B97F4A7C15ull};
+  RowFuse f;
+  if (pl.P > RC_FUSE) return f;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) {
     cudaGetLastError();
-    return QPM_OK;
+    return f;
   }
-  if (cap != cudaStreamCaptureStatusNone) return QPM_OK;
-  void *scratch = nullptr;
-  const qpm_status st = get_scratch(stream, FUSE_BYTES, &scratch);
-  *ctr = (unsigned *)scratch;
-  return st;
+  if (cap != cudaStreamCaptureStatusNone) return f;
+  f.words = (unsigned long long *)words;
+  f.tag = tag.fetch_add(1, std::memory_order_relaxed) & (~0ull >> RF_BITS);
+  return f;
 }
 
 static qpm_status eval_common(const qpm_problem *prob, const void *src, int64_t ld, int32_t NP,
@@ -460,10 +457,11 @@ static qpm_status eval_common(const qpm_problem *prob, const void *src, int64_t 
   const int W = kind == 2 ? (NP <= 64 ? 2 : 8) : 0;
   const RowPlan pl = kind == 2 ? packed_plan(NP, prob->N, W) : genes_plan(1, NP, prob->N);
   void *scratch;
-  st = get_scratch(stream, FUSE_BYTES + plan_bytes(pl, 1), &scratch);
+  const size_t partials = plan_bytes(pl, 1);
+  st = get_scratch(stream, partials + (kind == 2 ? 0 : fuse_bytes(pl)), &scratch);
   if (st != QPM_OK) return st;
-  float2 *part = (float2 *)((char *)scratch + FUSE_BYTES);
-  EvalOut out{nullptr, konst, (float2 *)d_eff, fit};
+  float2 *part = (float2 *)scratch;
+  EvalOut out{RowFuse{}, konst, (float2 *)d_eff, fit};
   if (kind == 2) {
     const bool vecw = (ld % 4 == 0) && (((uintptr_t)src & 15) == 0);
     const RowTables<1> tabs{{blk}};
@@ -471,8 +469,7 @@ static qpm_status eval_common(const qpm_problem *prob, const void *src, int64_t 
                 : launch_packed<2>(vecw, comp != 0, (const uint32_t *)src, ld, pl, tabs, part, stream);
     return st != QPM_OK ? st : launch_combine(pl, part, out, stream);
   }
-  st = fuse_counters(pl, stream, &out.ctr);
-  if (st != QPM_OK) return st;
+  out.fuse = row_fuse(pl, (char *)scratch + partials, stream);
   return launch_eval_rows(comp != 0, (const float *)src, ld, pl, blk, part, out, stream);
 }
 
@@ -565,9 +562,9 @@ extern "C" qpm_status qpm_eval_noalloc(const qpm_problem *prob, const float *gen
   if (st != QPM_OK) return st;
   st = launch_block_table(prob->N, prob->kappa1, prob->kappa2, blk, s);
   if (st != QPM_OK) return st;
-  // no counters in the shared array, whose words need not start at zero
+  // always the combining kernel: the call may be captured and replayed
   return launch_eval_rows(compensated != 0, genes, ld, pl, blk, part,
-                          EvalOut{nullptr, konst, (float2 *)d_eff, fit}, s);
+                          EvalOut{RowFuse{}, konst, (float2 *)d_eff, fit}, s);
 }
 
 qpm::TableLease::TableLease(const qpm_problem *problems, int count) {

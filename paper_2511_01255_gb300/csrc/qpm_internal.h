@@ -95,9 +95,17 @@ RowPlan row_plan(int NP, int N, int W, int slots, int gran, int maxsub, int min_
 // the plan of the float-gene sweep with K sign-block tables; whole: no row is split unless it
 // is longer than a run may be (fewest pieces)
 RowPlan genes_plan(int K, int NP, int N, bool whole = false);
-// counters of the plan's fused combination on this stream (NULL: the combining kernel); the
-// caller holds a TableLease until the sweep is enqueued
-qpm_status fuse_counters(const RowPlan &pl, cudaStream_t stream, unsigned **ctr);
+// What a sweep that combines its rows itself counts arrivals with (rows_last): a word per row block
+// behind the call's partials, whatever it holds before the call, and the call's own tag, which
+// no other call of the process has
+struct RowFuse {
+  unsigned long long *words = nullptr;  // NULL: the combining kernel
+  unsigned long long tag = 0;
+};
+// the plan's fused combination with the words at `words` (fuse_bytes): none where a row has many
+// pieces or the call is captured (a replay would find its own tag)
+RowFuse row_fuse(const RowPlan &pl, void *words, cudaStream_t stream);
+size_t fuse_bytes(const RowPlan &pl);
 constexpr int EVAL_MAX_ROWS = 128 * 65535;  // rows a call of the row sweeps takes
 // bytes of the plan's partial monoids for K problems
 inline size_t plan_bytes(const RowPlan &p, int K) {

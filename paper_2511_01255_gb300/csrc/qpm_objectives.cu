@@ -213,8 +213,8 @@ __device__ __forceinline__ void multi_close(const MultiOut<K> &o, int row, const
 template <int K, int W, int MODE>
 static __global__ void __launch_bounds__(W * 32, rs_ctas(K, W))
     k_multi_genes(const __grid_constant__ GeneMaps maps, const float *__restrict__ src, int64_t ld,
-                  RowPlan pl, RowTables<K> tabs, float2 *part, unsigned *ctr, MultiOut<K> out) {
-  rows_sweep<K, W, MODE, false>(maps, src, ld, pl, tabs, part, ctr,
+                  RowPlan pl, RowTables<K> tabs, float2 *part, RowFuse fuse, MultiOut<K> out) {
+  rows_sweep<K, W, MODE, false>(maps, src, ld, pl, tabs, part, fuse,
                                 [&](int row, const Mono *m) { multi_close<K>(out, row, m); });
 }
 
@@ -233,14 +233,14 @@ static __global__ void __launch_bounds__(RC_THREADS)
 
 template <int K, int W, int MODE>
 static qpm_status launch_multi_genes(const GeneMaps &gm, const float *g, int64_t ld, const RowPlan &pl,
-                                     const RowTables<K> &tabs, float2 *part, unsigned *ctr,
+                                     const RowTables<K> &tabs, float2 *part, const RowFuse &fuse,
                                      const MultiOut<K> &out, cudaStream_t s) {
   static SmemAttr attr;
   const void *fn = (const void *)k_multi_genes<K, W, MODE>;
   const qpm_status st = attr.set(fn, rs_smem(K, W));
   if (st != QPM_OK) return st;
   void *args[] = {(void *)&gm, (void *)&g, (void *)&ld, (void *)&pl, (void *)&tabs, (void *)&part,
-                  (void *)&ctr, (void *)&out};
+                  (void *)&fuse, (void *)&out};
   return launch_dependent(fn, dim3(pl.C), dim3(W * 32), args, rs_smem(K, W), s);
 }
 
@@ -254,16 +254,15 @@ static qpm_status launch_multi(const float2 *const *blk, const float2 *const *ko
   qpm_status st = make_gene_maps(&gm, &mode, g, pl.NP, pl.N, ld);
   if (st != QPM_OK) return st;
   float2 *part = (float2 *)scratch;
-  unsigned *ctr = nullptr;
-  st = fuse_counters(pl, s, &ctr);
-  if (st != QPM_OK) return st;
+  // partials and words are the caller's: calls with scratch of their own stay independent
+  const RowFuse fuse = row_fuse(pl, (char *)scratch + plan_bytes(pl, K), s);
   RowTables<K> tabs;
   MultiOut<K> out{{}, G0, beta, deff, obj};
   for (int k = 0; k < K; ++k) {
     tabs.blk[k] = blk[k];
     out.konst[k] = konst[k];
   }
-#define QPM_MG(W, M) st = launch_multi_genes<K, W, M>(gm, g, ld, pl, tabs, part, ctr, out, s)
+#define QPM_MG(W, M) st = launch_multi_genes<K, W, M>(gm, g, ld, pl, tabs, part, fuse, out, s)
   if (pl.W == MANY) {
     if (mode == ROWS_TMA) QPM_MG(MANY, ROWS_TMA);
     else QPM_MG(MANY, ROWS_TMA4);
@@ -272,7 +271,7 @@ static qpm_status launch_multi(const float2 *const *blk, const float2 *const *ko
     else QPM_MG(FEW, ROWS_TMA4);
   }
 #undef QPM_MG
-  if (st != QPM_OK || ctr) return st;
+  if (st != QPM_OK || fuse.words) return st;
   int runs = rc_runs(pl);
   const int rows = RC_THREADS / runs;
   void *args[] = {(void *)&pl, &runs, &part, &out};
@@ -325,7 +324,7 @@ extern "C" qpm_status qpm_eval_multi(const qpm_problem *probs, int32_t K, const 
     if (st != QPM_OK) return st;
   }
   const RowPlan pl = genes_plan(K, NP, N);
-  if (!scratch || scratch_bytes < plan_bytes(pl, K))
+  if (!scratch || scratch_bytes < plan_bytes(pl, K) + fuse_bytes(pl))
     return fail(QPM_ERR_ARG, "qpm_eval_multi: scratch smaller than qpm_eval_multi_scratch_bytes()");
 #define QPM_MW(KK) \
   launch_multi<KK>(blk, konst, genes, ld, pl, G0, beta, scratch, (float2 *)d_eff, objective, s)
@@ -335,5 +334,6 @@ extern "C" qpm_status qpm_eval_multi(const qpm_problem *probs, int32_t K, const 
 
 extern "C" size_t qpm_eval_multi_scratch_bytes(int32_t K, int32_t N, int32_t NP) {
   if (K < 1 || N < 1 || NP < 1) return 0;
-  return plan_bytes(genes_plan(std::min(K, (int32_t)MW_KMAX), NP, N), K);
+  const RowPlan pl = genes_plan(std::min(K, (int32_t)MW_KMAX), NP, N);
+  return plan_bytes(pl, K) + fuse_bytes(pl);
 }
