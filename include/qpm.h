@@ -153,6 +153,14 @@ int32_t qpm_abi_version(void);
  * TMA tiles; sign rows that start on 16-byte boundaries (signs 16-byte aligned,
  * ld_words a multiple of 4) are read with 16-byte accesses, others 4 bytes at a time.
  * Errors: N < 1, NP < 1, ld < N -> QPM_ERR_ARG.
+ *
+ * Stream capture: these calls, qpm_eval_shg, qpm_eval_multi and the relaxed pair may be
+ * made on a stream that is being captured.  Tables that are not there yet are then built
+ * outside the capture, before the call returns.  The graph keeps the tables and scratch of
+ * its own (one buffer per captured stream) for as long as it or an executable instance of
+ * it exists, past eviction and qpm_release_caches too, so it may be replayed on any stream
+ * and beside any other work, but not beside another instance of the same graph.  The
+ * caller's buffers, the scratch of qpm_eval_multi among them, are the caller's to keep.
  * ------------------------------------------------------------------------- */
 qpm_status qpm_eval(const qpm_problem *prob, const float *genes, int64_t ld, int32_t NP,
                     float *d_eff, float *fit, int32_t compensated, qpm_stream_t stream);
@@ -209,7 +217,8 @@ size_t qpm_eval_multi_scratch_bytes(int32_t K, int32_t N, int32_t NP);
 qpm_status qpm_eval_noalloc(const qpm_problem *prob, const float *genes, int64_t ld, int32_t NP,
                             float *d_eff, float *fit, int32_t compensated, qpm_stream_t stream);
 
-/* Free the cached phasor tables and scratch of the current device (synchronises it). */
+/* Free the cached phasor tables and scratch of the current device (synchronises it), but for
+ * what graphs still hold. */
 qpm_status qpm_release_caches(void);
 
 /* Measured issue rate of the current device for the ALU roofline (no counterpart

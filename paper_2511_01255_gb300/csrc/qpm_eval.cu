@@ -12,6 +12,7 @@
 #include <chrono>
 #include <map>
 #include <mutex>
+#include <new>
 #include <string.h>
 
 #include <string>
@@ -133,14 +134,23 @@ static __global__ void __launch_bounds__(RC_THREADS)
 
 // ------------------------------------------------------------- caches (host)
 namespace {
+// Device memory of the library that graphs may hold too: a captured call's nodes have its address
+// for as long as the graph or an executable instance of it lives, so a user object of the graph
+// counts it in `graphs`, and memory that is held is retired instead of freed.
+struct DevMem {
+  int dev = 0;
+  void *p[4] = {nullptr, nullptr, nullptr, nullptr};  // a table: phasors, partials, constants, sign blocks
+  size_t bytes = 0;                                   // scratch: of p[0]
+  unsigned long long capture = 0;                     // the last capture that took hold of it
+  cudaStream_t stream = nullptr;                      // scratch: the stream captured
+  std::atomic<int> graphs{0};
+  DevMem *next = nullptr;  // in g_kept
+};
 struct TableEntry {
-  float4 *table = nullptr;
-  double2 *part = nullptr;
-  float2 *konst = nullptr;
+  DevMem *mem = nullptr;
   cudaEvent_t ready = nullptr;
-  bool built = false;     // `ready` was seen complete: no stream needs to wait for it any more
-  float2 *blk = nullptr;  // sign-block table, built on the first packed call
-  cudaEvent_t blk_ready = nullptr;
+  bool built = false;  // `ready` was seen complete: no stream needs to wait for it any more
+  cudaEvent_t blk_ready = nullptr;  // of the sign-block table, built on the first call that needs it
   bool blk_built = false;
 };
 struct ScratchEntry {
@@ -150,18 +160,72 @@ struct ScratchEntry {
 std::mutex g_mu;
 std::map<std::tuple<int, int32_t, double, double>, TableEntry> g_tables;
 std::map<std::pair<int, cudaStream_t>, ScratchEntry> g_scratch;
+DevMem *g_kept = nullptr;  // captured calls' scratch, and tables no longer cached that graphs held
 constexpr size_t MAX_TABLES = 64;
+
+// This thread's calls that are not allowed beside a capture in the global or thread-local mode
+// (allocations, event queries; a forbidden one would end that capture) are made in the relaxed one.
+struct RelaxedMode {
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  RelaxedMode() { cudaThreadExchangeStreamCaptureMode(&mode); }
+  ~RelaxedMode() { cudaThreadExchangeStreamCaptureMode(&mode); }
+};
+
+void free_mem(DevMem *m) {
+  for (void *q : m->p)
+    if (q) cudaFree(q);
+  delete m;
+}
+
+void keep(DevMem *m) {
+  m->next = g_kept;
+  g_kept = m;
+}
+
+// the kept memory of `dev` whose graphs are all gone
+void free_unheld(int dev) {
+  for (DevMem **q = &g_kept; *q;) {
+    DevMem *m = *q;
+    if (m->dev == dev && m->graphs.load(std::memory_order_acquire) == 0) {
+      *q = m->next;
+      free_mem(m);
+    } else {
+      q = &m->next;
+    }
+  }
+}
+
+void CUDART_CB drop_hold(void *m) {  // on a thread of CUDA's: no CUDA call
+  static_cast<DevMem *>(m)->graphs.fetch_sub(1, std::memory_order_release);
+}
+
+// the capture's graph holds m from here on
+qpm_status hold(DevMem *m, const Capture &cap) {
+  if (m->capture == cap.id && m->graphs.load(std::memory_order_relaxed) > 0) return QPM_OK;
+  cudaUserObject_t obj;
+  QPM_CUDA(cudaUserObjectCreate(&obj, m, drop_hold, 1, cudaUserObjectNoDestructorSync));
+  m->graphs.fetch_add(1, std::memory_order_relaxed);
+  const cudaError_t e = cudaGraphRetainUserObject(cap.graph, obj, 1, cudaGraphUserObjectMove);
+  if (e != cudaSuccess) {
+    cudaUserObjectRelease(obj, 1);
+    return cuda_fail(e, "cudaGraphRetainUserObject");
+  }
+  m->capture = cap.id;
+  return QPM_OK;
+}
+
+void drop_entry(TableEntry &e) {
+  if (e.ready) cudaEventDestroy(e.ready);
+  if (e.blk_ready) cudaEventDestroy(e.blk_ready);
+  if (e.mem && e.mem->graphs.load(std::memory_order_acquire) > 0) keep(e.mem);
+  else if (e.mem) free_mem(e.mem);
+}
 
 qpm_status release_device_caches(int dev) {
   QPM_CUDA(cudaDeviceSynchronize());
   for (auto it = g_tables.begin(); it != g_tables.end();) {
     if (std::get<0>(it->first) == dev) {
-      cudaFree(it->second.table);
-      cudaFree(it->second.part);
-      cudaFree(it->second.konst);
-      cudaEventDestroy(it->second.ready);
-      if (it->second.blk) cudaFree(it->second.blk);
-      if (it->second.blk_ready) cudaEventDestroy(it->second.blk_ready);
+      drop_entry(it->second);
       it = g_tables.erase(it);
     } else {
       ++it;
@@ -175,6 +239,7 @@ qpm_status release_device_caches(int dev) {
       ++it;
     }
   }
+  free_unheld(dev);
   return QPM_OK;
 }
 
@@ -185,86 +250,111 @@ size_t device_table_count(int dev) {
 }
 
 // `stream` waits for `ev`, unless it was seen complete (a wait costs every call about 0.4 us of host
-// time).  Not asked while the stream is captured, where querying an event is not allowed.
-qpm_status wait_built(cudaStream_t stream, cudaEvent_t ev, bool &built) {
+// time); a captured call, which cannot wait for an event from outside its graph, waits here.
+qpm_status wait_built(cudaStream_t stream, const Capture &cap, cudaEvent_t ev, bool &built) {
   if (built) return QPM_OK;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(stream, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
-    // another thread's global-mode capture forbids queries here, and a forbidden one ends it
-    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
-    QPM_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
-    built = cudaEventQuery(ev) == cudaSuccess;
-    QPM_CUDA(cudaThreadExchangeStreamCaptureMode(&mode));
-    if (built) return QPM_OK;
+  {
+    RelaxedMode relaxed;
+    cudaError_t e = cudaEventQuery(ev);
+    if (e == cudaErrorNotReady && cap.graph) e = cudaEventSynchronize(ev);
+    built = e == cudaSuccess;
   }
+  if (built) return QPM_OK;
   cudaGetLastError();  // not ready
   QPM_CUDA(cudaStreamWaitEvent(stream, ev, 0));
   return QPM_OK;
 }
 
-// phasor table in natural order for (device, problem); built on `stream` on a miss.
-// blk (if non-NULL) receives the sign-block table, built on `stream` the first time
-// it is asked for.  Never evicts: TableLease makes room before its first lookup.
+// Runs build(stream) and records its end: on the caller's stream, `ready` behind it; in a captured
+// call on a stream outside the capture, complete on return (built; no event).
+template <class F>
+qpm_status build_table(cudaStream_t stream, const Capture &cap, cudaEvent_t *ready, bool *built, F &&build) {
+  cudaError_t e;
+  qpm_status st;
+  if (cap.graph) {
+    cudaStream_t side = nullptr;
+    QPM_CUDA(cudaStreamCreateWithFlags(&side, cudaStreamNonBlocking));
+    st = build(side);
+    e = cudaStreamSynchronize(side);
+    cudaStreamDestroy(side);
+    if (st == QPM_OK && e != cudaSuccess) st = cuda_fail(e, "building a phasor table");
+    *built = st == QPM_OK;
+    return st;
+  }
+  QPM_CUDA(cudaEventCreateWithFlags(ready, cudaEventDisableTiming));
+  st = build(stream);
+  if (st == QPM_OK && (e = cudaEventRecord(*ready, stream)) != cudaSuccess) st = cuda_fail(e, "cudaEventRecord");
+  return st;
+}
+
+// phasor table in natural order for (device, problem); built on a miss.
+// blk (if non-NULL) receives the sign-block table, built the first time it is asked for.
+// Never evicts: TableLease makes room before its first lookup.  A captured call's graph holds
+// what it is given; where the cache is full its tables are the graph's alone.
 // Caller holds g_mu.
-qpm_status get_table(const qpm_problem *p, cudaStream_t stream, const float4 **table,
+qpm_status get_table(const qpm_problem *p, cudaStream_t stream, const Capture &cap, const float4 **table,
                      const float2 **konst, const float2 **blk = nullptr) {
   int dev = 0;
   QPM_CUDA(cudaGetDevice(&dev));
   auto key = std::make_tuple(dev, p->N, p->kappa1, p->kappa2);
   auto it = g_tables.find(key);
-  if (it == g_tables.end()) {
-    TableEntry e;
+  TableEntry own;
+  const bool hit = it != g_tables.end(), cached = hit || !cap.graph || device_table_count(dev) < MAX_TABLES;
+  TableEntry &e = hit ? it->second : own;
+  if (!hit) {
+    RelaxedMode relaxed;
     const int32_t Npad = (p->N + 3) & ~3;
-    cudaError_t ce = cudaMalloc(&e.table, sizeof(float4) * (size_t)Npad);
-    if (ce == cudaSuccess) ce = cudaMalloc(&e.part, sizeof(double2) * (size_t)table_part_count(Npad));
-    if (ce == cudaSuccess) ce = cudaMalloc(&e.konst, sizeof(float2) * 4);
-    if (ce == cudaSuccess) ce = cudaEventCreateWithFlags(&e.ready, cudaEventDisableTiming);
+    e.mem = new (std::nothrow) DevMem;
+    if (!e.mem) return fail(QPM_ERR_CUDA, "out of host memory");
+    e.mem->dev = dev;
+    cudaError_t ce = cudaMalloc(&e.mem->p[0], sizeof(float4) * (size_t)Npad);
+    if (ce == cudaSuccess) ce = cudaMalloc(&e.mem->p[1], sizeof(double2) * (size_t)table_part_count(Npad));
+    if (ce == cudaSuccess) ce = cudaMalloc(&e.mem->p[2], sizeof(float2) * 4);
     qpm_status st = ce == cudaSuccess ? QPM_OK : cuda_fail(ce, "allocating a phasor table");
-    if (st == QPM_OK) {
-      TableSpec s{p->N, Npad, 1, Npad, p->kappa1, p->kappa2};
-      st = launch_table(s, e.table, e.part, e.konst, nullptr, stream);
-    }
-    if (st == QPM_OK && (ce = cudaEventRecord(e.ready, stream)) != cudaSuccess)
-      st = cuda_fail(ce, "cudaEventRecord");
+    if (st == QPM_OK)
+      st = build_table(stream, cap, &e.ready, &e.built, [&](cudaStream_t s) {
+        TableSpec ts{p->N, Npad, 1, Npad, p->kappa1, p->kappa2};
+        return launch_table(ts, (float4 *)e.mem->p[0], (double2 *)e.mem->p[1], (float2 *)e.mem->p[2],
+                            nullptr, s);
+      });
     if (st != QPM_OK) {  // the cache keeps no half-built entry
-      cudaFree(e.table);
-      cudaFree(e.part);
-      cudaFree(e.konst);
-      if (e.ready) cudaEventDestroy(e.ready);
+      drop_entry(e);
       return st;
     }
-    it = g_tables.emplace(key, e).first;
   } else {
-    const qpm_status st = wait_built(stream, it->second.ready, it->second.built);
+    const qpm_status st = wait_built(stream, cap, e.ready, e.built);
     if (st != QPM_OK) return st;
   }
-  *table = it->second.table;
-  *konst = it->second.konst;
-  if (blk) {
-    TableEntry &e = it->second;
-    if (!e.blk) {
-      const size_t nb = (size_t)(p->N + 3) / 4;
-      float2 *b = nullptr;
-      cudaEvent_t ev = nullptr;
-      QPM_CUDA(cudaMalloc(&b, sizeof(float2) * BLK_F2 * nb));
-      cudaError_t ce = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
-      qpm_status st = ce == cudaSuccess ? launch_block_table(p->N, p->kappa1, p->kappa2, b, stream)
-                                        : cuda_fail(ce, "cudaEventCreateWithFlags");
-      if (st == QPM_OK && (ce = cudaEventRecord(ev, stream)) != cudaSuccess)
-        st = cuda_fail(ce, "cudaEventRecord");
-      if (st != QPM_OK) {  // the entry keeps no half-built table
-        cudaFree(b);
-        if (ev) cudaEventDestroy(ev);
-        return st;
-      }
-      e.blk = b;
-      e.blk_ready = ev;
-    } else {
-      const qpm_status st = wait_built(stream, e.blk_ready, e.blk_built);
-      if (st != QPM_OK) return st;
+  qpm_status st = QPM_OK;
+  if (blk && !e.mem->p[3]) {
+    RelaxedMode relaxed;
+    void *b = nullptr;
+    const cudaError_t ce = cudaMalloc(&b, sizeof(float2) * BLK_F2 * ((size_t)(p->N + 3) / 4));
+    st = ce == cudaSuccess ? build_table(stream, cap, &e.blk_ready, &e.blk_built,
+                                         [&](cudaStream_t s) {
+                                           return launch_block_table(p->N, p->kappa1, p->kappa2,
+                                                                     (float2 *)b, s);
+                                         })
+                           : cuda_fail(ce, "allocating a sign-block table");
+    if (st == QPM_OK) {
+      e.mem->p[3] = b;
+    } else {  // the entry keeps no half-built table
+      if (b) cudaFree(b);
+      if (e.blk_ready) cudaEventDestroy(e.blk_ready);
+      e.blk_ready = nullptr;
     }
-    *blk = e.blk;
+  } else if (blk) {
+    st = wait_built(stream, cap, e.blk_ready, e.blk_built);
   }
+  if (st == QPM_OK && cap.graph) st = hold(e.mem, cap);
+  DevMem *const m = e.mem;
+  if (!hit && cached) g_tables.emplace(key, e);
+  else if (!hit && st == QPM_OK) keep(m);
+  else if (!hit) drop_entry(e);
+  if (st != QPM_OK) return st;
+  *table = (const float4 *)m->p[0];
+  *konst = (const float2 *)m->p[2];
+  if (blk) *blk = (const float2 *)m->p[3];
   return QPM_OK;
 }
 
@@ -279,11 +369,48 @@ qpm_status get_scratch(cudaStream_t stream, size_t bytes, void **ptr) {
       e.ptr = nullptr;
       e.bytes = 0;
     }
+    free_unheld(dev);
     QPM_CUDA(cudaMalloc(&e.ptr, bytes));
     e.bytes = bytes;
   }
   *ptr = e.ptr;
   return QPM_OK;
+}
+
+// Scratch of a captured call: never the stream's own, which later calls use and may replace.  The
+// calls captured on one stream in one capture run one after the other and share a block; other
+// captures get another, new or of graphs that are gone.
+qpm_status graph_scratch(cudaStream_t stream, const Capture &cap, size_t bytes, void **ptr) {
+  int dev = 0;
+  QPM_CUDA(cudaGetDevice(&dev));
+  DevMem *best = nullptr;
+  for (DevMem *m = g_kept; m; m = m->next) {
+    if (m->dev != dev || m->bytes < bytes) continue;
+    const bool held = m->graphs.load(std::memory_order_acquire) > 0;
+    if (held && m->capture == cap.id && m->stream == stream) {
+      *ptr = m->p[0];
+      return QPM_OK;
+    }
+    if (!held && (!best || m->bytes < best->bytes)) best = m;
+  }
+  if (!best) {
+    RelaxedMode relaxed;
+    free_unheld(dev);
+    best = new (std::nothrow) DevMem;
+    if (!best) return fail(QPM_ERR_CUDA, "out of host memory");
+    best->dev = dev;
+    const cudaError_t e = cudaMalloc(&best->p[0], bytes);
+    if (e != cudaSuccess) {
+      delete best;
+      return cuda_fail(e, "allocating the scratch of a captured call");
+    }
+    best->bytes = bytes;
+    keep(best);
+  }
+  best->stream = stream;
+  const qpm_status st = hold(best, cap);
+  if (st == QPM_OK) *ptr = best->p[0];
+  return st;
 }
 }  // namespace
 
@@ -423,19 +550,13 @@ size_t fuse_bytes(const RowPlan &pl) {
   return pl.P <= RC_FUSE ? sizeof(unsigned long long) * (size_t)RF_STRIDE * (size_t)pl.RB : 0;
 }
 
-RowFuse row_fuse(const RowPlan &pl, void *words, cudaStream_t stream) {
+RowFuse row_fuse(const RowPlan &pl, void *words, const TableLease &lease) {
   // tags count up from a start that no memory holds by chance (the clock, spread over 64 bits)
   static std::atomic<unsigned long long> tag{
       ((unsigned long long)std::chrono::steady_clock::now().time_since_epoch().count() | 1ull) *
       0x9E3779B97F4A7C15ull};
   RowFuse f;
-  if (pl.P > RC_FUSE) return f;
-  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) {
-    cudaGetLastError();
-    return f;
-  }
-  if (cap != cudaStreamCaptureStatusNone) return f;
+  if (pl.P > RC_FUSE || lease.captured()) return f;
   f.words = (unsigned long long *)words;
   f.tag = tag.fetch_add(1, std::memory_order_relaxed) & (~0ull >> RF_BITS);
   return f;
@@ -449,16 +570,16 @@ static qpm_status eval_common(const qpm_problem *prob, const void *src, int64_t 
   if (prob->N > (1 << 28)) return fail(QPM_ERR_UNSUPPORTED, "qpm_eval: N too large");
   if (kind == 2 ? (ld < (prob->N + 31) / 32) : (ld < prob->N))
     return fail(QPM_ERR_ARG, "qpm_eval: leading dimension smaller than the row");
-  TableLease lease(prob, 1);  // held until the launches below are enqueued
+  TableLease lease(prob, 1, stream);  // held until the launches below are enqueued
   const float2 *konst, *blk = nullptr;
-  qpm_status st = lease.block_table(prob, stream, &blk, &konst);
+  qpm_status st = lease.block_table(prob, &blk, &konst);
   if (st != QPM_OK) return st;
   if (NP > EVAL_MAX_ROWS) return fail(QPM_ERR_UNSUPPORTED, "qpm_eval: too many rows");
   const int W = kind == 2 ? (NP <= 64 ? 2 : 8) : 0;
   const RowPlan pl = kind == 2 ? packed_plan(NP, prob->N, W) : genes_plan(1, NP, prob->N);
   void *scratch;
   const size_t partials = plan_bytes(pl, 1);
-  st = get_scratch(stream, partials + (kind == 2 ? 0 : fuse_bytes(pl)), &scratch);
+  st = lease.scratch(partials + (kind == 2 ? 0 : fuse_bytes(pl)), &scratch);
   if (st != QPM_OK) return st;
   float2 *part = (float2 *)scratch;
   EvalOut out{RowFuse{}, konst, (float2 *)d_eff, fit};
@@ -469,7 +590,7 @@ static qpm_status eval_common(const qpm_problem *prob, const void *src, int64_t 
                 : launch_packed<2>(vecw, comp != 0, (const uint32_t *)src, ld, pl, tabs, part, stream);
     return st != QPM_OK ? st : launch_combine(pl, part, out, stream);
   }
-  out.fuse = row_fuse(pl, (char *)scratch + partials, stream);
+  out.fuse = row_fuse(pl, (char *)scratch + partials, lease);
   return launch_eval_rows(comp != 0, (const float *)src, ld, pl, blk, part, out, stream);
 }
 
@@ -567,7 +688,7 @@ extern "C" qpm_status qpm_eval_noalloc(const qpm_problem *prob, const float *gen
                           EvalOut{RowFuse{}, konst, (float2 *)d_eff, fit}, s);
 }
 
-qpm::TableLease::TableLease(const qpm_problem *problems, int count) {
+qpm::TableLease::TableLease(const qpm_problem *problems, int count, cudaStream_t stream) : stream_(stream) {
   g_mu.lock();
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
@@ -575,6 +696,17 @@ qpm::TableLease::TableLease(const qpm_problem *problems, int count) {
     st_ = cuda_fail(e, "cudaGetDevice");
     return;
   }
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  // (the query refuses the legacy stream beside another's capture: the launches will say so)
+  if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) cudaGetLastError();
+  else if (cap != cudaStreamCaptureStatusNone)
+    e = cudaStreamGetCaptureInfo(stream, &cap, &cap_.id, &cap_.graph, nullptr, nullptr, nullptr);
+  if (e != cudaSuccess || cap == cudaStreamCaptureStatusInvalidated) {
+    st_ = e != cudaSuccess ? cuda_fail(e, "cudaStreamGetCaptureInfo")
+                           : fail(QPM_ERR_CUDA, "the stream's capture has been invalidated");
+    return;
+  }
+  if (cap_.graph) return;  // a captured call evicts nothing: it must not wait for the device
   size_t misses = 0;
   for (int k = 0; k < count; ++k) {
     const qpm_problem &p = problems[k];
@@ -590,17 +722,20 @@ qpm::TableLease::TableLease(const qpm_problem *problems, int count) {
 
 qpm::TableLease::~TableLease() { g_mu.unlock(); }
 
-qpm_status qpm::TableLease::table(const qpm_problem *p, cudaStream_t stream, const float4 **table,
-                                  const float2 **konst) {
+qpm_status qpm::TableLease::table(const qpm_problem *p, const float4 **table, const float2 **konst) {
   if (st_ != QPM_OK) return st_;
-  return get_table(p, stream, table, konst);
+  return get_table(p, stream_, cap_, table, konst);
 }
 
-qpm_status qpm::TableLease::block_table(const qpm_problem *p, cudaStream_t stream,
-                                        const float2 **blk, const float2 **konst) {
+qpm_status qpm::TableLease::block_table(const qpm_problem *p, const float2 **blk, const float2 **konst) {
   if (st_ != QPM_OK) return st_;
   const float4 *table;
-  return get_table(p, stream, &table, konst, blk);
+  return get_table(p, stream_, cap_, &table, konst, blk);
+}
+
+qpm_status qpm::TableLease::scratch(size_t bytes, void **ptr) {
+  if (st_ != QPM_OK) return st_;
+  return cap_.graph ? graph_scratch(stream_, cap_, bytes, ptr) : get_scratch(stream_, bytes, ptr);
 }
 
 extern "C" qpm_status qpm_eval(const qpm_problem *prob, const float *genes, int64_t ld,

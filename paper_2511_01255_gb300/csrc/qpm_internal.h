@@ -58,22 +58,31 @@ constexpr int BLK_F2 = 24;  // float2 per block of 4 domains
 // MAX_TABLES problems per device; a lease that will look up `problems` distinct
 // problems makes room for all of them when it is created (freeing every table of
 // the device once, after a device synchronisation), never between two lookups.
+// Where the stream is being captured, what the lease gives out stays valid for as long as the
+// capture's graph, or an executable instance of it, lives.
+struct Capture {
+  cudaGraph_t graph = nullptr;  // NULL: the stream is not being captured
+  unsigned long long id = 0;
+};
 class TableLease {
  public:
-  TableLease(const qpm_problem *problems, int count);
+  TableLease(const qpm_problem *problems, int count, cudaStream_t stream);
   ~TableLease();
   TableLease(const TableLease &) = delete;
   TableLease &operator=(const TableLease &) = delete;
   // status of the set-up (a failed eviction is reported by the first lookup)
   qpm_status status() const { return st_; }
-  // natural-order phasor table and FP32 constants; built on `stream` on a miss
-  qpm_status table(const qpm_problem *p, cudaStream_t stream, const float4 **table,
-                   const float2 **konst);
-  // the same entry's sign-block table (built on `stream` the first time) and constants
-  qpm_status block_table(const qpm_problem *p, cudaStream_t stream, const float2 **blk,
-                         const float2 **konst);
+  bool captured() const { return cap_.graph != nullptr; }
+  // natural-order phasor table and FP32 constants; built on a miss
+  qpm_status table(const qpm_problem *p, const float4 **table, const float2 **konst);
+  // the same entry's sign-block table (built the first time) and constants
+  qpm_status block_table(const qpm_problem *p, const float2 **blk, const float2 **konst);
+  // scratch for one call's launches: the stream's, or the captured graph's own
+  qpm_status scratch(size_t bytes, void **ptr);
 
  private:
+  cudaStream_t stream_;
+  Capture cap_;
   qpm_status st_ = QPM_OK;
 };
 
@@ -104,7 +113,7 @@ struct RowFuse {
 };
 // the plan's fused combination with the words at `words` (fuse_bytes): none where a row has many
 // pieces or the call is captured (a replay would find its own tag)
-RowFuse row_fuse(const RowPlan &pl, void *words, cudaStream_t stream);
+RowFuse row_fuse(const RowPlan &pl, void *words, const TableLease &lease);
 size_t fuse_bytes(const RowPlan &pl);
 constexpr int EVAL_MAX_ROWS = 128 * 65535;  // rows a call of the row sweeps takes
 // bytes of the plan's partial monoids for K problems

@@ -247,7 +247,7 @@ static qpm_status launch_multi_genes(const GeneMaps &gm, const float *g, int64_t
 template <int K>
 static qpm_status launch_multi(const float2 *const *blk, const float2 *const *konst, const float *g,
                                int64_t ld, const RowPlan &pl, float G0, float beta, void *scratch,
-                               float2 *deff, float *obj, cudaStream_t s) {
+                               float2 *deff, float *obj, const TableLease &lease, cudaStream_t s) {
   constexpr int MANY = K == 1 ? 4 : 8, FEW = K == 1 ? 1 : 2;  // genes_plan's warps per CTA
   GeneMaps gm;
   int mode;
@@ -255,7 +255,7 @@ static qpm_status launch_multi(const float2 *const *blk, const float2 *const *ko
   if (st != QPM_OK) return st;
   float2 *part = (float2 *)scratch;
   // partials and words are the caller's: calls with scratch of their own stay independent
-  const RowFuse fuse = row_fuse(pl, (char *)scratch + plan_bytes(pl, K), s);
+  const RowFuse fuse = row_fuse(pl, (char *)scratch + plan_bytes(pl, K), lease);
   RowTables<K> tabs;
   MultiOut<K> out{{}, G0, beta, deff, obj};
   for (int k = 0; k < K; ++k) {
@@ -289,10 +289,10 @@ extern "C" qpm_status qpm_eval_shg(const qpm_problem *prob, const float *genes, 
   if (prob->N < 1 || NP < 1) return fail(QPM_ERR_ARG, "qpm_eval_shg: need N >= 1 and NP >= 1");
   if (ld < prob->N) return fail(QPM_ERR_ARG, "qpm_eval_shg: leading dimension smaller than the row");
   cudaStream_t s = (cudaStream_t)stream;
-  TableLease lease(prob, 1);  // held until the launch below is enqueued
+  TableLease lease(prob, 1, s);  // held until the launch below is enqueued
   const float4 *table;
   const float2 *konst;
-  qpm_status st = lease.table(prob, s, &table, &konst);
+  qpm_status st = lease.table(prob, &table, &konst);
   if (st != QPM_OK) return st;
   const bool vec = (ld % 4 == 0) && (((uintptr_t)genes & 15) == 0) && prob->N >= 4;
   const int rpc = (NP + sm_count() - 1) / sm_count(), grid = (NP + rpc - 1) / rpc;
@@ -318,16 +318,16 @@ extern "C" qpm_status qpm_eval_multi(const qpm_problem *probs, int32_t K, const 
   if (NP > EVAL_MAX_ROWS) return fail(QPM_ERR_UNSUPPORTED, "qpm_eval_multi: too many rows");
   // one lease for all K lookups and the launches: room for the K tables is made
   // before the first lookup, so no lookup can evict a table returned before it
-  TableLease lease(probs, K);
+  TableLease lease(probs, K, s);
   for (int k = 0; k < K; ++k) {
-    qpm_status st = lease.block_table(&probs[k], s, &blk[k], &konst[k]);
+    qpm_status st = lease.block_table(&probs[k], &blk[k], &konst[k]);
     if (st != QPM_OK) return st;
   }
   const RowPlan pl = genes_plan(K, NP, N);
   if (!scratch || scratch_bytes < plan_bytes(pl, K) + fuse_bytes(pl))
     return fail(QPM_ERR_ARG, "qpm_eval_multi: scratch smaller than qpm_eval_multi_scratch_bytes()");
 #define QPM_MW(KK) \
-  launch_multi<KK>(blk, konst, genes, ld, pl, G0, beta, scratch, (float2 *)d_eff, objective, s)
+  launch_multi<KK>(blk, konst, genes, ld, pl, G0, beta, scratch, (float2 *)d_eff, objective, lease, s)
   return K == 1 ? QPM_MW(1) : K == 2 ? QPM_MW(2) : K == 3 ? QPM_MW(3) : QPM_MW(4);
 #undef QPM_MW
 }
