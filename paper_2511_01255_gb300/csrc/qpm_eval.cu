@@ -159,7 +159,10 @@ struct ScratchEntry {
 };
 std::mutex g_mu;
 std::map<std::tuple<int, int32_t, double, double>, TableEntry> g_tables;
-std::map<std::pair<int, cudaStream_t>, ScratchEntry> g_scratch;
+// per (device, stream, thread's stream): the handle cudaStreamPerThread names another stream in each
+// thread, which its id tells apart (0 for the others)
+std::map<std::tuple<int, cudaStream_t, unsigned long long>, ScratchEntry> g_scratch;
+constexpr size_t MAX_THREADS = 64;  // threads whose scratch is kept per device
 DevMem *g_kept = nullptr;  // captured calls' scratch, and tables no longer cached that graphs held
 constexpr size_t MAX_TABLES = 64;
 
@@ -221,6 +224,18 @@ void drop_entry(TableEntry &e) {
   else if (e.mem) free_mem(e.mem);
 }
 
+// frees the scratch of `dev`, of its per-thread streams only if so asked (the device is idle)
+void drop_scratch(int dev, bool threads_only) {
+  for (auto it = g_scratch.begin(); it != g_scratch.end();) {
+    if (std::get<0>(it->first) == dev && (!threads_only || std::get<2>(it->first) != 0)) {
+      cudaFree(it->second.ptr);
+      it = g_scratch.erase(it);
+    } else {
+      ++it;
+    }
+  }
+}
+
 qpm_status release_device_caches(int dev) {
   QPM_CUDA(cudaDeviceSynchronize());
   for (auto it = g_tables.begin(); it != g_tables.end();) {
@@ -231,14 +246,7 @@ qpm_status release_device_caches(int dev) {
       ++it;
     }
   }
-  for (auto it = g_scratch.begin(); it != g_scratch.end();) {
-    if (it->first.first == dev) {
-      cudaFree(it->second.ptr);
-      it = g_scratch.erase(it);
-    } else {
-      ++it;
-    }
-  }
+  drop_scratch(dev, false);
   free_unheld(dev);
   return QPM_OK;
 }
@@ -361,7 +369,17 @@ qpm_status get_table(const qpm_problem *p, cudaStream_t stream, const Capture &c
 qpm_status get_scratch(cudaStream_t stream, size_t bytes, void **ptr) {
   int dev = 0;
   QPM_CUDA(cudaGetDevice(&dev));
-  ScratchEntry &e = g_scratch[std::make_pair(dev, stream)];
+  unsigned long long id = 0;
+  if (stream == cudaStreamPerThread) {
+    QPM_CUDA(cudaStreamGetId(stream, &id));
+    size_t n = 0;
+    for (const auto &kv : g_scratch) n += std::get<0>(kv.first) == dev && std::get<2>(kv.first) != 0;
+    if (n >= MAX_THREADS && !g_scratch.count(std::make_tuple(dev, stream, id))) {
+      QPM_CUDA(cudaDeviceSynchronize());
+      drop_scratch(dev, true);
+    }
+  }
+  ScratchEntry &e = g_scratch[std::make_tuple(dev, stream, id)];
   if (e.bytes < bytes) {
     if (e.ptr) {
       QPM_CUDA(cudaStreamSynchronize(stream));
