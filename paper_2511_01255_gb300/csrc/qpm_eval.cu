@@ -715,7 +715,9 @@ qpm::TableLease::TableLease(const qpm_problem *problems, int count, cudaStream_t
     return;
   }
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  // (the query refuses the legacy stream beside another's capture: the launches will say so)
+  // The query also makes the device's context current in a thread that has made no CUDA call yet:
+  // a call that finds its tables and scratch makes no other before it encodes tensor maps, which
+  // needs one.  (It refuses the legacy stream beside another's capture: the launches will say so.)
   if (cudaStreamIsCapturing(stream, &cap) != cudaSuccess) cudaGetLastError();
   else if (cap != cudaStreamCaptureStatusNone)
     e = cudaStreamGetCaptureInfo(stream, &cap, &cap_.id, &cap_.graph, nullptr, nullptr, nullptr);

@@ -75,3 +75,42 @@ def test_many_threads_one_after_the_other(q):
         t.join()
         torch.cuda.synchronize()
         assert torch.equal(D, ref)
+
+
+@pytest.mark.parametrize("ld", [512, 513])
+@pytest.mark.parametrize("kind", ["eval", "packed", "multi", "shg", "relaxed"])
+def test_first_cuda_call_of_a_thread(q, kind, ld):
+    """A thread whose first CUDA call is one of the library's, with every table and buffer there."""
+    import torch
+    N, NP = 512, 200
+    X = torch.from_numpy(np.random.default_rng(ld).uniform(-1, 1, (NP, ld)).astype(np.float32)).cuda()[:, :N]
+    words = torch.arange(NP * 16, dtype=torch.int32, device="cuda").view(NP, 16)
+    D, f, M = (torch.empty(s, device="cuda") for s in ((NP, 2), (NP,), (NP, 2, 2)))
+    S, g, one = q.relaxed_saved(NP, N), torch.empty((NP, ld), device="cuda")[:, :N], torch.ones(NP, device="cuda")
+    L, kaps = q.lib(), (q.Problem * 2)((N, K1, K2), (N, K1 * 1.01, K2))
+    need = L.qpm_eval_multi_scratch_bytes(2, N, NP)
+    scratch = torch.empty(need, dtype=torch.uint8, device="cuda")
+    ptr = [t.data_ptr() for t in (X, words, D, f, M, S, g, one, scratch)]
+    x, w, d, fp, m, s, gp, o, sc = ptr
+    calls = {  # through the C entries: the tensors' own checks make CUDA calls
+        "eval": lambda: L.qpm_eval(kaps, x, ld, NP, d, fp, 0, None),
+        "packed": lambda: L.qpm_eval_packed(kaps, w, 16, NP, d, fp, 0, None),
+        "multi": lambda: L.qpm_eval_multi(kaps, 2, x, ld, NP, 1e4, 0.5, m, fp, sc, need, None),
+        "shg": lambda: L.qpm_eval_shg(kaps, x, ld, NP, d, fp, None),
+        "relaxed": lambda: (L.qpm_deff_relaxed_fwd(kaps, x, ld, NP, d, fp, s, None) or
+                            L.qpm_deff_relaxed_bwd(kaps, x, ld, NP, d, s, o, gp, ld, None))}
+    outs = {"multi": [M, f], "relaxed": [D, f, g]}.get(kind, [D, f])
+    for _ in range(2):
+        assert calls[kind]() == 0
+        torch.cuda.synchronize()
+    ref, got = [t.clone() for t in outs], []
+    for t in outs:
+        t.fill_(float("nan"))
+    torch.cuda.synchronize()
+    t = threading.Thread(target=lambda: got.append((calls[kind](), L.qpm_last_error())))
+    t.start()
+    t.join()
+    torch.cuda.synchronize()
+    assert got[0][0] == 0, got
+    for a, b in zip(outs, ref):
+        assert torch.equal(a, b)
