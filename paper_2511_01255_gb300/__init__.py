@@ -357,6 +357,9 @@ def qpm_eval_multi(N, kappas, genes, G0, beta, objective, d_eff=None, stream=Non
     L = lib()
     nbytes = L.qpm_eval_multi_scratch_bytes(K, N, NP)
     scratch = torch.empty(max(1, nbytes), dtype=torch.uint8, device=genes.device)
+    if stream is not None:  # freed on return here, used there
+        scratch.record_stream(stream if isinstance(stream, torch.cuda.Stream) else
+                              torch.cuda.ExternalStream(stream.cuda_stream, device=genes.device))
     _check(L.qpm_eval_multi(probs, K, genes.data_ptr(), ld, NP, float(G0), float(beta), d, o,
                             scratch.data_ptr(), nbytes, _stream(stream)))
 

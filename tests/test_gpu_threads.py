@@ -114,3 +114,27 @@ def test_first_cuda_call_of_a_thread(q, kind, ld):
     assert got[0][0] == 0, got
     for a, b in zip(outs, ref):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("plain", [False, True])
+def test_multi_scratch_lives_until_its_stream_is_done(q, plain):
+    """qpm_eval_multi's scratch comes from the current stream's pool and is used on `stream`: memory
+    of the same size taken on the current stream meanwhile is other memory."""
+    import torch
+    N, NP, K = 100000, 512, 2
+    kaps = [(K1, K2), (K1 * 1.01, K2)]
+    X = torch.empty((NP, N), device="cuda").uniform_(-1, 1, generator=torch.Generator("cuda").manual_seed(3))
+    D, f = torch.empty((NP, K, 2), device="cuda"), torch.empty(NP, device="cuda")
+    q.qpm_eval_multi(N, kaps, X, 1e5, 0.5, f, D)
+    torch.cuda.synchronize()
+    ref, need = D.clone(), q.lib().qpm_eval_multi_scratch_bytes(K, N, NP)
+    side = torch.cuda.Stream()
+    s = SimpleNamespace(cuda_stream=side.cuda_stream) if plain else side  # any object with the handle
+    for _ in range(20):
+        torch.cuda.synchronize()
+        for _ in range(4):
+            q.qpm_eval_multi(N, kaps, X, 1e5, 0.5, f, D, stream=s)
+        for _ in range(30):
+            torch.empty(need, dtype=torch.uint8, device="cuda").fill_(255)
+        torch.cuda.synchronize()
+        assert torch.equal(D, ref)
