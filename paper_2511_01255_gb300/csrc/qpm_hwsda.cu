@@ -2341,6 +2341,11 @@ static TableJob table_job(const InstDev &I) {
   return TableJob{{I.N, I.Npad, I.T, I.c, I.kappa1, I.kappa2}, I.table, I.tpart, I.konst, I.konst64};
 }
 
+// A copy from pageable memory may return before its last bytes are on the device, and the streams
+// that read the descriptors next (qpm_init of many instances, the batched form) need not wait for
+// the legacy stream it ran on.
+static cudaError_t descriptors_landed() { return cudaStreamSynchronize(nullptr); }
+
 static qpm_status check_state(qpm_state *st, int gens) {
   if (!st) return fail(QPM_ERR_ARG, "NULL state");
   if (!st->inited) return fail(QPM_ERR_STATE, "qpm_init has not been called");
@@ -2571,6 +2576,7 @@ extern "C" qpm_status qpm_create(const qpm_problem *probs, const qpm_params *par
     for (int k = 0; k < n_inst; ++k) jobs[k] = table_job(st->h[k]);
     if (e == cudaSuccess)
       e = cudaMemcpy(st->d_jobs, jobs.data(), sizeof(TableJob) * n_inst, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = descriptors_landed();
     if (e != cudaSuccess) { cudaFree(st->arena); delete st; return cuda_fail(e, "cudaMemcpy"); }
     int maxpad = 0;
     for (int k = 0; k < n_inst; ++k) {
@@ -2601,6 +2607,7 @@ extern "C" qpm_status qpm_set_trace(qpm_state *st, int32_t inst, float *trace) {
     st->graph_n = -1;
   }
   cudaError_t e = cudaMemcpy(st->d_insts + inst, &st->h[inst], sizeof(InstDev), cudaMemcpyHostToDevice);
+  if (e == cudaSuccess) e = descriptors_landed();
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy(descriptor)");
   return QPM_OK;
 }
@@ -2908,6 +2915,7 @@ extern "C" qpm_status qpm_set_objective(qpm_state *st, int32_t inst, const qpm_o
   QPM_CUDA(cudaMemcpy(st->d_insts + inst, &I, sizeof(InstDev), cudaMemcpyHostToDevice));
   const TableJob job = table_job(I);
   QPM_CUDA(cudaMemcpy(st->d_jobs + inst, &job, sizeof(TableJob), cudaMemcpyHostToDevice));
+  QPM_CUDA(descriptors_landed());
   return QPM_OK;
 }
 
