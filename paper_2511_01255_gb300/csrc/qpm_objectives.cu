@@ -36,13 +36,17 @@ namespace qpm {
 static constexpr int SHG_WARPS = 16;
 static constexpr int SHG_Q = 2;                 // 128-domain pieces per segment
 static constexpr int SHG_SEG = 128 * SHG_Q;
-static constexpr int SHG_RB = 4;                // rows per item
+static constexpr int SHG_RB = 4;                // rows per item; 1 where a CTA has one row
 static constexpr int SHG_RMAX = 64;             // rows whose sums are kept at a time
 
 // VEC: rows of 16-byte aligned groups, lane l takes domains 4 l .. 4 l + 3 of a piece with one
 // load; else lane l takes domains l, l + 32, l + 64, l + 96, so that every load of a warp is 128
 // contiguous bytes whatever the rows' alignment.
-template <bool VEC>
+// RB: rows per item.  A CTA with one row (up to as many rows as SMs) takes items of one: repeating
+// that row four times cost the loads and sums of four, and since each of its items is another
+// segment, the phasors come with the genes an item ahead (a row of 1e5 domains: 51 us with items of
+// four rows, 32 for the form before them, 30 now; 15 unaligned).  The order of the sums is the same.
+template <bool VEC, int RB>
 static __global__ void __launch_bounds__(SHG_WARPS * 32, 1)
     k_shg(const float *__restrict__ genes, int64_t ld, int NP, int N, int rows_per_cta,
           const float4 *__restrict__ table, const float2 *__restrict__ konst,
@@ -55,7 +59,7 @@ static __global__ void __launch_bounds__(SHG_WARPS * 32, 1)
   const int nseg = (N + SHG_SEG - 1) / SHG_SEG;
   const int glast = 4 * (N >> 2) - 4;  // the row's last whole group (VEC: N >= 4)
   for (int64_t rs = (int64_t)blockIdx.x * rows_per_cta; rs < rend; rs += SHG_RMAX) {
-    const int r0 = (int)rs, rn = min(SHG_RMAX, rend - r0), nrb = (rn + SHG_RB - 1) / SHG_RB;
+    const int r0 = (int)rs, rn = min(SHG_RMAX, rend - r0), nrb = (rn + RB - 1) / RB;
     for (int e = threadIdx.x; e < SHG_WARPS * 2 * SHG_RMAX; e += SHG_WARPS * 32)
       (&sums[0][0])[e] = (&comp[0][0])[e] = 0.f;
     __syncthreads();
@@ -67,11 +71,18 @@ static __global__ void __launch_bounds__(SHG_WARPS * 32, 1)
     auto dom = [&](int sg, int k, int q) {
       return sg * SHG_SEG + 128 * k + (VEC ? 4 * lane + q : lane + 32 * q);
     };
-    float4 x[SHG_RB][SHG_Q], y[SHG_RB][SHG_Q];  // this item's genes, the next one's in flight
+    float4 x[RB][SHG_Q], y[RB][SHG_Q];  // this item's genes, the next one's in flight
+    float2 pn[SHG_Q * 4];               // RB 1: the next item's phasors
     auto fetch = [&]() {
+      if (RB == 1) {
 #pragma unroll
-      for (int r = 0; r < SHG_RB; ++r) {
-        const int row = min(r0 + nrb_x * SHG_RB + r, rend - 1);  // a repeated row's sums are dropped
+        for (int k = 0; k < SHG_Q; ++k)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) pn[4 * k + q] = __ldg((const float2 *)(table + min(dom(nseg_x, k, q), N - 1)));
+      }
+#pragma unroll
+      for (int r = 0; r < RB; ++r) {
+        const int row = min(r0 + nrb_x * RB + r, rend - 1);  // a repeated row's sums are dropped
         const float *g = genes + (int64_t)row * ld;
 #pragma unroll
         for (int k = 0; k < SHG_Q; ++k) {
@@ -96,24 +107,30 @@ static __global__ void __launch_bounds__(SHG_WARPS * 32, 1)
     bool fresh = true;
     for (int64_t it = i0; it < i1; ++it) {
 #pragma unroll
-      for (int r = 0; r < SHG_RB; ++r)
+      for (int r = 0; r < RB; ++r)
 #pragma unroll
         for (int k = 0; k < SHG_Q; ++k) x[r][k] = y[r][k];
+      if (RB == 1) {
+#pragma unroll
+        for (int k = 0; k < SHG_Q; ++k)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) p[4 * k + q] = dom(seg, k, q) < N ? pn[4 * k + q] : make_float2(0.f, 0.f);
+      }
       if (it + 1 < i1) fetch();
       if (VEC && (N & 3) != 0 && (seg + 1) * SHG_SEG > N) {  // the row's last, partial group
 #pragma unroll
         for (int k = 0; k < SHG_Q; ++k) {
           if (dom(seg, k, 0) == glast + 4) {
 #pragma unroll
-            for (int r = 0; r < SHG_RB; ++r) {
-              const float *g = genes + (int64_t)min(r0 + rb * SHG_RB + r, rend - 1) * ld;
+            for (int r = 0; r < RB; ++r) {
+              const float *g = genes + (int64_t)min(r0 + rb * RB + r, rend - 1) * ld;
               x[r][k] = make_float4(__ldg(g + dom(seg, k, 0)), __ldg(g + min(dom(seg, k, 1), N - 1)),
                                     __ldg(g + min(dom(seg, k, 2), N - 1)), 0.f);
             }
           }
         }
       }
-      if (fresh) {
+      if (RB > 1 && fresh) {
 #pragma unroll
         for (int k = 0; k < SHG_Q; ++k)
 #pragma unroll
@@ -123,9 +140,9 @@ static __global__ void __launch_bounds__(SHG_WARPS * 32, 1)
           }
         fresh = false;
       }
-      float v[2 * SHG_RB];  // (re, im) of the 4 rows' partial sums
+      float v[2 * RB];  // (re, im) of the rows' partial sums
 #pragma unroll
-      for (int r = 0; r < SHG_RB; ++r) {
+      for (int r = 0; r < RB; ++r) {
         float sx = 0.f, sy = 0.f;
 #pragma unroll
         for (int k = 0; k < SHG_Q; ++k) {
@@ -141,9 +158,10 @@ static __global__ void __launch_bounds__(SHG_WARPS * 32, 1)
         v[2 * r + 1] = sy;
       }
       // 8 values over 32 lanes: three halving exchanges leave lane l the value l / 4 summed
-      // over 8 lanes, two more steps sum the rest
+      // over 8 lanes, two more steps sum the rest (2 values: one exchange, four steps)
+      constexpr int G = 16 / RB;  // lanes per value
 #pragma unroll
-      for (int w = SHG_RB, o = 16; w >= 1; w >>= 1, o >>= 1) {
+      for (int w = RB, o = 16; w >= 1; w >>= 1, o >>= 1) {
         const bool up = (lane & o) != 0;
 #pragma unroll
         for (int e = 0; e < w; ++e) {
@@ -152,10 +170,10 @@ static __global__ void __launch_bounds__(SHG_WARPS * 32, 1)
         }
       }
       float t = v[0];
-      t += __shfl_xor_sync(0xffffffffu, t, 2);
-      t += __shfl_xor_sync(0xffffffffu, t, 1);
-      if ((lane & 3) == 0 && rb * SHG_RB + (lane >> 3) < rn) {
-        const int e = 2 * SHG_RB * rb + (lane >> 2);
+#pragma unroll
+      for (int o = G / 2; o >= 1; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+      if (lane % G == 0 && rb * RB + lane / (2 * G) < rn) {
+        const int e = 2 * RB * rb + lane / G;
         kahan_add(sums[warp][e], comp[warp][e], t);
       }
       if (++rb == nrb) {
@@ -298,8 +316,9 @@ extern "C" qpm_status qpm_eval_shg(const qpm_problem *prob, const float *genes, 
   const int rpc = (NP + sm_count() - 1) / sm_count(), grid = (NP + rpc - 1) / rpc;
   float2 *e = (float2 *)e_shg;
   void *args[] = {(void *)&genes, &ld, &NP, (void *)&prob->N, (void *)&rpc, (void *)&table, (void *)&konst, &e, &fit};
-  return launch_dependent(vec ? (const void *)k_shg<true> : (const void *)k_shg<false>, dim3(grid),
-                          dim3(SHG_WARPS * 32), args, 0, s);
+  const void *fn = rpc == 1 ? (vec ? (const void *)k_shg<true, 1> : (const void *)k_shg<false, 1>)
+                            : (vec ? (const void *)k_shg<true, SHG_RB> : (const void *)k_shg<false, SHG_RB>);
+  return launch_dependent(fn, dim3(grid), dim3(SHG_WARPS * 32), args, 0, s);
 }
 
 extern "C" qpm_status qpm_eval_multi(const qpm_problem *probs, int32_t K, const float *genes,

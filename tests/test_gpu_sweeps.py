@@ -140,3 +140,18 @@ def test_captured_rows_same_bits(q, N, NP, K):
         g.replay()
         torch.cuda.synchronize()
         assert torch.equal(D, ref)
+
+
+# up to as many rows as SMs a CTA has one row; from 64 rows per CTA on it keeps its sums in passes
+@pytest.mark.parametrize("NP", ["sms", "sms+1", "64sms+5"])
+@pytest.mark.parametrize("N,off", [(260, 0), (259, 1), (1030, 0)])
+def test_shg_rows_per_cta(q, orc, NP, N, off):
+    import torch
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    NP = {"sms": sms, "sms+1": sms + 1, "64sms+5": 64 * sms + 5}[NP]
+    view, X = rows_of(NP, N, N, off, N + NP)
+    E, f = torch.full((NP, 2), float("nan"), device="cuda"), torch.empty(NP, device="cuda")
+    q.qpm_eval_shg(N, K1, view, E, f)
+    E = E.cpu().numpy()
+    ref = orc.shg_genes(X, K1)
+    assert (np.abs(E[:, 0] + 1j * E[:, 1] - ref) / np.maximum(np.abs(ref), 1e-3 * N)).max() < TOL_D
