@@ -432,6 +432,12 @@ qpm_status graph_scratch(cudaStream_t stream, const Capture &cap, size_t bytes, 
 }
 }  // namespace
 
+// a row block of nunit units touches at most this many runs of floor(units / C) or more units
+static int row_pieces(const RowPlan &p) {
+  const int64_t q = std::max<int64_t>(1, (int64_t)p.RB * p.nunit / p.C);
+  return (int)std::min<int64_t>(std::min<int64_t>(p.nunit, p.C), (p.nunit + q - 1) / q + 1);
+}
+
 RowPlan row_plan(int NP, int N, int W, int slots, int gran, int maxsub, int min_units) {
   RowPlan p;
   p.NP = NP;
@@ -449,9 +455,7 @@ RowPlan row_plan(int NP, int N, int W, int slots, int gran, int maxsub, int min_
   int64_t C = std::max<int64_t>(1, rounds) * full;
   C = std::min(C, std::max<int64_t>(1, tot / min_units));
   p.C = (int)C;
-  // a row block of nunit units touches at most this many runs of floor(tot / C) or more units
-  const int64_t q = std::max<int64_t>(1, tot / C);
-  p.P = (int)std::min<int64_t>(std::min<int64_t>(p.nunit, C), (p.nunit + q - 1) / q + 1);
+  p.P = row_pieces(p);
   return p;
 }
 
@@ -465,9 +469,21 @@ static int genes_warps(int K, int NP) {
   };
   return alive(few) > alive(many) ? few : many;
 }
-RowPlan genes_plan(int K, int NP, int N, bool whole) {
+RowPlan genes_plan(int K, int NP, int N, bool aligned, bool whole) {
   const int W = genes_warps(K, NP);
-  if (!whole) return row_plan(NP, N, W, rs_ctas(K, W), 1, RS_MAXSUB, 4);
+  if (!whole) {
+    RowPlan p = row_plan(NP, N, W, rs_ctas(K, W), 1, RS_MAXSUB, 4);
+    // Whole rounds of CTAs, all in step, lose to runs of the full length where a few row blocks of
+    // very long aligned rows need three rounds or more (one table): 256 x 1e6 215 us against 194,
+    // 512 x 600000 232 / 208, 128 x 2e6 220 / 196, 64 x 3e6 179 / 165, 512 x 1e6 363 / 372.  Not with
+    // rows of odd pitch (256 x 1e6 185 / 212), more row blocks (1024 x 250000 168 / 184) or two rounds
+    // (1024 x 131072 89 / 110).
+    if (K == 1 && aligned && p.RB <= 4 && p.C > 2 * rs_ctas(K, W) * sm_count()) {
+      p.C = p.RB * ((p.nunit + RS_MAXSUB - 1) / RS_MAXSUB);
+      p.P = row_pieces(p);
+    }
+    return p;
+  }
   // runs of whole rows, cut only where a row is longer than a run may be
   const int nsub = (N + 31) / 32, runs = (nsub + RS_MAXSUB - 1) / RS_MAXSUB;
   RowPlan p = row_plan(NP, N, W, 1, (nsub + runs - 1) / runs, nsub, 1);
@@ -596,7 +612,8 @@ static qpm_status eval_common(const qpm_problem *prob, const void *src, int64_t 
   if (st != QPM_OK) return st;
   if (NP > EVAL_MAX_ROWS) return fail(QPM_ERR_UNSUPPORTED, "qpm_eval: too many rows");
   const int W = kind == 2 ? (NP <= 64 ? 2 : 8) : 0;
-  const RowPlan pl = kind == 2 ? packed_plan(NP, prob->N, W) : genes_plan(1, NP, prob->N);
+  const RowPlan pl = kind == 2 ? packed_plan(NP, prob->N, W)
+                               : genes_plan(1, NP, prob->N, rows_aligned((const float *)src, NP, ld));
   void *scratch;
   const size_t partials = plan_bytes(pl, 1);
   st = lease.scratch(partials + (kind == 2 ? 0 : fuse_bytes(pl)), &scratch);
@@ -675,10 +692,11 @@ extern "C" qpm_status qpm_eval_noalloc(const qpm_problem *prob, const float *gen
     return fail(QPM_ERR_ARG, "qpm_eval_noalloc: N above 2^28 or NP above 2^26");
   if (NP > EVAL_MAX_ROWS) return fail(QPM_ERR_UNSUPPORTED, "qpm_eval_noalloc: too many rows");
   const int32_t Npad = (prob->N + 3) & ~3;
-  RowPlan pl = genes_plan(1, NP, prob->N);
+  const bool aligned = rows_aligned(genes, NP, ld);
+  RowPlan pl = genes_plan(1, NP, prob->N, aligned);
   size_t need = noalloc_bytes(prob->N, pl);
   if (need > NOALLOC_SCRATCH_BYTES) {  // rows split no further than the longest run needs
-    pl = genes_plan(1, NP, prob->N, true);
+    pl = genes_plan(1, NP, prob->N, aligned, true);
     need = noalloc_bytes(prob->N, pl);
   }
   if (need > NOALLOC_SCRATCH_BYTES)

@@ -101,9 +101,13 @@ struct RowPlan {
 // slots: resident CTAs per SM; gran: sub-steps per unit; maxsub: longest run; min_units: no run
 // shorter than this while CTAs are left idle
 RowPlan row_plan(int NP, int N, int W, int slots, int gran, int maxsub, int min_units);
-// the plan of the float-gene sweep with K sign-block tables; whole: no row is split unless it
-// is longer than a run may be (fewest pieces)
-RowPlan genes_plan(int K, int NP, int N, bool whole = false);
+// the plan of the float-gene sweep with K sign-block tables; aligned: see rows_aligned; whole: no
+// row is split unless it is longer than a run may be (fewest pieces)
+RowPlan genes_plan(int K, int NP, int N, bool aligned, bool whole = false);
+// all rows start on 16-byte boundaries
+inline bool rows_aligned(const float *genes, int NP, int64_t ld) {
+  return ((uintptr_t)genes & 15) == 0 && (NP == 1 || ld % 4 == 0);
+}
 // What a sweep that combines its rows itself counts arrivals with (rows_last): a word per row block
 // behind the call's partials, whatever it holds before the call, and the call's own tag, which
 // no other call of the process has

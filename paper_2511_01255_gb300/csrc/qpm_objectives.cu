@@ -344,7 +344,7 @@ extern "C" qpm_status qpm_eval_multi(const qpm_problem *probs, int32_t K, const 
     qpm_status st = lease.block_table(&probs[k], &blk[k], &konst[k]);
     if (st != QPM_OK) return st;
   }
-  const RowPlan pl = genes_plan(K, NP, N);
+  const RowPlan pl = genes_plan(K, NP, N, rows_aligned(genes, NP, ld));
   if (!scratch || scratch_bytes < plan_bytes(pl, K) + fuse_bytes(pl))
     return fail(QPM_ERR_ARG, "qpm_eval_multi: scratch smaller than qpm_eval_multi_scratch_bytes()");
 #define QPM_MW(KK) \
@@ -355,6 +355,10 @@ extern "C" qpm_status qpm_eval_multi(const qpm_problem *probs, int32_t K, const 
 
 extern "C" size_t qpm_eval_multi_scratch_bytes(int32_t K, int32_t N, int32_t NP) {
   if (K < 1 || N < 1 || NP < 1) return 0;
-  const RowPlan pl = genes_plan(std::min(K, (int32_t)MW_KMAX), NP, N);
-  return plan_bytes(pl, K) + fuse_bytes(pl);
+  size_t bytes = 0;
+  for (const bool aligned : {false, true}) {
+    const RowPlan pl = genes_plan(std::min(K, (int32_t)MW_KMAX), NP, N, aligned);
+    bytes = std::max(bytes, plan_bytes(pl, K) + fuse_bytes(pl));
+  }
+  return bytes;
 }

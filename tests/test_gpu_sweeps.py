@@ -155,3 +155,20 @@ def test_shg_rows_per_cta(q, orc, NP, N, off):
     E = E.cpu().numpy()
     ref = orc.shg_genes(X, K1)
     assert (np.abs(E[:, 0] + 1j * E[:, 1] - ref) / np.maximum(np.abs(ref), 1e-3 * N)).max() < TOL_D
+
+
+# few row blocks of rows long enough for three rounds of CTAs: aligned rows take runs of the full
+# length instead, rows of odd pitch whole rounds; K = 1 of the multi-wavelength call splits alike
+@pytest.mark.parametrize("N,NP,ld", [(2900000, 33, 2900000), (2900000, 33, 2900001)])
+def test_long_rows(q, orc, N, NP, ld):
+    import torch
+    buf = torch.empty((NP, ld), device="cuda").uniform_(-1, 1, generator=torch.Generator("cuda").manual_seed(5))
+    X = buf[:, :N]
+    D, M, f = (torch.full(s, float("nan"), device="cuda") for s in ((NP, 2), (NP, 1, 2), (NP,)))
+    q.qpm_eval(N, K1, K2, X, D)
+    q.qpm_eval_multi(N, [(K1, K2)], X, 1e5, 0.5, f, M)
+    torch.cuda.synchronize()
+    assert torch.equal(D, M[:, 0])
+    rows = [0, 31, 32]
+    ref = orc.deff_closed_genes(X[rows].cpu().numpy(), K1, K2)
+    assert deff_err(D[rows].cpu().numpy(), ref, N).max() < TOL_D
