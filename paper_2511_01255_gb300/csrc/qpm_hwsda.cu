@@ -67,6 +67,7 @@ struct InstDev {
   // first one's table and constants are table / konst), G0, beta; minimised for the
   // multi-wavelength kinds
   int32_t obj, K, minimize;
+  int32_t wide;          // launches form: the kernels of 112 registers a thread, not 80 (occupancy)
   const uint32_t *dthr;  // [G][7] discrete GWO (combine 2): social, flip, plus[0..4] thresholds
   float G0, beta;
   const float4 *mtab[8];   // [Npad] permuted phasor tables of the K problems
@@ -1137,12 +1138,16 @@ __device__ bool last_cta(unsigned *ctr) {
 // The multi-wavelength kinds (MK) stage the rows only: their K phasor tables are read
 // through L1, which keeps them (the rows bypass it).
 //
-// Registers: 80 a thread keep three 256-thread CTAs on an SM (N = 12000, NP = 1000, graph form:
-// 134-138 us per generation; with 72 registers 139, with 64 149).  Launch bounds of 512 threads
-// let the compiler take 128 and halve the CTAs of short rows (discrete GWO 110 against 94 us at
-// N = 2331).  The K scans of MK need 128, for CTAs of up to 512 threads.
-template <bool COMP, bool DUAL, int MK = 0>
-static __global__ void __maxnreg__(MK ? 128 : 80) k_de(InstDev I) {
+// WIDE: 112 registers a thread instead of 80; `occupancy` picks the form.  Two 256-thread CTAs an SM
+// instead of three, but no spills and more loads in flight.  Long rows are faster so (us per
+// generation, graph form, 112 against 80: N = 12000, NP = 1000 123 / 131, compensated 124 / 133; 3300 x
+// 1000 in teams of 128 60 / 68, compensated 62 / 70; 4000 x 500 35.4 / 37.7; 1e5 x 1024 782 / 801); the
+// short rows of DUAL and the discrete GWO where it costs them no round of individuals (1320 x 5000,
+// 17 rounds for 11: 102 / 92, discrete 120 / 101; discrete 1000 x 1000 in teams of 128, 2 rounds each:
+// 29.6 / 34.0).  72 and 64 registers are slower throughout.  The K scans of MK take 128 (96: 3 % slower
+// at K = 4 cascaded problems, 10-35 % at K = 8 SHG ones).
+template <bool COMP, bool DUAL, int MK = 0, bool WIDE = true>
+static __global__ void __maxnreg__(MK ? 128 : WIDE ? 112 : 80) k_de(InstDev I) {
   constexpr bool STG = !DUAL, TSS = MK != 0;
   extern __shared__ float4 dyn[];
   float4 *stg = dyn;
@@ -1187,8 +1192,8 @@ static __global__ void __maxnreg__(MK ? 128 : 80) k_de(InstDev I) {
   }
 }
 
-template <bool COMP, bool DUAL, int MK = 0>
-static __global__ void __maxnreg__(MK ? 128 : 80) k_gwo(InstDev I) {
+template <bool COMP, bool DUAL, int MK = 0, bool WIDE = true>
+static __global__ void __maxnreg__(MK ? 128 : WIDE ? 112 : 80) k_gwo(InstDev I) {
   constexpr bool STG = !DUAL, TSS = MK != 0;
   extern __shared__ float4 dyn[];
   float4 *stg = dyn;
@@ -1365,8 +1370,8 @@ static __global__ void __launch_bounds__(512, 1) k_gwo_mt(InstDev I) {
 }
 
 // Steps 4-5 with the four-leader discrete GWO (launches form)
-template <bool COMP>
-static __global__ void __maxnreg__(80) k_gwo_disc(InstDev I) {
+template <bool COMP, bool WIDE>
+static __global__ void __maxnreg__(WIDE ? 112 : 80) k_gwo_disc(InstDev I) {
   extern __shared__ float4 dyn[];
   Mono *sh = (Mono *)dyn;
   const int g = *I.gen;
@@ -2160,11 +2165,15 @@ struct Variant {
 static constexpr int TS_MAX_NPAD = 4096;  // phasor table in shared memory up to 64 KB
 static constexpr size_t BATCH_TS_MAX_BYTES = 160 * 1024;  // batched form: table in smem up to 160 KB
 
-template <bool COMP, bool DUAL>
-static Variant variant2(const InstDev &I) {
+// rows short enough to be read from both of an individual's slots before its slot is known (DUAL)
+static bool short_rows(const InstDev &I) { return I.c <= 8; }
+
+template <bool COMP, bool DUAL, bool WIDE>
+static Variant variant3(const InstDev &I) {
   Variant v;
-  v.de = (const void *)k_de<COMP, DUAL>;
-  v.gwo = (const void *)k_gwo<COMP, DUAL>;
+  v.de = (const void *)k_de<COMP, DUAL, 0, WIDE>;
+  v.gwo = I.combine == 2 ? (const void *)k_gwo_disc<COMP, WIDE>  // the discrete GWO: its own kernel
+                         : (const void *)k_gwo<COMP, DUAL, 0, WIDE || !DUAL>;
   // k_de / k_gwo read the table from global memory: long rows stage rows and table
   v.smem = (DUAL ? 0 : sizeof(float4) * stg_f4_per_thread(false) * (size_t)I.T) + smem_bytes(I.T);
   const bool wide = I.T > 256;
@@ -2181,6 +2190,12 @@ static Variant variant2(const InstDev &I) {
     v.persist_smem = stg + smem_bytes(I.T);
   }
   return v;
+}
+
+template <bool COMP>
+static Variant variant2(const InstDev &I) {
+  if (short_rows(I)) return I.wide ? variant3<COMP, true, true>(I) : variant3<COMP, true, false>(I);
+  return I.wide ? variant3<COMP, false, true>(I) : variant3<COMP, false, false>(I);
 }
 
 // the multi-wavelength kinds: launches form only, rows staged; their K tables in shared
@@ -2238,12 +2253,7 @@ static Variant variant_multi(const InstDev &I) {
 static Variant variant_of(const InstDev &I) {
   if (I.obj == OBJ_MULTI_THG) return variant_multi<OBJ_MULTI_THG>(I);
   if (I.obj == OBJ_MULTI_SHG) return variant_multi<OBJ_MULTI_SHG>(I);
-  const bool dual = I.c <= 8;
-  Variant v = I.compensated ? (dual ? variant2<true, true>(I) : variant2<true, false>(I))
-                            : (dual ? variant2<false, true>(I) : variant2<false, false>(I));
-  if (I.combine == 2)  // the discrete GWO (launches form): its own GWO kernel
-    v.gwo = I.compensated ? (const void *)k_gwo_disc<true> : (const void *)k_gwo_disc<false>;
-  return v;
+  return I.compensated ? variant2<true>(I) : variant2<false>(I);
 }
 
 // the shared-memory attribute of a persistent variant is the same for every
@@ -2290,19 +2300,38 @@ static qpm_status batch_grid(const qpm_state *st, int cs, int *grid) {
   return QPM_OK;
 }
 
-static qpm_status occupancy(const InstDev &I, int *plain, int *persist) {
+static qpm_status plain_occupancy(const InstDev &I, int *plain) {
   const Variant v = variant_of(I);
-  int a = 0, a2 = 0, b = 0;
-  QPM_CUDA(cudaFuncSetAttribute(v.persist, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)persist_smem_cap(I.Npad <= TS_MAX_NPAD)));
+  int a = 0, b = 0;
   // the largest dynamic shared memory any instance's k_de / k_gwo can need
   const int plain_cap = (int)(sizeof(float4) * stg_f4_per_thread(false) * 512 + smem_bytes(512));
   QPM_CUDA(cudaFuncSetAttribute(v.de, cudaFuncAttributeMaxDynamicSharedMemorySize, plain_cap));
   QPM_CUDA(cudaFuncSetAttribute(v.gwo, cudaFuncAttributeMaxDynamicSharedMemorySize, plain_cap));
   QPM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, v.de, I.T, v.smem));
-  QPM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a2, v.gwo, I.T, v.smem));
+  QPM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, v.gwo, I.T, v.smem));
+  *plain = std::max(1, std::min(a, b));
+  return QPM_OK;
+}
+
+// resident CTAs per SM of the plain and the persistent kernels; sets I.wide
+static qpm_status occupancy(InstDev &I, int *plain, int *persist) {
+  int wide = 0, narrow = 0;
+  I.wide = 1;
+  qpm_status r = plain_occupancy(I, &wide);
+  if (r != QPM_OK) return r;
+  *plain = wide;
+  if (short_rows(I) || I.combine == 2) {  // 112 registers where that is no more rounds of individuals
+    I.wide = 0;
+    if ((r = plain_occupancy(I, &narrow)) != QPM_OK) return r;
+    auto rounds = [&](int occ) { return (I.NP + occ * sm_count() - 1) / (occ * sm_count()); };
+    I.wide = rounds(wide) <= rounds(narrow);
+    *plain = I.wide ? wide : narrow;
+  }
+  const Variant v = variant_of(I);
+  int b = 0;
+  QPM_CUDA(cudaFuncSetAttribute(v.persist, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)persist_smem_cap(I.Npad <= TS_MAX_NPAD)));
   QPM_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, v.persist, I.T, v.persist_smem));
-  *plain = std::max(1, std::min(a, a2));
   *persist = std::max(1, b);
   return QPM_OK;
 }
@@ -2447,6 +2476,7 @@ extern "C" qpm_status qpm_create(const qpm_problem *probs, const qpm_params *par
         I.T = W.T;
         I.Npad = W.Npad;
         I.c = W.c;
+        I.wide = W.wide;
         occ_plain = wp;
         occ_persist = wq;
       }
