@@ -251,7 +251,7 @@ qpm_status qpm_measure_latency(int32_t kind, int32_t ctas, double *ns_out, qpm_s
 
 /* Exhaustive self-check of one of the library's arithmetic shortcuts against
  * the plain operation it replaces (no counterpart in the paper), over all 2^32
- * 32-bit patterns x:
+ * 32-bit patterns x (kinds 0 and 1 work on pairs: x in either half):
  *   kind 0: the GWO mean's division by 3 (Markstein's residual correction of
  *           x * RN(1/3)) against the IEEE division x / 3 (two NaNs agree);
  *   kind 1: the GWO's r1 and 2 r2 built in the significand of a float above 2^23 and

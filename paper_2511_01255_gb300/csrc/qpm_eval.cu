@@ -459,7 +459,7 @@ RowPlan row_plan(int NP, int N, int W, int slots, int gran, int maxsub, int min_
   return p;
 }
 
-// Warps per CTA.  One table: 4 (12 warps an SM in 3 CTAs); a single group of rows: 1 (6 warps an
+// Warps per CTA.  One table: 4 (12 warps an SM in 3 CTAs); a single group of rows: 1 (5 warps an
 // SM, where 4 would keep 3 alive).  K tables: 8 warps share the staged steps (8 warps an SM),
 // or 2 where that keeps more warps alive (few row groups).
 static int genes_warps(int K, int NP) {

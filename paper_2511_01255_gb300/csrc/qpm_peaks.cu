@@ -97,17 +97,18 @@ static __global__ void __launch_bounds__(PK_THREADS) k_peak_philox(uint2 key, ui
   if (s == 0x2545F491u && key.x == 0u) sink[blockIdx.x] = s;
 }
 
-// every float bit pattern x: div3_rn(x) against the IEEE division x / 3 (bitwise;
-// two NaNs agree); per-thread counts and first bad pattern, one atomic each
+// every float bit pattern x, in either half of a pair with another value: div3_rn2 against the
+// IEEE division x / 3 (bitwise; two NaNs agree); per-thread counts and first bad pattern, one
+// atomic each
 static __global__ void k_check_div3(unsigned long long *bad, uint32_t *first) {
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   unsigned long long n = 0;
   uint32_t f = 0xFFFFFFFFu;
   for (uint64_t b = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; b < (1ull << 32); b += stride) {
     const float x = __uint_as_float((uint32_t)b);
-    const float q = div3_rn2(f2_pack(1.0f, x)).y, ref = __fdiv_rn(x, 3.0f);
-    const bool same = __float_as_uint(q) == __float_as_uint(ref) || (q != q && ref != ref);
-    if (!same) {
+    const float ref = __fdiv_rn(x, 3.0f);
+    auto same = [&](float q) { return __float_as_uint(q) == __float_as_uint(ref) || (q != q && ref != ref); };
+    if (!same(div3_rn2(f2_pack(x, 1.0f)).x) || !same(div3_rn2(f2_pack(1.0f, x)).y)) {
       ++n;
       f = min(f, (uint32_t)b);
     }
@@ -118,8 +119,8 @@ static __global__ void k_check_div3(unsigned long long *bad, uint32_t *first) {
   }
 }
 
-// every 32-bit word w: the GWO's r1 and 2 r2 built in the significand against the
-// same values through conversions, r = (16-bit half) 2^-16 (bitwise)
+// every 32-bit word w, in either half of a pair with another: the GWO's r1 and 2 r2 built in the
+// significand against the same values through conversions, r = (16-bit half) 2^-16 (bitwise)
 static __global__ void k_check_gwo_uniforms(unsigned long long *bad, uint32_t *first) {
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   unsigned long long n = 0;
@@ -128,9 +129,10 @@ static __global__ void k_check_gwo_uniforms(unsigned long long *bad, uint32_t *f
     const uint32_t w = (uint32_t)b;
     const float r1 = __fmul_rn(__uint2float_rn(w >> 16), 0x1p-16f);
     const float r2 = __fmul_rn(__uint2float_rn(w & 0xFFFFu), 0x1p-16f);
-    const bool same = __float_as_uint(f2_unpack(u16hi2(w, ~w)).x) == __float_as_uint(r1) &&
-                      __float_as_uint(f2_unpack(twice_u16lo2(~w, w)).y) == __float_as_uint(__fmul_rn(2.0f, r2));
-    if (!same) {
+    const float c = __fmul_rn(2.0f, r2);
+    auto same = [](float a, float b) { return __float_as_uint(a) == __float_as_uint(b); };
+    if (!same(f2_unpack(u16hi2(w, ~w)).x, r1) || !same(f2_unpack(u16hi2(~w, w)).y, r1) ||
+        !same(f2_unpack(twice_u16lo2(w, ~w)).x, c) || !same(f2_unpack(twice_u16lo2(~w, w)).y, c)) {
       ++n;
       f = min(f, w);
     }

@@ -72,3 +72,20 @@ def test_many_instances_start_like_single_launches(q):
         for k in range(4):
             for a, b in zip(got[k], st.population(k)):
                 assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("sizes", [[(100, 5), (257, 64), (1000, 7), (3300, 33)], [(8000, 4), (129, 70)]])
+def test_many_instances_of_mixed_sizes_start_like_single_launches(q, sizes):
+    """Tables of several and of unequal numbers of CTAs, several domain groups per thread."""
+    import torch
+    n = len(sizes)
+    probs = [(N, K1 + 0.01 * k, K2) for k, (N, _) in enumerate(sizes)]
+    prms = [q.Params(NP, 2, 0.5, 0.9, 3 + k, 0, k % 2, 32, 0) for k, (_, NP) in enumerate(sizes)]
+    with q.State(probs, prms) as st:
+        st.init()
+        got = [[a.clone() for a in st.population(k) + st.best(k)] for k in range(n)]
+    with q.State(probs + [(64, K1, K2)], prms + [q.Params(8, 2, 0.5, 0.9, 3, 0, 0, 64, 0)]) as st:
+        st.init()
+        for k in range(n):
+            for a, b in zip(got[k], st.population(k) + st.best(k)):
+                assert torch.equal(a, b)
