@@ -201,3 +201,25 @@ def test_batched_adaptive_F_lockstep(q, orc):
         else:
             assert np.all(Fg == np.float32(0.5))
     st.close()
+
+
+@pytest.mark.parametrize("extra", [[], [(12000, 2 * math.pi / 7.1, 2 * math.pi / 1.6, 9, 0, 0)]])
+def test_batched_seeds_of_their_own(q, extra):
+    """Instances of different seeds run the kernel that builds each one's round keys (tables in
+    shared memory, or one instance too long for it): the launches form's populations."""
+    import torch
+    inst = INSTANCES + extra
+    pops = []
+    for mode, ctas in ((q.RUN_LAUNCHES, 1), (q.RUN_BATCHED, 1), (q.RUN_BATCHED, 4)):
+        st = q.State([(N, k1, k2) for N, k1, k2, _, _, _ in inst],
+                     [q.Params(NP, 5, 0.5, 0.9, 100 + 7 * k, comb, comp)
+                      for k, (_, _, _, NP, comp, comb) in enumerate(inst)])
+        st.set_batch_cluster(ctas)
+        st.init()
+        st.run(5, mode)
+        torch.cuda.synchronize()
+        pops.append([st.population(k)[0].cpu().numpy() for k in range(len(inst))])
+        st.close()
+    for other in pops[1:]:
+        for a, b in zip(pops[0], other):
+            assert np.array_equal(a, b)
