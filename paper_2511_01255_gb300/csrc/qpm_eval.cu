@@ -30,14 +30,14 @@ namespace qpm {
 // 64 rows).
 constexpr int ep_ctas(int W) { return W == 8 ? 3 : 8; }
 
-// float genes: see rows_sweep; FUSE: the sweep combines the rows itself
-template <int W, int MODE, bool COMP, bool FUSE>
+// float genes: see rows_sweep; words in `fuse`: the sweep combines the rows itself
+template <int W, int MODE, bool COMP>
 static __global__ void __launch_bounds__(W * 32, rs_ctas(1, W))
     k_eval_genes(const __grid_constant__ GeneMaps maps, const float *__restrict__ src, int64_t ld,
                  RowPlan pl, RowTables<1> tabs, float2 *part, RowFuse fuse,
                  const float2 *__restrict__ konst, float2 *__restrict__ deff,
                  float *__restrict__ fit) {
-  rows_sweep<1, W, MODE, COMP, FUSE>(maps, src, ld, pl, tabs, part, fuse, [&](int row, const Mono *m) {
+  rows_sweep<1, W, MODE, COMP>(maps, src, ld, pl, tabs, part, fuse, [&](int row, const Mono *m) {
     const float2 D = deff_from(m[0], konst[0], konst[1]);
     deff[row] = D;
     if (fit) fit[row] = fit_of(D);
@@ -521,12 +521,12 @@ struct EvalOut {
   float *fit;
 };
 
-template <int W, int MODE, bool COMP, bool FUSE>
+template <int W, int MODE, bool COMP>
 static qpm_status launch_genes(const GeneMaps &gm, const float *g, int64_t ld, const RowPlan &pl,
                                const RowTables<1> &tabs, float2 *part, const EvalOut &out,
                                cudaStream_t stream) {
   static SmemAttr attr;
-  const void *fn = (const void *)k_eval_genes<W, MODE, COMP, FUSE>;
+  const void *fn = (const void *)k_eval_genes<W, MODE, COMP>;
   const qpm_status st = attr.set(fn, rs_smem(1, W));
   if (st != QPM_OK) return st;
   void *args[] = {(void *)&gm, (void *)&g, (void *)&ld, (void *)&pl, (void *)&tabs, (void *)&part,
@@ -553,10 +553,9 @@ static qpm_status launch_eval_rows(bool comp, const float *g, int64_t ld, const 
   qpm_status st = make_gene_maps(&gm, &mode, g, pl.NP, pl.N, ld);
   if (st != QPM_OK) return st;
   const RowTables<1> tabs{{blk}};
-#define QPM_EGF(WW, M, F)                                                          \
-  (comp ? launch_genes<WW, M, true, F>(gm, g, ld, pl, tabs, part, out, stream)     \
-        : launch_genes<WW, M, false, F>(gm, g, ld, pl, tabs, part, out, stream))
-#define QPM_EG(WW, M) st = out.fuse.words ? QPM_EGF(WW, M, true) : QPM_EGF(WW, M, false)
+#define QPM_EG(WW, M)                                                       \
+  st = comp ? launch_genes<WW, M, true>(gm, g, ld, pl, tabs, part, out, stream) \
+            : launch_genes<WW, M, false>(gm, g, ld, pl, tabs, part, out, stream)
   if (pl.W == 4) {
     if (mode == ROWS_TMA) QPM_EG(4, ROWS_TMA);
     else QPM_EG(4, ROWS_TMA4);
@@ -565,7 +564,6 @@ static qpm_status launch_eval_rows(bool comp, const float *g, int64_t ld, const 
     else QPM_EG(1, ROWS_TMA4);
   }
 #undef QPM_EG
-#undef QPM_EGF
   if (st != QPM_OK || out.fuse.words) return st;
   return launch_combine(pl, part, out, stream);
 }

@@ -228,11 +228,11 @@ __device__ __forceinline__ void multi_close(const MultiOut<K> &o, int row, const
 
 // The qpm_eval sweep with K sign-block tables: for K = 1 the same split and order, so it
 // reproduces qpm_eval's plain scan bit for bit.
-template <int K, int W, int MODE, bool FUSE>
+template <int K, int W, int MODE>
 static __global__ void __launch_bounds__(W * 32, rs_ctas(K, W))
     k_multi_genes(const __grid_constant__ GeneMaps maps, const float *__restrict__ src, int64_t ld,
                   RowPlan pl, RowTables<K> tabs, float2 *part, RowFuse fuse, MultiOut<K> out) {
-  rows_sweep<K, W, MODE, false, FUSE>(maps, src, ld, pl, tabs, part, fuse,
+  rows_sweep<K, W, MODE, false>(maps, src, ld, pl, tabs, part, fuse,
                                 [&](int row, const Mono *m) { multi_close<K>(out, row, m); });
 }
 
@@ -249,12 +249,12 @@ static __global__ void __launch_bounds__(RC_THREADS)
   if (run == 0 && row < pl.NP) multi_close<K>(out, row, acc);
 }
 
-template <int K, int W, int MODE, bool FUSE>
+template <int K, int W, int MODE>
 static qpm_status launch_multi_genes(const GeneMaps &gm, const float *g, int64_t ld, const RowPlan &pl,
                                      const RowTables<K> &tabs, float2 *part, const RowFuse &fuse,
                                      const MultiOut<K> &out, cudaStream_t s) {
   static SmemAttr attr;
-  const void *fn = (const void *)k_multi_genes<K, W, MODE, FUSE>;
+  const void *fn = (const void *)k_multi_genes<K, W, MODE>;
   const qpm_status st = attr.set(fn, rs_smem(K, W));
   if (st != QPM_OK) return st;
   void *args[] = {(void *)&gm, (void *)&g, (void *)&ld, (void *)&pl, (void *)&tabs, (void *)&part,
@@ -280,9 +280,7 @@ static qpm_status launch_multi(const float2 *const *blk, const float2 *const *ko
     tabs.blk[k] = blk[k];
     out.konst[k] = konst[k];
   }
-#define QPM_MG(W, M)                                                                             \
-  st = fuse.words ? launch_multi_genes<K, W, M, true>(gm, g, ld, pl, tabs, part, fuse, out, s)   \
-                  : launch_multi_genes<K, W, M, false>(gm, g, ld, pl, tabs, part, fuse, out, s)
+#define QPM_MG(W, M) st = launch_multi_genes<K, W, M>(gm, g, ld, pl, tabs, part, fuse, out, s)
   if (pl.W == MANY) {
     if (mode == ROWS_TMA) QPM_MG(MANY, ROWS_TMA);
     else QPM_MG(MANY, ROWS_TMA4);

@@ -220,9 +220,9 @@ static_assert(RC_FUSE < (1 << RF_BITS), "the count must not run into the tag");
 // every CTA, before its piece, sets a word without the tag to (tag, 0), once for all of them
 // whoever comes first, and after it adds 1.  So a call on another stream, one that was captured and
 // never replayed, or memory never written cannot disturb the count, as they would one that has to
-// start at 0.  The look waits together with the piece's table entries and the arrival is one round
-// trip to L2: compensated 5000 x 1000 per call 8.0 us, 7.7 with a counter that starts at 0, 8.4 with
-// a flag per piece and a look at all of them after it, 11.1 with the arrival by compare-and-swap.
+// start at 0.  The look costs nothing (it waits together with the piece's table entries) and the
+// arrival is one round trip to L2.  (The whole of it after the piece, by compare-and-swap or by a
+// flag per piece and a look at all of them: 10.8 and 8.1 us for a call of 5000 x 1000, 7.2 so.)
 __device__ __forceinline__ unsigned long long rows_look(const unsigned long long *word) {
   unsigned long long w;
   asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(word) : "memory");
@@ -282,10 +282,9 @@ __device__ __forceinline__ void fused_combine(const RowPlan &pl, const float2 *p
 // registers behind one CTA barrier per step.  A wait on an mbarrier is bounded (%globaltimer);
 // one that runs out makes the rows' results NaN and stops the warp's copies.
 // Partials: part[((piece K + k) 3 + {A, B, C}) NPpad + row].
-// FUSE (a form of its own, whose combination takes it from 126 to 156 registers with one table and
-// from 150 to 255 with three; with a plan of at most RC_FUSE pieces a row): the CTA that completes a row block, found by
+// fuse (with a plan of at most RC_FUSE pieces a row): the CTA that completes a row block, found by
 // the block's word (rows_last), combines it and calls close(row, the K monoids).
-template <int K, int W, int MODE, bool COMP, bool FUSE, class Close>
+template <int K, int W, int MODE, bool COMP, class Close>
 __device__ __forceinline__ void rows_sweep(const GeneMaps &maps, const float *__restrict__ src,
                                            int64_t ld, const RowPlan &pl, const RowTables<K> &tabs,
                                            float2 *part, const RowFuse &fuse, Close &&close) {
@@ -360,14 +359,14 @@ __device__ __forceinline__ void rows_sweep(const GeneMaps &maps, const float *__
       }
     }
     unsigned long long word = 0;
-    if (FUSE && threadIdx.x == 0) word = rows_look(fuse.words + (size_t)b * RF_STRIDE);
+    if (fuse.words && threadIdx.x == 0) word = rows_look(fuse.words + (size_t)b * RF_STRIDE);
     __syncthreads();  // the table buffers of the piece before are free
 #pragma unroll
     for (int p = 0; p < K; ++p) {
       R[p].store(tab + p * RS_TAB);
       if (nsteps > 1) R[p].load(tabs.blk[p], (m0 >> 2) + 32, nb);
     }
-    if (FUSE && threadIdx.x == 0) rows_open(fuse.words + (size_t)b * RF_STRIDE, fuse.tag, word);
+    if (fuse.words && threadIdx.x == 0) rows_open(fuse.words + (size_t)b * RF_STRIDE, fuse.tag, word);
     RowAcc<COMP> acc[K];
 #pragma unroll
     for (int p = 0; p < K; ++p) acc[p].zero();
@@ -441,7 +440,7 @@ __device__ __forceinline__ void rows_sweep(const GeneMaps &maps, const float *__
         o[2 * (size_t)pl.NPpad] = m.C;
       }
     }
-    if constexpr (FUSE) {
+    if (fuse.words) {
       const int P = rp_pieces(pl, b);
       if (rows_last(fuse.words + (size_t)b * RF_STRIDE, P)) fused_combine<K>(pl, part, P, b * W * 32 + (int)threadIdx.x, close);
     }
