@@ -146,7 +146,7 @@ int32_t qpm_abi_version(void);
  * The per-problem phasor table is built on first use of (device, N, kappa1,
  * kappa2) and cached by the library (library-owned device memory, released by
  * qpm_release_caches); the scan's partial results use a library-owned scratch
- * buffer grown on demand.  The cache holds at most 64 problems per device: a call
+ * buffer per stream, allocated on the stream's first call and grown on demand.  The cache holds at most 64 problems per device: a call
  * that needs room for new problems first synchronises the device and frees all of
  * that device's tables and scratch (never while another host thread's call is
  * between its table lookup and its launches).  Gene rows of any alignment are read as
@@ -178,8 +178,9 @@ qpm_status qpm_eval_packed(const qpm_problem *prob, const uint32_t *signs, int64
  *   to be minimised, for K <= 4 problems of equal N sharing one read of the
  *   genes.  d_eff device float2 [NP][K] (may be NULL), objective device float [NP].
  *   scratch: caller-owned device memory of at least
- *   qpm_eval_multi_scratch_bytes(K, N, NP) bytes, 8-byte aligned (the rows' partial sums
- *   and the words that count them; it may hold anything before the call).
+ *   qpm_eval_multi_scratch_bytes(K, N, NP) bytes, 8-byte aligned (the rows' partial sums;
+ *   it may hold anything before the call).  Calls on different streams with scratch of their own are
+ *   independent.  The library adds a 16 KB buffer of its own per stream (see qpm_eval).
  * Phasor tables as for qpm_eval.  Errors: K outside [1, 4], unequal N, N < 1,
  * NP < 1, ld < N, small scratch -> QPM_ERR_ARG.
  * ------------------------------------------------------------------------- */

@@ -9,7 +9,6 @@
 
 #include <algorithm>
 #include <atomic>
-#include <chrono>
 #include <map>
 #include <mutex>
 #include <new>
@@ -30,14 +29,14 @@ namespace qpm {
 // 64 rows).
 constexpr int ep_ctas(int W) { return W == 8 ? 3 : 8; }
 
-// float genes: see rows_sweep; words in `fuse`: the sweep combines the rows itself
+// float genes: see rows_sweep; ctr not NULL: the sweep combines the rows itself
 template <int W, int MODE, bool COMP>
 static __global__ void __launch_bounds__(W * 32, rs_ctas(1, W))
     k_eval_genes(const __grid_constant__ GeneMaps maps, const float *__restrict__ src, int64_t ld,
-                 RowPlan pl, RowTables<1> tabs, float2 *part, RowFuse fuse,
+                 RowPlan pl, RowTables<1> tabs, float2 *part, unsigned *ctr,
                  const float2 *__restrict__ konst, float2 *__restrict__ deff,
                  float *__restrict__ fit) {
-  rows_sweep<1, W, MODE, COMP>(maps, src, ld, pl, tabs, part, fuse, [&](int row, const Mono *m) {
+  rows_sweep<1, W, MODE, COMP>(maps, src, ld, pl, tabs, part, ctr, [&](int row, const Mono *m) {
     const float2 D = deff_from(m[0], konst[0], konst[1]);
     deff[row] = D;
     if (fit) fit[row] = fit_of(D);
@@ -154,13 +153,14 @@ struct TableEntry {
   bool blk_built = false;
 };
 struct ScratchEntry {
-  void *ptr = nullptr;
+  void *ptr = nullptr;  // FUSE_BLOCKS counters, then partial sums
   size_t bytes = 0;
 };
 std::mutex g_mu;
 std::map<std::tuple<int, int32_t, double, double>, TableEntry> g_tables;
 // per (device, stream, thread's stream): the handle cudaStreamPerThread names another stream in each
-// thread, which its id tells apart (0 for the others)
+// thread, which its id tells apart (0 for the others: a destroyed stream's handle does not come back
+// before its work is done)
 std::map<std::tuple<int, cudaStream_t, unsigned long long>, ScratchEntry> g_scratch;
 constexpr size_t MAX_THREADS = 64;  // threads whose scratch is kept per device
 DevMem *g_kept = nullptr;  // captured calls' scratch, and tables no longer cached that graphs held
@@ -300,10 +300,8 @@ qpm_status build_table(cudaStream_t stream, const Capture &cap, cudaEvent_t *rea
 // Never evicts: TableLease makes room before its first lookup.  A captured call's graph holds
 // what it is given; where the cache is full its tables are the graph's alone.
 // Caller holds g_mu.
-qpm_status get_table(const qpm_problem *p, cudaStream_t stream, const Capture &cap, const float4 **table,
-                     const float2 **konst, const float2 **blk = nullptr) {
-  int dev = 0;
-  QPM_CUDA(cudaGetDevice(&dev));
+qpm_status get_table(int dev, const qpm_problem *p, cudaStream_t stream, const Capture &cap,
+                     const float4 **table, const float2 **konst, const float2 **blk = nullptr) {
   auto key = std::make_tuple(dev, p->N, p->kappa1, p->kappa2);
   auto it = g_tables.find(key);
   TableEntry own;
@@ -366,9 +364,8 @@ qpm_status get_table(const qpm_problem *p, cudaStream_t stream, const Capture &c
   return QPM_OK;
 }
 
-qpm_status get_scratch(cudaStream_t stream, size_t bytes, void **ptr) {
-  int dev = 0;
-  QPM_CUDA(cudaGetDevice(&dev));
+// Scratch of a stream that is not being captured, so that clearing the counters runs here and now.
+qpm_status get_scratch(int dev, cudaStream_t stream, size_t bytes, void **ptr) {
   unsigned long long id = 0;
   if (stream == cudaStreamPerThread) {
     QPM_CUDA(cudaStreamGetId(stream, &id));
@@ -389,6 +386,12 @@ qpm_status get_scratch(cudaStream_t stream, size_t bytes, void **ptr) {
     }
     free_unheld(dev);
     QPM_CUDA(cudaMalloc(&e.ptr, bytes));
+    const cudaError_t ce = cudaMemsetAsync(e.ptr, 0, FUSE_BYTES, stream);
+    if (ce != cudaSuccess) {  // no scratch without its counters
+      cudaFree(e.ptr);
+      e.ptr = nullptr;
+      return cuda_fail(ce, "clearing the scratch counters");
+    }
     e.bytes = bytes;
   }
   *ptr = e.ptr;
@@ -398,9 +401,7 @@ qpm_status get_scratch(cudaStream_t stream, size_t bytes, void **ptr) {
 // Scratch of a captured call: never the stream's own, which later calls use and may replace.  The
 // calls captured on one stream in one capture run one after the other and share a block; other
 // captures get another, new or of graphs that are gone.
-qpm_status graph_scratch(cudaStream_t stream, const Capture &cap, size_t bytes, void **ptr) {
-  int dev = 0;
-  QPM_CUDA(cudaGetDevice(&dev));
+qpm_status graph_scratch(int dev, cudaStream_t stream, const Capture &cap, size_t bytes, void **ptr) {
   DevMem *best = nullptr;
   for (DevMem *m = g_kept; m; m = m->next) {
     if (m->dev != dev || m->bytes < bytes) continue;
@@ -438,7 +439,7 @@ static int row_pieces(const RowPlan &p) {
   return (int)std::min<int64_t>(std::min<int64_t>(p.nunit, p.C), (p.nunit + q - 1) / q + 1);
 }
 
-RowPlan row_plan(int NP, int N, int W, int slots, int gran, int maxsub, int min_units) {
+RowPlan row_plan(int NP, int N, int W, int64_t full, int gran, int maxsub, int min_units) {
   RowPlan p;
   p.NP = NP;
   p.N = N;
@@ -449,7 +450,7 @@ RowPlan row_plan(int NP, int N, int W, int slots, int gran, int maxsub, int min_
   p.nsub = (N + 31) / 32;
   p.gran = gran;
   p.nunit = (p.nsub + gran - 1) / gran;
-  const int64_t tot = (int64_t)p.RB * p.nunit, full = (int64_t)slots * sm_count();
+  const int64_t tot = (int64_t)p.RB * p.nunit;
   // whole rounds of the resident CTAs, as few as keep every run within maxsub
   const int64_t rounds = (tot * gran + full * maxsub - 1) / (full * maxsub);
   int64_t C = std::max<int64_t>(1, rounds) * full;
@@ -472,13 +473,14 @@ static int genes_warps(int K, int NP) {
 RowPlan genes_plan(int K, int NP, int N, bool aligned, bool whole) {
   const int W = genes_warps(K, NP);
   if (!whole) {
-    RowPlan p = row_plan(NP, N, W, rs_ctas(K, W), 1, RS_MAXSUB, 4);
+    const int full = rs_ctas(K, W) * sm_count();
+    RowPlan p = row_plan(NP, N, W, full, 1, RS_MAXSUB, 4);
     // Whole rounds of CTAs, all in step, lose to runs of the full length where a few row blocks of
     // very long aligned rows need three rounds or more (one table): 256 x 1e6 215 us against 194,
     // 512 x 600000 232 / 208, 128 x 2e6 220 / 196, 64 x 3e6 179 / 165, 512 x 1e6 363 / 372.  Not with
     // rows of odd pitch (256 x 1e6 185 / 212), more row blocks (1024 x 250000 168 / 184) or two rounds
     // (1024 x 131072 89 / 110).
-    if (K == 1 && aligned && p.RB <= 4 && p.C > 2 * rs_ctas(K, W) * sm_count()) {
+    if (K == 1 && aligned && p.RB <= 4 && p.C > 2 * full) {
       p.C = p.RB * ((p.nunit + RS_MAXSUB - 1) / RS_MAXSUB);
       p.P = row_pieces(p);
     }
@@ -492,7 +494,7 @@ RowPlan genes_plan(int K, int NP, int N, bool aligned, bool whole) {
   return p;
 }
 static RowPlan packed_plan(int NP, int N, int W) {
-  return row_plan(NP, N, W, ep_ctas(W), 4, 128, 1);
+  return row_plan(NP, N, W, ep_ctas(W) * sm_count(), 4, 128, 1);
 }
 
 qpm_status make_gene_maps(GeneMaps *gm, int *mode, const float *genes, int NP, int N, int64_t ld) {
@@ -512,10 +514,10 @@ qpm_status make_gene_maps(GeneMaps *gm, int *mode, const float *genes, int NP, i
   return QPM_OK;
 }
 
-// what closes a call: the fused combination (no words: the combining kernel), the constants and
+// what closes a call: the counters of the fused combination (NULL: the combining kernel), the constants and
 // the outputs
 struct EvalOut {
-  RowFuse fuse;
+  unsigned *ctr;
   const float2 *konst;
   float2 *deff;
   float *fit;
@@ -530,7 +532,7 @@ static qpm_status launch_genes(const GeneMaps &gm, const float *g, int64_t ld, c
   const qpm_status st = attr.set(fn, rs_smem(1, W));
   if (st != QPM_OK) return st;
   void *args[] = {(void *)&gm, (void *)&g, (void *)&ld, (void *)&pl, (void *)&tabs, (void *)&part,
-                  (void *)&out.fuse, (void *)&out.konst, (void *)&out.deff, (void *)&out.fit};
+                  (void *)&out.ctr, (void *)&out.konst, (void *)&out.deff, (void *)&out.fit};
   return launch_dependent(fn, dim3(pl.C), dim3(W * 32), args, rs_smem(1, W), stream);
 }
 
@@ -564,7 +566,7 @@ static qpm_status launch_eval_rows(bool comp, const float *g, int64_t ld, const 
     else QPM_EG(1, ROWS_TMA4);
   }
 #undef QPM_EG
-  if (st != QPM_OK || out.fuse.words) return st;
+  if (st != QPM_OK || out.ctr) return st;
   return launch_combine(pl, part, out, stream);
 }
 
@@ -580,20 +582,8 @@ static qpm_status launch_packed(bool vecw, bool comp, const uint32_t *src, int64
   return launch_dependent(fn, dim3(pl.C), dim3(W * 32), args, 0, stream);
 }
 
-size_t fuse_bytes(const RowPlan &pl) {
-  return pl.P <= RC_FUSE ? sizeof(unsigned long long) * (size_t)RF_STRIDE * (size_t)pl.RB : 0;
-}
-
-RowFuse row_fuse(const RowPlan &pl, void *words, const TableLease &lease) {
-  // tags count up from a start that no memory holds by chance (the clock, spread over 64 bits)
-  static std::atomic<unsigned long long> tag{
-      ((unsigned long long)std::chrono::steady_clock::now().time_since_epoch().count() | 1ull) *
-      0x9E3779B97F4A7C15ull};
-  RowFuse f;
-  if (pl.P > RC_FUSE || lease.captured()) return f;
-  f.words = (unsigned long long *)words;
-  f.tag = tag.fetch_add(1, std::memory_order_relaxed) & (~0ull >> RF_BITS);
-  return f;
+bool row_fuse(const RowPlan &pl, const TableLease &lease) {
+  return pl.P <= RC_FUSE && pl.RB <= FUSE_BLOCKS && !lease.captured();
 }
 
 static qpm_status eval_common(const qpm_problem *prob, const void *src, int64_t ld, int32_t NP,
@@ -613,11 +603,10 @@ static qpm_status eval_common(const qpm_problem *prob, const void *src, int64_t 
   const RowPlan pl = kind == 2 ? packed_plan(NP, prob->N, W)
                                : genes_plan(1, NP, prob->N, rows_aligned((const float *)src, NP, ld));
   void *scratch;
-  const size_t partials = plan_bytes(pl, 1);
-  st = lease.scratch(partials + (kind == 2 ? 0 : fuse_bytes(pl)), &scratch);
+  st = lease.scratch(FUSE_BYTES + plan_bytes(pl, 1), &scratch);
   if (st != QPM_OK) return st;
-  float2 *part = (float2 *)scratch;
-  EvalOut out{RowFuse{}, konst, (float2 *)d_eff, fit};
+  float2 *part = (float2 *)((char *)scratch + FUSE_BYTES);
+  EvalOut out{nullptr, konst, (float2 *)d_eff, fit};
   if (kind == 2) {
     const bool vecw = (ld % 4 == 0) && (((uintptr_t)src & 15) == 0);
     const RowTables<1> tabs{{blk}};
@@ -625,7 +614,7 @@ static qpm_status eval_common(const qpm_problem *prob, const void *src, int64_t 
                 : launch_packed<2>(vecw, comp != 0, (const uint32_t *)src, ld, pl, tabs, part, stream);
     return st != QPM_OK ? st : launch_combine(pl, part, out, stream);
   }
-  out.fuse = row_fuse(pl, (char *)scratch + partials, lease);
+  if (row_fuse(pl, lease)) out.ctr = (unsigned *)scratch;
   return launch_eval_rows(comp != 0, (const float *)src, ld, pl, blk, part, out, stream);
 }
 
@@ -721,17 +710,17 @@ extern "C" qpm_status qpm_eval_noalloc(const qpm_problem *prob, const float *gen
   if (st != QPM_OK) return st;
   // always the combining kernel: the call may be captured and replayed
   return launch_eval_rows(compensated != 0, genes, ld, pl, blk, part,
-                          EvalOut{RowFuse{}, konst, (float2 *)d_eff, fit}, s);
+                          EvalOut{nullptr, konst, (float2 *)d_eff, fit}, s);
 }
 
 qpm::TableLease::TableLease(const qpm_problem *problems, int count, cudaStream_t stream) : stream_(stream) {
   g_mu.lock();
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
+  cudaError_t e = cudaGetDevice(&dev_);
   if (e != cudaSuccess) {
     st_ = cuda_fail(e, "cudaGetDevice");
     return;
   }
+  const int dev = dev_;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   // The query also makes the device's context current in a thread that has made no CUDA call yet:
   // a call that finds its tables and scratch makes no other before it encodes tensor maps, which
@@ -762,18 +751,19 @@ qpm::TableLease::~TableLease() { g_mu.unlock(); }
 
 qpm_status qpm::TableLease::table(const qpm_problem *p, const float4 **table, const float2 **konst) {
   if (st_ != QPM_OK) return st_;
-  return get_table(p, stream_, cap_, table, konst);
+  return get_table(dev_, p, stream_, cap_, table, konst);
 }
 
 qpm_status qpm::TableLease::block_table(const qpm_problem *p, const float2 **blk, const float2 **konst) {
   if (st_ != QPM_OK) return st_;
   const float4 *table;
-  return get_table(p, stream_, cap_, &table, konst, blk);
+  return get_table(dev_, p, stream_, cap_, &table, konst, blk);
 }
 
 qpm_status qpm::TableLease::scratch(size_t bytes, void **ptr) {
   if (st_ != QPM_OK) return st_;
-  return cap_.graph ? graph_scratch(stream_, cap_, bytes, ptr) : get_scratch(stream_, bytes, ptr);
+  return cap_.graph ? graph_scratch(dev_, stream_, cap_, bytes, ptr)
+                    : get_scratch(dev_, stream_, bytes, ptr);
 }
 
 extern "C" qpm_status qpm_eval(const qpm_problem *prob, const float *genes, int64_t ld,

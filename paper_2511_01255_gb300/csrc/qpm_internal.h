@@ -77,10 +77,12 @@ class TableLease {
   qpm_status table(const qpm_problem *p, const float4 **table, const float2 **konst);
   // the same entry's sign-block table (built the first time) and constants
   qpm_status block_table(const qpm_problem *p, const float2 **blk, const float2 **konst);
-  // scratch for one call's launches: the stream's, or the captured graph's own
+  // scratch for one call's launches: the stream's, which starts with FUSE_BLOCKS counters that are 0
+  // between calls, or the captured graph's own
   qpm_status scratch(size_t bytes, void **ptr);
 
  private:
+  int dev_ = 0;
   cudaStream_t stream_;
   Capture cap_;
   qpm_status st_ = QPM_OK;
@@ -98,9 +100,9 @@ struct RowPlan {
   int C;      // CTAs
   int P;      // pieces of a row at most
 };
-// slots: resident CTAs per SM; gran: sub-steps per unit; maxsub: longest run; min_units: no run
+// full: resident CTAs of the GPU; gran: sub-steps per unit; maxsub: longest run; min_units: no run
 // shorter than this while CTAs are left idle
-RowPlan row_plan(int NP, int N, int W, int slots, int gran, int maxsub, int min_units);
+RowPlan row_plan(int NP, int N, int W, int64_t full, int gran, int maxsub, int min_units);
 // the plan of the float-gene sweep with K sign-block tables; aligned: see rows_aligned; whole: no
 // row is split unless it is longer than a run may be (fewest pieces)
 RowPlan genes_plan(int K, int NP, int N, bool aligned, bool whole = false);
@@ -108,17 +110,11 @@ RowPlan genes_plan(int K, int NP, int N, bool aligned, bool whole = false);
 inline bool rows_aligned(const float *genes, int NP, int64_t ld) {
   return ((uintptr_t)genes & 15) == 0 && (NP == 1 || ld % 4 == 0);
 }
-// What a sweep that combines its rows itself counts arrivals with (rows_last): a word per row block
-// behind the call's partials, whatever it holds before the call, and the call's own tag, which
-// no other call of the process has
-struct RowFuse {
-  unsigned long long *words = nullptr;  // NULL: the combining kernel
-  unsigned long long tag = 0;
-};
-// the plan's fused combination with the words at `words` (fuse_bytes): none where a row has many
-// pieces or the call is captured (a replay would find its own tag)
-RowFuse row_fuse(const RowPlan &pl, void *words, const TableLease &lease);
-size_t fuse_bytes(const RowPlan &pl);
+// whether the sweep combines the rows itself, with the counters of the stream's scratch: where a row
+// has few pieces and the call is not captured, whose replays may run beside the stream's calls
+constexpr int FUSE_BLOCKS = 4096;  // row blocks of such a plan at most
+constexpr size_t FUSE_BYTES = sizeof(unsigned) * FUSE_BLOCKS;
+bool row_fuse(const RowPlan &pl, const TableLease &lease);
 constexpr int EVAL_MAX_ROWS = 128 * 65535;  // rows a call of the row sweeps takes
 // bytes of the plan's partial monoids for K problems
 inline size_t plan_bytes(const RowPlan &p, int K) {

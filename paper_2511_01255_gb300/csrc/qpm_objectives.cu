@@ -231,8 +231,8 @@ __device__ __forceinline__ void multi_close(const MultiOut<K> &o, int row, const
 template <int K, int W, int MODE>
 static __global__ void __launch_bounds__(W * 32, rs_ctas(K, W))
     k_multi_genes(const __grid_constant__ GeneMaps maps, const float *__restrict__ src, int64_t ld,
-                  RowPlan pl, RowTables<K> tabs, float2 *part, RowFuse fuse, MultiOut<K> out) {
-  rows_sweep<K, W, MODE, false>(maps, src, ld, pl, tabs, part, fuse,
+                  RowPlan pl, RowTables<K> tabs, float2 *part, unsigned *ctr, MultiOut<K> out) {
+  rows_sweep<K, W, MODE, false>(maps, src, ld, pl, tabs, part, ctr,
                                 [&](int row, const Mono *m) { multi_close<K>(out, row, m); });
 }
 
@@ -251,36 +251,40 @@ static __global__ void __launch_bounds__(RC_THREADS)
 
 template <int K, int W, int MODE>
 static qpm_status launch_multi_genes(const GeneMaps &gm, const float *g, int64_t ld, const RowPlan &pl,
-                                     const RowTables<K> &tabs, float2 *part, const RowFuse &fuse,
+                                     const RowTables<K> &tabs, float2 *part, unsigned *ctr,
                                      const MultiOut<K> &out, cudaStream_t s) {
   static SmemAttr attr;
   const void *fn = (const void *)k_multi_genes<K, W, MODE>;
   const qpm_status st = attr.set(fn, rs_smem(K, W));
   if (st != QPM_OK) return st;
   void *args[] = {(void *)&gm, (void *)&g, (void *)&ld, (void *)&pl, (void *)&tabs, (void *)&part,
-                  (void *)&fuse, (void *)&out};
+                  (void *)&ctr, (void *)&out};
   return launch_dependent(fn, dim3(pl.C), dim3(W * 32), args, rs_smem(K, W), s);
 }
 
 template <int K>
 static qpm_status launch_multi(const float2 *const *blk, const float2 *const *konst, const float *g,
                                int64_t ld, const RowPlan &pl, float G0, float beta, void *scratch,
-                               float2 *deff, float *obj, const TableLease &lease, cudaStream_t s) {
+                               float2 *deff, float *obj, TableLease &lease, cudaStream_t s) {
   constexpr int MANY = K == 1 ? 4 : 8, FEW = K == 1 ? 1 : 2;  // genes_plan's warps per CTA
   GeneMaps gm;
   int mode;
   qpm_status st = make_gene_maps(&gm, &mode, g, pl.NP, pl.N, ld);
   if (st != QPM_OK) return st;
   float2 *part = (float2 *)scratch;
-  // partials and words are the caller's: calls with scratch of their own stay independent
-  const RowFuse fuse = row_fuse(pl, (char *)scratch + plan_bytes(pl, K), lease);
+  unsigned *ctr = nullptr;
+  if (row_fuse(pl, lease)) {
+    void *counters = nullptr;
+    if ((st = lease.scratch(FUSE_BYTES, &counters)) != QPM_OK) return st;
+    ctr = (unsigned *)counters;
+  }
   RowTables<K> tabs;
   MultiOut<K> out{{}, G0, beta, deff, obj};
   for (int k = 0; k < K; ++k) {
     tabs.blk[k] = blk[k];
     out.konst[k] = konst[k];
   }
-#define QPM_MG(W, M) st = launch_multi_genes<K, W, M>(gm, g, ld, pl, tabs, part, fuse, out, s)
+#define QPM_MG(W, M) st = launch_multi_genes<K, W, M>(gm, g, ld, pl, tabs, part, ctr, out, s)
   if (pl.W == MANY) {
     if (mode == ROWS_TMA) QPM_MG(MANY, ROWS_TMA);
     else QPM_MG(MANY, ROWS_TMA4);
@@ -289,7 +293,7 @@ static qpm_status launch_multi(const float2 *const *blk, const float2 *const *ko
     else QPM_MG(FEW, ROWS_TMA4);
   }
 #undef QPM_MG
-  if (st != QPM_OK || fuse.words) return st;
+  if (st != QPM_OK || ctr) return st;
   int runs = rc_runs(pl);
   const int rows = RC_THREADS / runs;
   void *args[] = {(void *)&pl, &runs, &part, &out};
@@ -313,7 +317,7 @@ extern "C" qpm_status qpm_eval_shg(const qpm_problem *prob, const float *genes, 
   qpm_status st = lease.table(prob, &table, &konst);
   if (st != QPM_OK) return st;
   const bool vec = (ld % 4 == 0) && (((uintptr_t)genes & 15) == 0) && prob->N >= 4;
-  const int rpc = (NP + sm_count() - 1) / sm_count(), grid = (NP + rpc - 1) / rpc;
+  const int sms = sm_count(), rpc = (NP + sms - 1) / sms, grid = (NP + rpc - 1) / rpc;
   float2 *e = (float2 *)e_shg;
   void *args[] = {(void *)&genes, &ld, &NP, (void *)&prob->N, (void *)&rpc, (void *)&table, (void *)&konst, &e, &fit};
   const void *fn = rpc == 1 ? (vec ? (const void *)k_shg<true, 1> : (const void *)k_shg<false, 1>)
@@ -343,7 +347,7 @@ extern "C" qpm_status qpm_eval_multi(const qpm_problem *probs, int32_t K, const 
     if (st != QPM_OK) return st;
   }
   const RowPlan pl = genes_plan(K, NP, N, rows_aligned(genes, NP, ld));
-  if (!scratch || scratch_bytes < plan_bytes(pl, K) + fuse_bytes(pl))
+  if (!scratch || scratch_bytes < plan_bytes(pl, K))
     return fail(QPM_ERR_ARG, "qpm_eval_multi: scratch smaller than qpm_eval_multi_scratch_bytes()");
 #define QPM_MW(KK) \
   launch_multi<KK>(blk, konst, genes, ld, pl, G0, beta, scratch, (float2 *)d_eff, objective, lease, s)
@@ -353,10 +357,6 @@ extern "C" qpm_status qpm_eval_multi(const qpm_problem *probs, int32_t K, const 
 
 extern "C" size_t qpm_eval_multi_scratch_bytes(int32_t K, int32_t N, int32_t NP) {
   if (K < 1 || N < 1 || NP < 1) return 0;
-  size_t bytes = 0;
-  for (const bool aligned : {false, true}) {
-    const RowPlan pl = genes_plan(std::min(K, (int32_t)MW_KMAX), NP, N, aligned);
-    bytes = std::max(bytes, plan_bytes(pl, K) + fuse_bytes(pl));
-  }
-  return bytes;
+  const size_t bytes = plan_bytes(genes_plan(std::min(K, (int32_t)MW_KMAX), NP, N, false), K);
+  return K > 1 ? bytes : std::max(bytes, plan_bytes(genes_plan(1, NP, N, true), 1));  // only K = 1 looks at it
 }

@@ -213,34 +213,19 @@ __host__ __device__ constexpr int rs_ctas(int K, int W) {
 // path), but one CTA's threads have the loads of about 16 pieces (6 registers each) in flight at a
 // time, and rows cut finer than that are few and long, where the kernel spreads them over the GPU.
 constexpr int RC_FUSE = 16;
-constexpr int RF_STRIDE = 16;  // words from one row block's to the next's: a 128-byte line each
-constexpr int RF_BITS = 5;  // of a row block's word for the CTAs arrived, 0 .. RC_FUSE; the tag has the others
-static_assert(RC_FUSE < (1 << RF_BITS), "the count must not run into the tag");
-// A row block's word is (the call's tag, the CTAs arrived) and needs no state from before the call:
-// every CTA, before its piece, sets a word without the tag to (tag, 0), once for all of them
-// whoever comes first, and after it adds 1.  So a call on another stream, one that was captured and
-// never replayed, or memory never written cannot disturb the count, as they would one that has to
-// start at 0.  The look costs nothing (it waits together with the piece's table entries) and the
-// arrival is one round trip to L2.  (The whole of it after the piece, by compare-and-swap or by a
-// flag per piece and a look at all of them: 10.8 and 8.1 us for a call of 5000 x 1000, 7.2 so.)
-__device__ __forceinline__ unsigned long long rows_look(const unsigned long long *word) {
-  unsigned long long w;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(word) : "memory");
-  return w;
-}
-__device__ __forceinline__ void rows_open(unsigned long long *word, unsigned long long tag,
-                                          unsigned long long w) {
-  if ((w >> RF_BITS) != tag) atomicCAS(word, w, tag << RF_BITS);  // fails where another CTA has done it
-}
-// true in every thread of the CTA that is the last of the n to arrive, and then the others' partials
-// are visible to it
-__device__ __forceinline__ bool rows_last(unsigned long long *word, int n) {
+// True in every thread of the CTA that is the last of the n to arrive at *ctr, which it leaves at 0 (the
+// counter wraps), and then the others' partials are visible to it.  The counters are 0 between calls:
+// they belong to one stream, whose calls follow one another, and captured calls use none.  (Words
+// that need no state, tagged by each call, cost a call the look at them or the tag's write before
+// the piece: 946 x 1106 11.1 us instead of 10.5, compensated 5000 x 1000 8.0 instead of 7.7; a flag
+// per piece and a look at all of them 8.4; the arrival by compare-and-swap 11.1.)
+__device__ __forceinline__ bool rows_last(unsigned *ctr, int n) {
   __shared__ unsigned last_sh;
   __syncthreads();
   if (n == 1) return true;
   if (threadIdx.x == 0) {
     __threadfence();
-    last_sh = (atomicAdd(word, 1ull) & ((1u << RF_BITS) - 1u)) == (unsigned)n - 1u;
+    last_sh = atomicInc(ctr, (unsigned)n - 1u) == (unsigned)n - 1u;
     __threadfence();
   }
   __syncthreads();
@@ -282,12 +267,14 @@ __device__ __forceinline__ void fused_combine(const RowPlan &pl, const float2 *p
 // registers behind one CTA barrier per step.  A wait on an mbarrier is bounded (%globaltimer);
 // one that runs out makes the rows' results NaN and stops the warp's copies.
 // Partials: part[((piece K + k) 3 + {A, B, C}) NPpad + row].
-// fuse (with a plan of at most RC_FUSE pieces a row): the CTA that completes a row block, found by
-// the block's word (rows_last), combines it and calls close(row, the K monoids).
+// ctr (with a plan of at most RC_FUSE pieces a row): the CTA that completes a row block, found by
+// the block's counter (rows_last), combines it and calls close(row, the K monoids).  (As a form of
+// its own the sweep without it has 126 registers instead of 156 with one table, which gave 1024 x 1e5
+// 0.3 us of 67.9 and cost 64 x 1e5 1.1 us of 10.8.)
 template <int K, int W, int MODE, bool COMP, class Close>
 __device__ __forceinline__ void rows_sweep(const GeneMaps &maps, const float *__restrict__ src,
                                            int64_t ld, const RowPlan &pl, const RowTables<K> &tabs,
-                                           float2 *part, const RowFuse &fuse, Close &&close) {
+                                           float2 *part, unsigned *ctr, Close &&close) {
   extern __shared__ unsigned char rs_raw[];
   unsigned char *base = rs_raw + ((1024 - (smem_u32(rs_raw) & 1023)) & 1023);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -358,15 +345,12 @@ __device__ __forceinline__ void rows_sweep(const GeneMaps &maps, const float *__
             tail |= 1u << q;
       }
     }
-    unsigned long long word = 0;
-    if (fuse.words && threadIdx.x == 0) word = rows_look(fuse.words + (size_t)b * RF_STRIDE);
     __syncthreads();  // the table buffers of the piece before are free
 #pragma unroll
     for (int p = 0; p < K; ++p) {
       R[p].store(tab + p * RS_TAB);
       if (nsteps > 1) R[p].load(tabs.blk[p], (m0 >> 2) + 32, nb);
     }
-    if (fuse.words && threadIdx.x == 0) rows_open(fuse.words + (size_t)b * RF_STRIDE, fuse.tag, word);
     RowAcc<COMP> acc[K];
 #pragma unroll
     for (int p = 0; p < K; ++p) acc[p].zero();
@@ -440,9 +424,9 @@ __device__ __forceinline__ void rows_sweep(const GeneMaps &maps, const float *__
         o[2 * (size_t)pl.NPpad] = m.C;
       }
     }
-    if (fuse.words) {
+    if (ctr) {
       const int P = rp_pieces(pl, b);
-      if (rows_last(fuse.words + (size_t)b * RF_STRIDE, P)) fused_combine<K>(pl, part, P, b * W * 32 + (int)threadIdx.x, close);
+      if (rows_last(ctr + b, P)) fused_combine<K>(pl, part, P, b * W * 32 + (int)threadIdx.x, close);
     }
   }
   if (!ok && lane == 0) {  // copies of a failed warp may still be in flight

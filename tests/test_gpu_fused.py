@@ -1,9 +1,8 @@
 """GPU parity of the rows that a sweep combines itself (few pieces a row).
 
-The CTAs of a row block find out which of them is last by a word behind the partial sums.  The
-words need no state from before the call: neither in a caller's scratch nor in the library's own,
-whatever ran (or was only captured) on that stream before, and calls with scratch of their own do
-not disturb each other.  The reference is the combining kernel, which a captured call takes and
+The CTAs of a row block find out which of them is last by counters that belong to the stream and are
+0 between calls, whatever ran (or was only captured) on it before: calls of different streams do not
+disturb each other, also where one handle names several, and a caller's scratch may hold anything.  The reference is the combining kernel, which a captured call takes and
 which has the same bits, or the FP64 oracle.
 """
 import math
@@ -108,7 +107,7 @@ def test_multi_scratch_holds_anything(q, orc, fill):
     K, shapes = 3, [(1000, 300), (129, 129), (640, 900)]
     need = max(q.lib().qpm_eval_multi_scratch_bytes(K, N, NP) for N, NP in shapes)
     scratch = torch.full((need,), fill, dtype=torch.uint8, device="cuda")
-    for r in range(2):  # the second round finds the other shapes' words and sums
+    for r in range(2):  # the second round finds the other shapes' sums
         for N, NP in shapes:
             X, Xn = genes(NP, N, N + r)
             D, f = torch.full((NP, K, 2), float("nan"), device="cuda"), torch.empty(NP, device="cuda")

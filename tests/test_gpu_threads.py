@@ -138,3 +138,33 @@ def test_multi_scratch_lives_until_its_stream_is_done(q, plain):
             torch.empty(need, dtype=torch.uint8, device="cuda").fill_(255)
         torch.cuda.synchronize()
         assert torch.equal(D, ref)
+
+
+@pytest.mark.parametrize("N,NP", [(30000, 300), (2000, 300)])
+def test_destroyed_streams_whose_handle_comes_back(q, N, NP):
+    """A stream is destroyed with its calls still pending; the next stream often has its handle."""
+    import ctypes
+    import torch
+    rt = torch.cuda.cudart()
+    rng = np.random.default_rng(N)
+    X = [torch.from_numpy(rng.uniform(-1, 1, (NP, N)).astype(np.float32)).cuda() for _ in range(2)]
+    ref = [torch.empty((NP, 2), device="cuda") for _ in range(2)]
+    for x, r in zip(X, ref):
+        q.qpm_eval(N, K1, K2, x, r)
+    D = [torch.empty((NP, 2), device="cuda") for _ in range(2)]
+    handles = set()
+    for _ in range(100):  # more streams than scratch buffers of ended ones are kept
+        for d in D:
+            d.fill_(float("nan"))
+        torch.cuda.synchronize()
+        for x, d in zip(X, D):
+            h = ctypes.c_void_p()
+            assert int(rt.cudaStreamCreate(ctypes.addressof(h))) == 0
+            handles.add(h.value)
+            for _ in range(5):
+                q.qpm_eval(N, K1, K2, x, d, stream=SimpleNamespace(cuda_stream=h.value))
+            assert int(rt.cudaStreamDestroy(h.value)) == 0
+        torch.cuda.synchronize()
+        for d, r in zip(D, ref):
+            assert torch.equal(d, r)
+    assert len(handles) < 200  # some came back
