@@ -1403,11 +1403,40 @@ static __global__ void __maxnreg__(WIDE ? 112 : 80) k_gwo_disc(InstDev I) {
 // share of the keys, every warp takes its top three with redux.sync and warp 0 those of the warps.
 // (Warp 0 reading all keys and merging lane triples by shuffles: 7.89 against 7.31 us per
 // generation at N = 1000, NP = 256; at N = 2500 9.8 / 9.1 with 152 individuals, 26.3 / 25.1 with 900, 126
-// / 122 with 5000; at N = 1e5 and 1024 individuals 677 / 675.)  The keys are written in
-// the DE phase only, so a CTA that is still choosing leaders never sees a fitness
+// / 122 with 5000; at N = 1e5 and 1024 individuals 677 / 675.)  Teams of one or two warps on long rows
+// (NARROW) take that form: many of them search at once on an SM, and it has fewer instructions (N =
+// 3300, NP = 1000 58.8 / 64.4 in teams of 32, 43.8 / 45.9 of 64, 38.0 / 37.4 of 128; NP = 5000 249 / 286 in
+// teams of 32, 172 / 186 of 64).  The keys are
+// written in the DE phase only, so a CTA that is still choosing leaders never sees a fitness
 // already changed by another CTA's GWO selection.
+template <bool NARROW>
 __device__ void leaders_from_keys(const unsigned long long *keys, int NP, int32_t *lead,
                                   int32_t *lead_sh, int32_t *slot_sh) {
+  if (NARROW && blockDim.x <= 64) {
+    if (threadIdx.x < 32) {
+      unsigned long long k0 = 0, k1 = 0, k2 = 0;
+      for (int i = threadIdx.x; i < NP; i += 32) top3_insert(k0, k1, k2, keys[i]);
+      for (int s = 16; s > 0; s >>= 1) {
+        const unsigned long long p0 = __shfl_xor_sync(0xffffffffu, k0, s);
+        const unsigned long long p1 = __shfl_xor_sync(0xffffffffu, k1, s);
+        const unsigned long long p2 = __shfl_xor_sync(0xffffffffu, k2, s);
+        top3_insert(k0, k1, k2, p0);
+        top3_insert(k0, k1, k2, p1);
+        top3_insert(k0, k1, k2, p2);
+      }
+      if (threadIdx.x == 0) {
+        lead_sh[0] = slot_key_index(k0);
+        lead_sh[1] = slot_key_index(k1);
+        lead_sh[2] = slot_key_index(k2);
+        slot_sh[0] = (int32_t)(k0 & 1u);
+        slot_sh[1] = (int32_t)(k1 & 1u);
+        slot_sh[2] = (int32_t)(k2 & 1u);
+        if (lead) { lead[0] = lead_sh[0]; lead[1] = lead_sh[1]; lead[2] = lead_sh[2]; }
+      }
+    }
+    __syncthreads();
+    return;
+  }
   __shared__ unsigned long long wtop[3 * 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   unsigned long long k0 = 0, k1 = 0, k2 = 0;
@@ -1520,7 +1549,7 @@ static __global__ void __launch_bounds__(MAXT, MAXT > 256 ? 1 : 2)
       own1 = own0;
     }
     // every CTA finds the leaders itself (Sec. 3.2 Step 3) from the DE keys
-    leaders_from_keys(I.dekey, I.NP, blockIdx.x == 0 ? I.lead : nullptr, lead_sh, lslot_sh);
+    leaders_from_keys<!DUAL>(I.dekey, I.NP, blockIdx.x == 0 ? I.lead : nullptr, lead_sh, lslot_sh);
     const int la = lead_sh[0], lb = lead_sh[1], ld = lead_sh[2];
     // Step 6, the adaptive F of the next generation: by the CTA of the alpha leader (which
     // moves no wolf) when every CTA holds one individual, else by the last CTA, before its
