@@ -889,7 +889,6 @@ __device__ void adaptive_F_block(const InstDev &I, const unsigned long long *key
   __shared__ unsigned long long red_s[2][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   uint32_t mx = 0u, mn = 0xFFFFFFFFu, cnt = 0u;
-#pragma unroll 8
   for (int i = threadIdx.x; i < I.NP; i += blockDim.x) {
     const unsigned long long k = keys[i];
     const uint32_t fb = I.minimize ? ~(uint32_t)(k >> 32) : (uint32_t)(k >> 32);  // f's bits
@@ -917,7 +916,6 @@ __device__ void adaptive_F_block(const InstDev &I, const unsigned long long *key
   uint32_t emax = (mx >> 23) & 0xFFu;
   if (emax == 0) emax = 1;
   unsigned long long s1 = 0ull, s2 = 0ull;
-#pragma unroll 8
   for (int i = threadIdx.x; i < I.NP; i += blockDim.x) {
     const uint32_t hi = (uint32_t)(keys[i] >> 32);
     const uint32_t n = af_quantise(I.minimize ? ~hi : hi, emax);
