@@ -2108,6 +2108,7 @@ struct qpm_state {
   std::vector<qpm_problem> probs;
   std::vector<qpm_params> params;
   std::vector<int> grid_plain, grid_persist;
+  std::vector<int> grid_init, grid_load;  // k_init and k_load_population of the single kinds
   std::vector<int> grid_mt;  // CTAs of the multi-team kernels of the multi-wavelength kinds
   void *arena = nullptr;
   int g = 0;
@@ -2424,6 +2425,8 @@ extern "C" qpm_status qpm_create(const qpm_problem *probs, const qpm_params *par
   st->params.assign(params, params + n_inst);
   st->h.resize(n_inst);
   st->grid_plain.resize(n_inst);
+  st->grid_init.resize(n_inst);
+  st->grid_load.resize(n_inst);
   st->grid_mt.assign(n_inst, 0);
   st->grid_persist.resize(n_inst);
   st->objs.assign(n_inst, qpm_objective{});
@@ -2480,6 +2483,14 @@ extern "C" qpm_status qpm_create(const qpm_problem *probs, const qpm_params *par
       }
     }
     st->grid_plain[k] = std::min(I.NP, occ_plain * nsm);
+    int occ_init = 1;  // of its own: it needs fewer registers than the phases
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+        &occ_init, I.compensated ? (const void *)k_init<true> : (const void *)k_init<false>, I.T, smem_bytes(I.T));
+    if (e != cudaSuccess) { delete st; return cuda_fail(e, "occupancy of k_init"); }
+    st->grid_init[k] = std::min(I.NP, std::max(1, occ_init) * nsm);
+    // 768 threads an SM: more of them read the caller's rows more slowly (5000 x 13200 191 us for 170, 5000 x
+    // 1320 29 for 25)
+    st->grid_load[k] = std::min(I.NP, std::max(1, std::min(occ_init, 768 / I.T)) * nsm);
     st->grid_persist[k] = std::min(I.NP, occ_persist * nsm);
     base[k] = total;
     const size_t NP = (size_t)I.NP, Np = (size_t)I.Npad;
@@ -2668,8 +2679,8 @@ extern "C" qpm_status qpm_init(qpm_state *st, qpm_stream_t stream) {
     const size_t sm = smem_bytes(I.T), smm = smem_bytes_multi(I.T);
     if (I.obj == OBJ_MULTI_THG) k_init<false, OBJ_MULTI_THG><<<st->grid_plain[k], I.T, smm, s>>>(I);
     else if (I.obj == OBJ_MULTI_SHG) k_init<false, OBJ_MULTI_SHG><<<st->grid_plain[k], I.T, smm, s>>>(I);
-    else if (I.compensated) k_init<true><<<st->grid_plain[k], I.T, sm, s>>>(I);
-    else k_init<false><<<st->grid_plain[k], I.T, sm, s>>>(I);
+    else if (I.compensated) k_init<true><<<st->grid_init[k], I.T, sm, s>>>(I);
+    else k_init<false><<<st->grid_init[k], I.T, sm, s>>>(I);
     QPM_CUDA(cudaGetLastError());
   }
   st->g = 0;
@@ -3008,9 +3019,9 @@ extern "C" qpm_status qpm_set_population(qpm_state *st, int32_t inst, const floa
   else if (I.obj == OBJ_MULTI_SHG)
     k_load_population<false, OBJ_MULTI_SHG><<<st->grid_plain[inst], I.T, smm, s>>>(I, genes, ld, generation);
   else if (I.compensated)
-    k_load_population<true><<<st->grid_plain[inst], I.T, sm, s>>>(I, genes, ld, generation);
+    k_load_population<true><<<st->grid_load[inst], I.T, sm, s>>>(I, genes, ld, generation);
   else
-    k_load_population<false><<<st->grid_plain[inst], I.T, sm, s>>>(I, genes, ld, generation);
+    k_load_population<false><<<st->grid_load[inst], I.T, sm, s>>>(I, genes, ld, generation);
   QPM_CUDA(cudaGetLastError());
   st->g = generation;
   return QPM_OK;
