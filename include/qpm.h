@@ -156,11 +156,12 @@ int32_t qpm_abi_version(void);
  *
  * Stream capture: these calls, qpm_eval_shg, qpm_eval_multi and the relaxed pair may be
  * made on a stream that is being captured.  Tables that are not there yet are then built
- * outside the capture, before the call returns.  The graph keeps the tables and scratch of
- * its own (one buffer per captured stream) for as long as it or an executable instance of
+ * outside the capture, before the call returns.  The graph keeps the tables, and scratch of
+ * its own (one buffer per captured stream), for as long as it or an executable instance of
  * it exists, past eviction and qpm_release_caches too, so it may be replayed on any stream
- * and beside any other work, but not beside another instance of the same graph.  The
- * caller's buffers, the scratch of qpm_eval_multi among them, are the caller's to keep.
+ * and beside any other work, but not beside another instance of the same graph.  Captured
+ * calls evict nothing and may take the cache to 128 problems.  The caller's buffers, the
+ * scratch of qpm_eval_multi among them, are the caller's to keep.
  * ------------------------------------------------------------------------- */
 qpm_status qpm_eval(const qpm_problem *prob, const float *genes, int64_t ld, int32_t NP,
                     float *d_eff, float *fit, int32_t compensated, qpm_stream_t stream);

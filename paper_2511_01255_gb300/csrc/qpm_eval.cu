@@ -164,7 +164,7 @@ std::map<std::tuple<int, int32_t, double, double>, TableEntry> g_tables;
 std::map<std::tuple<int, cudaStream_t, unsigned long long>, ScratchEntry> g_scratch;
 constexpr size_t MAX_THREADS = 64;  // threads whose scratch is kept per device
 DevMem *g_kept = nullptr;  // captured calls' scratch, and tables no longer cached that graphs held
-constexpr size_t MAX_TABLES = 64;
+constexpr size_t MAX_TABLES = 64;  // captured calls, which evict nothing, may add as many again
 
 // This thread's calls that are not allowed beside a capture in the global or thread-local mode
 // (allocations, event queries; a forbidden one would end that capture) are made in the relaxed one.
@@ -305,7 +305,7 @@ qpm_status get_table(int dev, const qpm_problem *p, cudaStream_t stream, const C
   auto key = std::make_tuple(dev, p->N, p->kappa1, p->kappa2);
   auto it = g_tables.find(key);
   TableEntry own;
-  const bool hit = it != g_tables.end(), cached = hit || !cap.graph || device_table_count(dev) < MAX_TABLES;
+  const bool hit = it != g_tables.end(), cached = hit || !cap.graph || device_table_count(dev) < 2 * MAX_TABLES;
   TableEntry &e = hit ? it->second : own;
   if (!hit) {
     RelaxedMode relaxed;

@@ -152,24 +152,33 @@ def test_two_captured_streams_of_one_graph(q):
             assert torch.equal(o, x)
 
 
-def test_full_cache(q, orc):
-    """A problem that no longer fits the cache, first met in a capture."""
+@pytest.mark.parametrize("n", [1, 70])
+def test_full_cache(q, orc, n):
+    """Problems that no longer fit the cache, first met in a capture: the first 64 of them still go
+    there, the others' tables are the graph's alone.  Each is used twice."""
     import torch
     q.qpm_release_caches()
     X, Xn = genes(40, 300)
-    D = torch.empty((40, 2), device="cuda")
+    D, E = torch.empty((40, 2), device="cuda"), torch.empty((n, 40, 2), device="cuda")
     for k in range(64):
         q.qpm_eval(300, K1 + 0.001 * k, K2, X, D)
     torch.cuda.synchronize()
     s = torch.cuda.Stream()
-    g = capture(lambda: q.qpm_eval(300, K1 / 2, K2, X, D), s)
-    ref = orc.deff_closed_genes(Xn, K1 / 2, K2)
+
+    def call():
+        for k in range(n):
+            q.qpm_eval(300, K1 / 2 + 0.001 * k, K2, X, D)
+            q.qpm_eval(300, K1 / 2 + 0.001 * k, K2, X, E[k])
+
+    g = capture(call, s)
     for _ in range(2):
-        D.fill_(float("nan"))
+        E.fill_(float("nan"))
         g.replay()
         torch.cuda.synchronize()
-        assert deff_err(D.cpu().numpy(), ref, 300).max() < TOL_D
-        q.qpm_eval(300, K1 / 2, K2, X, D)  # evicts the 64
+        for k in (0, n // 2, n - 1):
+            ref = orc.deff_closed_genes(Xn, K1 / 2 + 0.001 * k, K2)
+            assert deff_err(E[k].cpu().numpy(), ref, 300).max() < TOL_D
+        q.qpm_eval(300, K1 / 3, K2, X, D)  # evicts what no graph holds
         q.qpm_release_caches()
 
 
