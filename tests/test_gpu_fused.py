@@ -71,8 +71,10 @@ def captured(call, out):
     return out.clone()
 
 
-# row blocks that begin inside a CTA's run, with one and with three tables
-@pytest.mark.parametrize("N,NP,K", [(777, 700, 1), (1100, 5000, 1), (3000, 5000, 3), (590, 3000, 2)])
+# row blocks that begin inside a CTA's run, with one and with three tables; the last two also have row
+# blocks that lie in one run whole
+@pytest.mark.parametrize("N,NP,K", [(777, 700, 1), (1100, 5000, 1), (3000, 5000, 3), (590, 3000, 2),
+                                    (100, 100000, 1), (90, 70000, 3)])
 def test_runs_across_row_blocks_same_bits(q, N, NP, K):
     import torch
     P, crossing = pieces(K, NP, N)
@@ -184,3 +186,17 @@ def test_first_call_of_a_stream_captured(q, orc):
     g.replay()
     torch.cuda.synchronize()
     assert deff_err(D.cpu().numpy(), ref, N).max() < TOL_D
+
+
+def test_more_row_blocks_than_counters(q, orc):
+    """Above 4096 row blocks (of 128 rows) the combining kernel takes over."""
+    import torch
+    N, NP = 40, 4096 * 128 + 6001
+    X = torch.empty((NP, N), device="cuda").uniform_(-1, 1, generator=torch.Generator("cuda").manual_seed(2))
+    D, f = torch.full((NP, 2), float("nan"), device="cuda"), torch.empty(NP, device="cuda")
+    q.qpm_eval(N, K1, K2, X, D, f)
+    torch.cuda.synchronize()
+    assert not bool(torch.isnan(D).any())
+    rows = list(range(0, NP, 5003)) + [4096 * 128 - 1, 4096 * 128, NP - 1]
+    ref = orc.deff_closed_genes(X[rows].cpu().numpy(), K1, K2)
+    assert deff_err(D[rows].cpu().numpy(), ref, N).max() < TOL_D
